@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "fixed_rows.cuh"
 #include "lp_internal.cuh"
 
 namespace lp {
@@ -136,7 +137,10 @@ struct lp_ctx {
   int32_t* glist = nullptr;   // particles with ghost entries (compact, any order)
   int32_t* olist = nullptr;   // particles with one-sided stencils (compact, any order)
   int* gcount = nullptr;      // the two lists' lengths
-  int32_t* perm = nullptr;    // fit thread -> particle (LP_MIXED_FF)
+  int32_t* perm = nullptr;    // fit thread -> particle (LP_MIXED_FF, LP_FP64)
+  float4* fs = nullptr;       // FP32 copies of the fields (fixed-point rows of LP_FP64)
+  int32_t* slow = nullptr;    // particles left to the plain FP64 rows
+  uint8_t* kx = nullptr;      // 1: offsets outside the fixed-point range
   float *Tg = nullptr, *T2 = nullptr;  // twin sums (allocated on first free-surface step)
   double* Y0[7] = {};                  // Heun: state at the start of the step (on first use)
   double* stage = nullptr;             // lp_step on host arrays: 7 x cap_n (on first use)
@@ -419,6 +423,7 @@ StepArgs step_args(lp_ctx* c, int n, const StepConsts& K) {
   A.grids = c->d_grids;
   A.XU = c->XU; A.Lff = c->Lff; A.P1s = c->P1s; A.R1 = c->R1;
   A.perm = LP_ROW_ORDER ? c->perm : nullptr;
+  A.fs = c->fs; A.slow = c->slow; A.slow_count = c->fb_count + 1; A.kx = c->kx;
   A.Xfix = c->Xfix;
   A.gcnt = c->gcnt;
   A.glist = c->glist; A.gcount = c->gcount;
@@ -494,7 +499,7 @@ void run_step(lp_ctx* c, int n, const StepConsts& K, int prec, bool rebuild, cud
     launch_copy_state(n, c->Y0, c->X[c->cx], st);
     c->launches += 1;
   }
-  cudaMemsetAsync(c->fb_count, 0, sizeof(int32_t), st);
+  cudaMemsetAsync(c->fb_count, 0, 3 * sizeof(int32_t), st);
   StepArgs A = step_args(c, n, K);
   phase_mark(c, LP_PHASE_PASS1, true, st);
   launch_pass1(prec, A, st, c->bs_p1);
@@ -502,7 +507,9 @@ void run_step(lp_ctx* c, int n, const StepConsts& K, int prec, bool rebuild, cud
   phase_mark(c, LP_PHASE_PASS2, true, st);
   launch_pass2(prec, A, st, c->bs_p2);
   phase_mark(c, LP_PHASE_PASS2, false, st);
-  c->launches += prec == LP_MIXED_FF ? (K.free_surface ? 9 : 7) + (A.perm ? 1 : 0) : 4;
+  c->launches += prec == LP_MIXED_FF ? (K.free_surface ? 9 : 7) + (A.perm ? 1 : 0)
+                 : prec == LP_FP64   ? 9 + (A.perm ? 1 : 0)
+                                     : 4;
   c->steps += 1;
   c->cx ^= 1;
 }
@@ -715,7 +722,7 @@ lp_status lp_ctx_create(const lp_ctx_desc* desc, lp_ctx** out) {
   if (s == LP_OK) s = dalloc(c, &c->facf, n * kTri);
   if (s == LP_OK) s = dalloc(c, &c->fbslot, n);
   if (s == LP_OK) s = dalloc(c, &c->fb_list, (size_t)c->fb_cap);
-  if (s == LP_OK) s = dalloc(c, &c->fb_count, 1);
+  if (s == LP_OK) s = dalloc(c, &c->fb_count, 3);  // and the two slow counts
   if (s == LP_OK) s = dalloc(c, &c->fbgrad, (size_t)c->fb_cap * 6);
   if (s == LP_OK) s = dalloc(c, &c->d_grids, (size_t)c->cap_cols);
   if (s == LP_OK) s = dalloc(c, &c->d_mui, (size_t)c->cap_cols);
@@ -735,6 +742,9 @@ lp_status lp_ctx_create(const lp_ctx_desc* desc, lp_ctx** out) {
   if (s == LP_OK) s = dalloc(c, &c->olist, n);
   if (s == LP_OK) s = dalloc(c, &c->gcount, 2);
   if (s == LP_OK) s = dalloc(c, &c->perm, n);
+  if (s == LP_OK) s = dalloc(c, &c->fs, n);
+  if (s == LP_OK) s = dalloc(c, &c->slow, n);
+  if (s == LP_OK) s = dalloc(c, &c->kx, n);
   c->capc = std::min(c->cap + 32, 96);
   if (s == LP_OK) s = dalloc(c, &c->cand, n * c->capc);
   if (s == LP_OK) s = dalloc(c, &c->ccnt, n);
@@ -1024,6 +1034,29 @@ lp_status lp_mui_stress(lp_ctx* c, const lp_mui* mui, const lp_eos* eos, int64_t
 }
 
 namespace {
+// Scales of the fixed-point rows (fixed_rows.cuh) for the stencil radius r:
+// r 2^k = f 2^60 with f in (1/2, 1], so an offset's integer part is at most
+// f 2^28, and products are cut to at most 2^28 as well. fx_lim leaves a tenth
+// of the radius for stencils that are held while the particles move.
+void fixed_consts(StepConsts& K) {
+  int e;
+  const double f = std::frexp(K.radius, &e);  // radius = f 2^e, f in [1/2, 1)
+  K.fx_k = 60 - e;
+  K.fx_sq = f * f <= 0.5 ? 27 : 28;
+  K.fx_qs = (float)std::ldexp(1.0, -K.fx_sq);
+  K.fx_lim = (int)((K.fx_sq == 27 ? 0.777 : 1.1) * 0x1p28);
+  const double unit = std::ldexp(1.0, 32 - K.fx_k);  // of an offset's integer part
+  const double l = unit * K.inv_h;
+  const double q = l * l * std::ldexp(1.0, K.fx_sq);  // of a product as a factor
+  K.fx_g2 = l * l; K.fx_g3 = l * q; K.fx_g4 = q * q;
+  K.fx_lin = l; K.fx_quad = q;
+  K.fx_F2 = fx_of(2.0 * K.floor_z, K.fx_k);
+  K.fx_Lx = fx_of(K.Lx, K.fx_k);
+  K.fx_Ly = fx_of(K.Ly, K.fx_k);
+  K.fx_hLx = K.Lx > 0.0 ? (float)(0.5 * K.Lx) : INFINITY;
+  K.fx_hLy = K.Ly > 0.0 ? (float)(0.5 * K.Ly) : INFINITY;
+}
+
 StepConsts step_consts(const lp_eos* eos, const lp_params* q, double dt, int cap) {
   StepConsts K{};
   K.phi_c = eos->phi_c; K.phi_min = eos->phi_min; K.phi_max = eos->phi_max;
@@ -1044,6 +1077,7 @@ StepConsts step_consts(const lp_eos* eos, const lp_params* q, double dt, int cap
   K.ih2_h = (float)ih2; K.ih2_l = (float)(ih2 - (double)K.ih2_h);
   K.phic_h = (float)K.phi_c; K.phic_l = (float)(K.phi_c - (double)K.phic_h);
   K.rho = (float)(q->radius / q->h * (1.0 + 0x1p-10));
+  fixed_consts(K);
   if (K.free_surface) {
     // ghost particles (Sec. 3.1 items 6 and 9): fixed-point grid K r <= 8192
     double g = 1.0;
@@ -1577,7 +1611,7 @@ lp_status lp_step_adjoint(lp_ctx* c, const lp_particles* initial, const lp_mui* 
     S.x = in[0]; S.y = in[1]; S.z = in[2]; S.u = in[3]; S.v = in[4]; S.w = in[5]; S.V = in[6];
     S.xo = out[0]; S.yo = out[1]; S.zo = out[2]; S.uo = out[3]; S.vo = out[4]; S.wo = out[5];
     S.Vo = out[6];
-    cudaMemsetAsync(c->fb_count, 0, sizeof(int32_t), st);
+    cudaMemsetAsync(c->fb_count, 0, 3 * sizeof(int32_t), st);
     launch_pass1(LP_FP64, S, st);
     launch_pass2(LP_FP64, S, st);
   };

@@ -9,7 +9,9 @@
 // threshold, or fewer than 9 rows) are queued for a separate FP64 pivoted-QR
 // kernel, the same algorithm the paper names (QR least squares).
 //
-// FP64 mode: everything in FP64. MIXED mode: moments, right-hand sides and the
+// FP64 mode: the sums over the rows in 64-bit fixed point (fixed_rows.cuh;
+// plain FP64 rows for the particles that do not fit it, and in
+// lp_fit_derivatives), the factor, the solves and the rest in FP64. MIXED mode: moments, right-hand sides and the
 // Cholesky factor in FP32 on the scaled, centred offsets, followed by one FP64
 // refinement sweep (residual r = b - A c and A^T r in FP64, correction solved
 // with the FP32 factor).
@@ -88,6 +90,54 @@ __global__ void __launch_bounds__(kRowGroup) k_row_order(int n, const int32_t* _
 __device__ __forceinline__ int fit_particle(const StepArgs& A) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   return (A.perm && t < A.n) ? A.perm[t] : t;
+}
+
+// FP64 with fixed-point rows (fixed_rows.cuh). 786,000 particles, per step:
+// moments and factor 0.71 ms, right-hand sides and solves 0.97 ms, pass 2
+// 0.85 ms; with the rows in FP64, on whose pipe they were bound (91 % busy),
+// pass 1 took 5.58 and pass 2 2.66 ms. 3 blocks of 128 threads at 168
+// registers: at 128 registers (4 blocks) the sums spill (the column's four
+// steps 12.1 -> 13.2 ms).
+constexpr int kFxBlock = 128;
+__global__ void k_fx_split(const StepArgs A) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < A.n) fx_split_state_body(A, s);
+}
+__global__ void k_fx_split_p1(const StepArgs A) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < A.n) fx_split_p1_body(A, s);
+}
+template <bool PER, bool GH>
+__global__ void __launch_bounds__(kFxBlock, 3) k_gram_fx(const StepArgs A) {
+  const int s = fit_particle(A);
+  if (s < A.n) gram_fx_body<PER, GH>(A, s);
+}
+template <bool PER>
+__global__ void __launch_bounds__(kFxBlock, 3) k_pass1_fx(const StepArgs A) {
+  const int s = fit_particle(A);
+  if (s < A.n) pass1_fx_body<PER>(A, s);
+}
+template <bool PER, bool GH>
+__global__ void __launch_bounds__(kFxBlock, 3) k_pass2_fx(const StepArgs A) {
+  const int s = fit_particle(A);
+  pass2_body<kFixedRows, PER, GH>(A, s, s < A.n);
+}
+// the particles that the fixed-point rows left to the plain FP64 rows
+template <bool PER>
+__global__ void __launch_bounds__(64) k_pass1_slow(const StepArgs A) {
+  const int cnt = min(A.slow_count[0], A.n);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x)
+    pass1_body<LP_FP64, PER>(A, A.slow[t]);
+}
+template <bool PER>
+__global__ void __launch_bounds__(64) k_pass2_slow(const StepArgs A) {
+  const int cnt = min(A.slow_count[1], A.n);
+  const int lane = threadIdx.x & 31;
+  // a warp at a time, so that every lane calls the body
+  for (int b = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; b < cnt; b += gridDim.x * blockDim.x) {
+    const int t = b + lane;
+    pass2_body<LP_FP64, PER>(A, t < cnt ? A.slow[t] : 0, t < cnt);
+  }
 }
 
 // (PER: periodic axes, offsets take their nearest image)
@@ -502,8 +552,21 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
   const int nb = (A.n + bs - 1) / bs;
   const bool per = A.K.periodic != 0;
   if (prec == LP_FP64) {
-    if (per) k_pass1<LP_FP64, true><<<nb, bs, 0, st>>>(A);
-    else k_pass1<LP_FP64, false><<<nb, bs, 0, st>>>(A);
+    k_fx_split<<<(A.n + 255) / 256, 256, 0, st>>>(A);
+    if (A.perm) k_row_order<<<(A.n + kRowGroup - 1) / kRowGroup, kRowGroup, 0, st>>>(A.n, A.cnt, const_cast<int32_t*>(A.perm));
+    const int b = bs < kFxBlock ? bs : kFxBlock;
+    const int nf = (A.n + b - 1) / b;
+    if (per) {
+      if (A.K.free_surface) k_gram_fx<true, true><<<nf, b, 0, st>>>(A);
+      else k_gram_fx<true, false><<<nf, b, 0, st>>>(A);
+      k_pass1_fx<true><<<nf, b, 0, st>>>(A);
+      k_pass1_slow<true><<<152, 64, 0, st>>>(A);
+    } else {
+      if (A.K.free_surface) k_gram_fx<false, true><<<nf, b, 0, st>>>(A);
+      else k_gram_fx<false, false><<<nf, b, 0, st>>>(A);
+      k_pass1_fx<false><<<nf, b, 0, st>>>(A);
+      k_pass1_slow<false><<<152, 64, 0, st>>>(A);
+    }
   } else if (prec == LP_MIXED) {
     if (per) k_pass1<LP_MIXED, true><<<nb, bs, 0, st>>>(A);
     else k_pass1<LP_MIXED, false><<<nb, bs, 0, st>>>(A);
@@ -533,12 +596,22 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
       else k_pass2_twins<false><<<kTwinBlocks, 128, 0, st>>>(A);
     }
   }
+  if (prec == LP_FP64) k_fx_split_p1<<<(A.n + 255) / 256, 256, 0, st>>>(A);
   k_pass2_fallback<<<152, 64, 0, st>>>(A);
   const int nb = (A.n + bs - 1) / bs;
   const bool per = A.K.periodic != 0;
   if (prec == LP_FP64) {
-    if (per) k_pass2<LP_FP64, true><<<nb, bs, 0, st>>>(A);
-    else k_pass2<LP_FP64, false><<<nb, bs, 0, st>>>(A);
+    const int b = bs < kFxBlock ? bs : kFxBlock;
+    const int nf = (A.n + b - 1) / b;
+    if (per) {
+      if (A.K.free_surface) k_pass2_fx<true, true><<<nf, b, 0, st>>>(A);
+      else k_pass2_fx<true, false><<<nf, b, 0, st>>>(A);
+      k_pass2_slow<true><<<152, 64, 0, st>>>(A);
+    } else {
+      if (A.K.free_surface) k_pass2_fx<false, true><<<nf, b, 0, st>>>(A);
+      else k_pass2_fx<false, false><<<nf, b, 0, st>>>(A);
+      k_pass2_slow<false><<<152, 64, 0, st>>>(A);
+    }
   } else if (prec == LP_MIXED) {
     if (per) k_pass2<LP_MIXED, true><<<nb, bs, 0, st>>>(A);
     else k_pass2<LP_MIXED, false><<<nb, bs, 0, st>>>(A);

@@ -3,9 +3,13 @@
 // fit.cu for the method.
 #pragma once
 
+#include "fixed_rows.cuh"
 #include "lp_internal.cuh"
 
 namespace lp {
+
+// precision of the pass-2 body: LP_FP64 with its rows in fixed point
+constexpr int kFixedRows = 3;
 
 // mirror velocity factor of component a
 __device__ __forceinline__ double usign(int mode, int a) {
@@ -17,34 +21,40 @@ __device__ __forceinline__ double usign(int mode, int a) {
 __device__ __forceinline__ void pass1_finish(const StepArgs& A, int s, const double (*c)[kNB]) {
   const int n = A.n;
   const double ih = A.K.inv_h, ih2 = ih * ih;
+  // Multiply-adds are written out (here and in the acceleration): left to the
+  // compiler, which product of a sum is contracted may differ between kernels
+  // that must agree bit for bit.
   double G[3][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) G[a][b] = c[a][b] * ih;
-  const double div = (G[0][0] + G[1][1]) + G[2][2];
-  const double d3 = div * (1.0 / 3.0);
-  const double gxx = G[0][0] - d3, gyy = G[1][1] - d3, gzz = G[2][2] - d3;
-  const double gxy = 0.5 * (G[0][1] + G[1][0]);
-  const double gxz = 0.5 * (G[0][2] + G[2][0]);
-  const double gyz = 0.5 * (G[1][2] + G[2][1]);
-  const double ss = gxx * gxx + gyy * gyy + gzz * gzz + 2.0 * (gxy * gxy + gxz * gxz + gyz * gyz);
+    for (int b = 0; b < 3; ++b) G[a][b] = __dmul_rn(c[a][b], ih);
+  const double div = __dadd_rn(__dadd_rn(G[0][0], G[1][1]), G[2][2]);
+  const double third = -1.0 / 3.0;
+  const double gxx = __fma_rn(div, third, G[0][0]), gyy = __fma_rn(div, third, G[1][1]);
+  const double gzz = __fma_rn(div, third, G[2][2]);
+  const double gxy = __dmul_rn(0.5, __dadd_rn(G[0][1], G[1][0]));
+  const double gxz = __dmul_rn(0.5, __dadd_rn(G[0][2], G[2][0]));
+  const double gyz = __dmul_rn(0.5, __dadd_rn(G[1][2], G[2][1]));
+  // (1/2) gdot:gdot
+  const double dia = __fma_rn(gzz, gzz, __fma_rn(gyy, gyy, __dmul_rn(gxx, gxx)));
+  const double off = __fma_rn(gyz, gyz, __fma_rn(gxz, gxz, __dmul_rn(gxy, gxy)));
+  const double ss = __fma_rn(0.5, dia, off);
   double* p = A.p1;
   p[(P1_GD + 0) * n + s] = gxx; p[(P1_GD + 1) * n + s] = gyy; p[(P1_GD + 2) * n + s] = gzz;
   p[(P1_GD + 3) * n + s] = gxy; p[(P1_GD + 4) * n + s] = gxz; p[(P1_GD + 5) * n + s] = gyz;
-  p[P1_GN * n + s] = sqrt(0.5 * ss);
+  p[P1_GN * n + s] = sqrt(ss);
   // Hessian columns: 3 xx, 4 yy, 5 zz, 6 xy, 7 xz, 8 yz
-  double lap[3];
+  const double dd[3] = {__dadd_rn(__dadd_rn(c[0][3], c[1][6]), c[2][7]),
+                        __dadd_rn(__dadd_rn(c[0][6], c[1][4]), c[2][8]),
+                        __dadd_rn(__dadd_rn(c[0][7], c[1][8]), c[2][5])};
 #pragma unroll
-  for (int a = 0; a < 3; ++a) lap[a] = (c[a][3] + c[a][4]) + c[a][5];
-  const double ddx = (c[0][3] + c[1][6]) + c[2][7];
-  const double ddy = (c[0][6] + c[1][4]) + c[2][8];
-  const double ddz = (c[0][7] + c[1][8]) + c[2][5];
-  p[(P1_LD + 0) * n + s] = (0.5 * lap[0] + ddx * (1.0 / 6.0)) * ih2;
-  p[(P1_LD + 1) * n + s] = (0.5 * lap[1] + ddy * (1.0 / 6.0)) * ih2;
-  p[(P1_LD + 2) * n + s] = (0.5 * lap[2] + ddz * (1.0 / 6.0)) * ih2;
+  for (int a = 0; a < 3; ++a) {
+    const double lap = __dadd_rn(__dadd_rn(c[a][3], c[a][4]), c[a][5]);
+    p[(P1_LD + a) * n + s] = __dmul_rn(__fma_rn(0.5, lap, __dmul_rn(dd[a], 1.0 / 6.0)), ih2);
+  }
   const double Vi = A.V[s];
-  p[P1_VN * n + s] = Vi + A.K.dt * (Vi * div);
+  p[P1_VN * n + s] = __fma_rn(A.K.dt, __dmul_rn(Vi, div), Vi);
   p[P1_DIV * n + s] = div;
 }
 
@@ -67,8 +77,9 @@ __device__ __forceinline__ void ghost_rhs2(const StepArgs& A, double gni, double
                                            double* bv) {
   const double phi = 1.0 / Vi;
   const bool inertial = phi > A.K.phi_min && phi <= A.K.phi_max;
-  const double gng = inertial ? gni * (A.K.ghost_num / (A.K.phi_c - phi)) : gni;
-  *bg = gng - gni;
+  const double gng =
+      inertial ? __dmul_rn(gni, A.K.ghost_num / __dsub_rn(A.K.phi_c, phi)) : gni;
+  *bg = __dsub_rn(gng, gni);
   *bv = A.K.ghost_V - Vi;
 }
 
@@ -231,6 +242,65 @@ __device__ __forceinline__ void pass1_body(const StepArgs& A, int s) {
     }
     pass1_finish(A, s, c);
   }
+}
+
+// Pass 1 of LP_FP64 with the rows in fixed point (fixed_rows.cuh), in two
+// kernels: the moments and the FP64 factor, then the right-hand sides, solves
+// and derived values. 31 or 27 sums of three registers each are live, so one
+// kernel for both would not fit. A particle whose rows do not fit is queued
+// for pass1_body<LP_FP64>.
+template <bool PER, bool GH>
+__device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
+  const int64_t n = A.n;
+  const int m = min(A.cnt[s], A.cap);
+  double L[kTri];
+  {
+    double mo[31];
+    const bool fits = fx_moments<PER, GH>(A, s, m, mo);
+    A.kx[s] = fits ? 0 : 1;
+    if (!fits) {
+      fx_push(A, s, 0);
+      return;
+    }
+    gram_of_moments(mo, L);
+  }
+  const bool ok = fx_chol9(L, 1e-9) && m >= kNB;
+  if (!ok) {
+    push_fallback(A, s);
+    return;
+  }
+  A.fbslot[s] = -1;
+#pragma unroll
+  for (int k = 0; k < kTri; ++k) A.fac[k * n + s] = L[k];
+}
+template <bool PER>
+__device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
+  if (A.kx[s] || A.fbslot[s] != -1) return;  // queued for the plain rows or the QR fit
+  const int64_t n = A.n;
+  const int m = min(A.cnt[s], A.cap);  // ghost rows carry b = 0: no right-hand side
+  const int mm = A.K.mirror_mode;
+  const int sgn[3] = {mm == LP_MIRROR_NOSLIP ? -1 : 1, mm == LP_MIRROR_NOSLIP ? -1 : 1,
+                      mm != LP_MIRROR_NONE ? -1 : 1};
+  double R[3][kNB];
+  if (!fx_rhs<3, PER, false>(A, s, m, sgn, nullptr, R)) {
+    fx_push(A, s, 0);
+    return;
+  }
+  {
+    double L[kTri];
+#pragma unroll
+    for (int k = 0; k < kTri; ++k) L[k] = A.fac[k * n + s];
+    fx_chol9_solve(L, R[0]);
+    fx_chol9_solve(L, R[1]);
+    fx_chol9_solve(L, R[2]);
+  }
+  if (A.coef1) {
+#pragma unroll
+    for (int f = 0; f < 3; ++f)
+#pragma unroll
+      for (int q = 0; q < kNB; ++q) A.coef1[(int64_t)(f * kNB + q) * n + s] = R[f][q];
+  }
+  pass1_finish(A, s, R);
 }
 
 // pivoted-QR fallback of pass 1 (grid-stride over the queued particles)
@@ -991,12 +1061,17 @@ __device__ __forceinline__ void accel_ff(const StepArgs& A, int s, const ff* gg,
 // ------------------------------------------------------------ pass 2
 
 // every lane of the warp must call it (live or not)
-template <int PREC, bool PER = false>
+// (GH: the stencils may carry ghosts; only the fixed-point rows ask)
+template <int PREC, bool PER = false, bool GH = true>
 __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) {
   int regime = 1;
   bool overc = false, nonfin = false, below = false;
   float disp = 0.f;  // displacement from the search positions (filter skipping)
-  if (live) {
+  if (PREC == kFixedRows && live && A.kx[s]) {  // the offsets do not fit: plain FP64 rows
+    fx_push(A, s, 1);
+    live = false;
+  }
+  if (live) do {
     const int n = A.n;
     const double xi = A.x[s], yi = A.y[s], zi = A.z[s];
     const double ih = A.K.inv_h, f2 = 2.0 * A.K.floor_z;
@@ -1023,6 +1098,34 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
         ffit = true;
 #pragma unroll
         for (int q = 0; q < 3; ++q) gg[q] = gV[q] = 0.0;  // set below where needed
+      } else if (PREC == kFixedRows) {
+        double R[2][kNB], bG[2] = {0.0, 0.0};
+        if (GH && A.K.free_surface) ghost_rhs2(A, gni, Vi, &bG[0], &bG[1]);
+        const int sgn[2] = {0, 1};
+        if (!fx_rhs<2, PER, GH>(A, s, m, sgn, bG, R)) {  // plain FP64 rows
+          fx_push(A, s, 1);
+          live = false;
+          break;
+        }
+        {
+          double L[kTri];
+#pragma unroll
+          for (int k = 0; k < kTri; ++k) L[k] = A.fac[(int64_t)k * n + s];
+          fx_chol9_solve(L, R[0]);
+          fx_chol9_solve(L, R[1]);
+        }
+        if (A.coef2) {
+#pragma unroll
+          for (int q = 0; q < kNB; ++q) {
+            A.coef2[(int64_t)q * n + s] = R[0][q];
+            A.coef2[(int64_t)(kNB + q) * n + s] = R[1][q];
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          gg[q] = __dmul_rn(R[0][q], ih);
+          gV[q] = __dmul_rn(R[1][q], ih);
+        }
       } else if (PREC == LP_FP64) {
         double R[2][kNB];
 #pragma unroll
@@ -1168,18 +1271,22 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
       const double g02 = A.p1[(P1_GD + 4) * n + s], g12 = A.p1[(P1_GD + 5) * n + s];
       const double g3[3][3] = {{g00, g01, g02}, {g01, g11, g12}, {g02, g12, g22}};
       const double G = gni;
-      const double GV2 = G / (Vi * Vi);
+      const double GV2 = G / __dmul_rn(Vi, Vi);
+      const double SG = __dmul_rn(cl.S, G), MG2 = __dmul_rn(__dmul_rn(2.0, cl.M), G);
+      const double NG = __dmul_rn(cl.N, G);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         // V [ -(|g|/V^2)(S|g| V_c + R g_cj V_j) + 2M|g| |g|_c + N g_cj |g|_j
         //     + N|g| ((1/2) Lap u_c + (1/6) d_c div u) ] + g_c
-        const double gjVj = (g3[c][0] * gV[0] + g3[c][1] * gV[1]) + g3[c][2] * gV[2];
-        const double gjGj = (g3[c][0] * gg[0] + g3[c][1] * gg[1]) + g3[c][2] * gg[2];
-        const double t1 = -GV2 * (cl.S * G * gV[c] + cl.R * gjVj);
-        const double t2 = 2.0 * cl.M * G * gg[c];
-        const double t3 = cl.N * gjGj;
-        const double t4 = cl.N * G * A.p1[(P1_LD + c) * n + s];
-        acc[c] = Vi * (((t1 + t2) + t3) + t4) + gvec[c];
+        const double gjVj =
+            __fma_rn(g3[c][2], gV[2], __fma_rn(g3[c][1], gV[1], __dmul_rn(g3[c][0], gV[0])));
+        const double gjGj =
+            __fma_rn(g3[c][2], gg[2], __fma_rn(g3[c][1], gg[1], __dmul_rn(g3[c][0], gg[0])));
+        const double t1 = __fma_rn(SG, gV[c], __dmul_rn(cl.R, gjVj));
+        double t = __fma_rn(MG2, gg[c], -__dmul_rn(GV2, t1));
+        t = __fma_rn(cl.N, gjGj, t);
+        t = __fma_rn(NG, A.p1[(P1_LD + c) * n + s], t);
+        acc[c] = __fma_rn(Vi, t, gvec[c]);
       }
     } else {
       regime = 2;
@@ -1188,22 +1295,24 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
         for (int q = 0; q < 3; ++q) gV[q] = ff_to_double(gVf[q]);
       // sigma = -phi_s (alpha + beta phi) I  =>  a = beta grad V / V + g
 #pragma unroll
-      for (int c = 0; c < 3; ++c) acc[c] = (A.K.beta * gV[c]) / Vi + gvec[c];
+      for (int c = 0; c < 3; ++c)
+        acc[c] = __dadd_rn(__dmul_rn(A.K.beta, gV[c]) / Vi, gvec[c]);
       overc = phi > A.K.phi_c;
     }
     // ---- update (Sec. 3.1 items 8, 10)
     const double dt = A.K.dt;
     const double un = A.u[s], vn = A.v[s], wn = A.w[s];
-    const double u1 = un + dt * acc[0], v1 = vn + dt * acc[1], w1 = wn + dt * acc[2];
+    const double u1 = __fma_rn(dt, acc[0], un), v1 = __fma_rn(dt, acc[1], vn);
+    const double w1 = __fma_rn(dt, acc[2], wn);
     // x with the mean velocity (the paper's step) or with u^n (Heun stage)
     const double hx = A.K.euler ? dt : 0.5 * dt;
-    double x1 = xi + hx * (A.K.euler ? un : un + u1);
-    double y1 = yi + hx * (A.K.euler ? vn : vn + v1);
+    double x1 = __fma_rn(hx, A.K.euler ? un : __dadd_rn(un, u1), xi);
+    double y1 = __fma_rn(hx, A.K.euler ? vn : __dadd_rn(vn, v1), yi);
     if (PER) {  // periodic axes: back into [0, L)
       x1 = wrap_pos(x1, A.K.Lx);
       y1 = wrap_pos(y1, A.K.Ly);
     }
-    const double z1 = zi + hx * (A.K.euler ? wn : wn + w1);
+    const double z1 = __fma_rn(hx, A.K.euler ? wn : __dadd_rn(wn, w1), zi);
     A.uo[s] = u1; A.vo[s] = v1; A.wo[s] = w1;
     A.xo[s] = x1; A.yo[s] = y1; A.zo[s] = z1;
     A.Vo[s] = Vnext;
@@ -1221,7 +1330,7 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
       }
     }
     below = A.K.mirror_mode != LP_MIRROR_NONE && z1 < A.K.floor_z;
-  }
+  } while (false);
   warp_count(&A.dg->n_gas, live && regime == 0);
   warp_count(&A.dg->n_quasistatic, live && regime == 2);
   warp_count(&A.dg->n_over_c, live && overc);

@@ -1,0 +1,422 @@
+// Stencil rows in 64-bit fixed point: the sums of the LP_FP64 fits.
+//
+// GB300 issues FP64 at about 1.7 lanes per SM and clock, against 118 for FP32
+// and 25 for 32 x 32 + 64-bit integer multiply-adds (measured). A stencil's
+// sums took 82 FP64 operations per row in pass 1 and 36 in pass 2, and bound
+// the FP64 step (pass 1 5.6 ms, pass 2 2.7 ms on 786,000 particles). Every
+// factor of those sums is bounded once the row's scale is known, so here they
+// run in fixed point on the integer and FP32 pipes and only the 9 x 9
+// factor and solves stay FP64.
+//
+// A factor v is held as h + l, h a 28-bit integer and l the rest of it in
+// units of h, |l| <= 1/2, as a float. A sum of products a b is
+//   H += a.h b.h            exact, one 32 x 32 + 64-bit multiply-add
+//   M += a.h b.l + a.l b.h  two FP32 multiply-adds (a.l b.l is below 2^-56),
+//                           moved into H every four rows
+// so a sum errs by about 2^-51 of its largest possible term, less than an FP64
+// sum over the same rows, which rounds at 2^-53 of the running sum (36 rows) in
+// each row; 64 rows of 2^56 cannot overflow H. 7.0 cycles per accumulation and
+// scheduler, measured; an FP64 multiply-add takes about 75.
+//
+// Positions are integers X = x 2^k modulo 2^64, with r 2^k in (2^59, 2^60]
+// for the stencil radius r: the conversion is exact for all but the last bits
+// of tiny coordinates, and differences of neighbours are exact whatever the
+// distance from the origin (the modular wrap cancels). Field values (u, v, w;
+// |gdot|, V) are converted per stencil row with the exponent of the stencil's
+// largest difference, found in a first walk over FP32 copies.
+//
+// What does not fit (offsets beyond about the radius, which only stencils held
+// fixed over several steps can have; fields whose differences are not finite
+// or are below 2^-90; non-finite positions) is queued for a kernel that runs
+// the plain FP64 rows.
+#pragma once
+
+#include "lp_internal.cuh"
+
+namespace lp {
+
+// round(v 2^k) modulo 2^64 (0 for non-finite v, which callers sort out)
+__host__ __device__ __forceinline__ unsigned long long fx_of(double v, int k) {
+#ifdef __CUDA_ARCH__
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+#else
+  unsigned long long b;
+  __builtin_memcpy(&b, &v, sizeof b);
+#endif
+  const int e = (int)((b >> 52) & 0x7ff);
+  const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
+  const int sh = e - 1075 + k;
+  const unsigned long long left = sh < 64 ? m << (sh & 63) : 0ull;
+  const int t = -sh - 1;  // right shift by -sh, rounded
+  const unsigned long long right = t < 64 ? ((m >> (t & 63)) + 1ull) >> 1 : 0ull;
+  const unsigned long long r = sh >= 0 ? left : right;
+  return (b >> 63) ? 0ull - r : r;
+}
+
+// one particle of the rows: fixed-point position (with the FP32 coordinates
+// that choose the nearest image; xf is NaN for a non-finite position) and the
+// FP64 field values of the pass
+struct __align__(64) FxRec {
+  unsigned long long X, Y, Z;
+  float xf, yf;
+  double f[4];
+};
+
+struct FxV {  // value h + l; hf = float(h)
+  int h;
+  float hf, l;
+};
+__device__ __forceinline__ FxV fx_split(unsigned long long D) {
+  FxV v;
+  v.h = (int)((D + 0x80000000ull) >> 32);
+  v.hf = (float)v.h;
+  v.l = __fmul_rn((float)(int)(unsigned)D, 0x1p-32f);
+  return v;
+}
+// product of two values, rounded to an integer in units of h h
+__device__ __forceinline__ long long fx_mul(const FxV& a, const FxV& b) {
+  const float c = __fmaf_rn(a.l, b.hf, __fmul_rn(a.hf, b.l));
+  return (long long)a.h * b.h + (long long)__float2int_rn(c);
+}
+// a product as a factor again: units 2^sq
+__device__ __forceinline__ FxV fx_quad(long long Q, int sq, float qs) {
+  FxV v;
+  v.h = (int)((Q + (1ll << (sq - 1))) >> sq);
+  v.hf = (float)v.h;
+  v.l = __fmul_rn((float)(int)((unsigned)Q - ((unsigned)v.h << sq)), qs);
+  return v;
+}
+__device__ __forceinline__ void fx_acc(long long& H, float& M, const FxV& a, const FxV& b) {
+  H += (long long)a.h * b.h;
+  M = __fmaf_rn(a.hf, b.l, M);
+  M = __fmaf_rn(a.l, b.hf, M);
+}
+// M, rounded to an integer, moves into H: every fourth row (and after a row
+// that counts twice), so that |M| < 2^31 and its rounding stays small
+__device__ __forceinline__ void fx_flush(long long& H, float& M) {
+  H += (long long)__float2int_rn(M);
+  M = 0.f;
+}
+__device__ __forceinline__ bool fx_flush_at(int k) { return (k & 3) == 3; }
+__device__ __forceinline__ double pow2_of(int e) {  // 2^e, a normal double
+  return __longlong_as_double((long long)(1023 + e) << 52);
+}
+
+// offsets of entry j of a particle at `me` (PER: nearest images)
+template <bool PER>
+__device__ __forceinline__ void fx_offsets(const StepConsts& K, const FxRec& me,
+                                           unsigned long long Xj, unsigned long long Yj,
+                                           unsigned long long Zj, float xf, float yf, bool mir,
+                                           unsigned long long* D) {
+  D[0] = Xj - me.X;
+  D[1] = Yj - me.Y;
+  D[2] = (mir ? K.fx_F2 - Zj : Zj) - me.Z;
+  if (PER) {
+    const float dx = xf - me.xf, dy = yf - me.yf;
+    if (fabsf(dx) > K.fx_hLx) D[0] -= dx > 0.f ? K.fx_Lx : 0ull - K.fx_Lx;
+    if (fabsf(dy) > K.fx_hLy) D[1] -= dy > 0.f ? K.fx_Ly : 0ull - K.fx_Ly;
+  }
+}
+
+// row loop state: the neighbour's position one row ahead, its code two rows ahead
+struct FxPosLoad {
+  ulonglong2 xy;
+  ulonglong2 zf;  // Z and the two floats
+  __device__ __forceinline__ void fetch(const FxRec* R, uint32_t code, int n, int s) {
+    int j = code & kIndexMask;
+    if ((unsigned)j >= (unsigned)n) j = s;  // never read outside the arrays (row skipped)
+    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(R + j);
+    xy = p[0];
+    zf = p[1];
+  }
+  __device__ __forceinline__ float xf() const { return __uint_as_float((unsigned)zf.y); }
+  __device__ __forceinline__ float yf() const { return __uint_as_float((unsigned)(zf.y >> 32)); }
+};
+
+__device__ __forceinline__ void fx_rec_pos(FxRec& r, const FxRec* R, int s) {
+  FxPosLoad p;
+  const ulonglong2* q = reinterpret_cast<const ulonglong2*>(R + s);
+  p.xy = q[0];
+  p.zf = q[1];
+  r.X = p.xy.x; r.Y = p.xy.y; r.Z = p.zf.x;
+  r.xf = p.xf(); r.yf = p.yf();
+}
+
+__device__ __forceinline__ void fx_push(const StepArgs& A, int s, int list) {
+  A.slow[atomicAdd(&A.slow_count[list], 1)] = s;  // each particle once per list of n
+}
+
+// FP32 copy of a field for the scale walk: 0 only for 0, so that a tiny value
+// cannot pass for it
+__device__ __forceinline__ float fx_float(double v) {
+  const float f = __double2float_rn(v);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return (fabsf(f) < 0x1p-100f && (b << 1)) ? copysignf(0x1p-100f, (b >> 63) ? -1.f : 1.f) : f;
+}
+
+// records of pass 1: positions, u, v, w
+__device__ __forceinline__ void fx_split_state_body(const StepArgs& A, int s) {
+  FxRec* R = reinterpret_cast<FxRec*>(A.XU);
+  const double x = A.x[s], y = A.y[s], z = A.z[s];
+  const int k = A.K.fx_k;
+  FxRec r;
+  r.X = fx_of(x, k); r.Y = fx_of(y, k); r.Z = fx_of(z, k);
+  const bool fin = isfinite(x) && isfinite(y) && isfinite(z);
+  r.xf = fin ? __double2float_rn(x) : __int_as_float(0x7fffffff);
+  r.yf = __double2float_rn(y);
+  r.f[0] = A.u[s]; r.f[1] = A.v[s]; r.f[2] = A.w[s]; r.f[3] = 0.0;
+  R[s] = r;
+  A.fs[s] = make_float4(fx_float(r.f[0]), fx_float(r.f[1]), fx_float(r.f[2]), 0.f);
+}
+// fields of pass 2: |gdot|^n and the V of its fit
+__device__ __forceinline__ void fx_split_p1_body(const StepArgs& A, int s) {
+  FxRec* R = reinterpret_cast<FxRec*>(A.XU);
+  const double g = A.p1[P1_GN * A.n + s], v = A.K.euler ? A.V[s] : A.p1[P1_VN * A.n + s];
+  *reinterpret_cast<double2*>(&R[s].f[0]) = make_double2(g, v);
+  A.fs[s] = make_float4(fx_float(g), fx_float(v), 0.f, 0.f);
+}
+
+// The 31 moments of a stencil (order of ff_moments_add) in units of the
+// lattice spacing. GH: flagged entries (kGhostBit) also stand for their point
+// reflection, so they add their even moments twice and no odd ones. False: the
+// row does not fit the fixed-point range.
+template <bool PER, bool GH>
+__device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo) {
+  const int n = A.n;
+  const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
+  const StepConsts& K = A.K;
+  FxRec me;
+  fx_rec_pos(me, R, s);
+  long long H[31];
+  float M[31];  // (degree 2 needs no M)
+#pragma unroll
+  for (int q = 0; q < 31; ++q) { H[q] = 0; M[q] = 0.f; }
+  unsigned big = 0;  // OR of the offsets' magnitudes
+  bool bad = !(me.xf == me.xf);
+  uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
+  uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
+  FxPosLoad P;
+  P.fetch(R, code, n, s);
+  for (int k = 0; k < m; ++k) {
+    const uint32_t c0 = code;
+    const FxPosLoad p = P;
+    if (k + 1 < m) {
+      code = nxt;
+      P.fetch(R, code, n, s);
+      if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
+    }
+    if ((c0 & kIndexMask) >= (uint32_t)n) continue;  // stale or corrupt stencil entry
+    unsigned long long D[3];
+    fx_offsets<PER>(K, me, p.xy.x, p.xy.y, p.zf.x, p.xf(), p.yf(), c0 >> 31, D);
+    bad = bad || !(p.xf() == p.xf());
+    FxV d[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      d[a] = fx_split(D[a]);
+      big = max(big, (unsigned)(d[a].h ^ (d[a].h >> 31)));
+    }
+    long long Q[6] = {fx_mul(d[0], d[0]), fx_mul(d[1], d[1]), fx_mul(d[2], d[2]),
+                      fx_mul(d[0], d[1]), fx_mul(d[0], d[2]), fx_mul(d[1], d[2])};
+    FxV q[6];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) q[t] = fx_quad(Q[t], K.fx_sq, K.fx_qs);
+    FxV w[6];  // the first factor of the even moments (twice for a flagged entry)
+    const bool twin = GH && (c0 & kGhostBit);
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      w[t] = q[t];
+      if (twin) {
+        w[t].h <<= 1; w[t].hf *= 2.f; w[t].l *= 2.f;
+        Q[t] <<= 1;
+      }
+      H[t] += Q[t];
+    }
+    if (twin) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) d[a] = FxV{0, 0.f, 0.f};
+    }
+    // q: 0 xx, 1 yy, 2 zz, 3 xy, 4 xz, 5 yz
+    fx_acc(H[6], M[6], d[0], q[0]);   fx_acc(H[7], M[7], d[1], q[1]);
+    fx_acc(H[8], M[8], d[2], q[2]);   fx_acc(H[9], M[9], d[1], q[0]);
+    fx_acc(H[10], M[10], d[2], q[0]); fx_acc(H[11], M[11], d[0], q[1]);
+    fx_acc(H[12], M[12], d[2], q[1]); fx_acc(H[13], M[13], d[0], q[2]);
+    fx_acc(H[14], M[14], d[1], q[2]); fx_acc(H[15], M[15], d[2], q[3]);
+    fx_acc(H[16], M[16], w[0], q[0]); fx_acc(H[17], M[17], w[1], q[1]);
+    fx_acc(H[18], M[18], w[2], q[2]); fx_acc(H[19], M[19], w[0], q[3]);
+    fx_acc(H[20], M[20], w[0], q[4]); fx_acc(H[21], M[21], w[1], q[3]);
+    fx_acc(H[22], M[22], w[1], q[5]); fx_acc(H[23], M[23], w[2], q[4]);
+    fx_acc(H[24], M[24], w[2], q[5]); fx_acc(H[25], M[25], w[0], q[1]);
+    fx_acc(H[26], M[26], w[0], q[2]); fx_acc(H[27], M[27], w[1], q[2]);
+    fx_acc(H[28], M[28], w[0], q[5]); fx_acc(H[29], M[29], w[1], q[4]);
+    fx_acc(H[30], M[30], w[2], q[3]);
+    if (fx_flush_at(k) || twin) {
+#pragma unroll
+      for (int t = 6; t < 31; ++t) fx_flush(H[t], M[t]);
+    }
+  }
+  if (bad || big > (unsigned)K.fx_lim) return false;
+#pragma unroll
+  for (int t = 0; t < 31; ++t) {
+    const double g = t < 6 ? K.fx_g2 : (t < 16 ? K.fx_g3 : K.fx_g4);
+    if (t >= 6) fx_flush(H[t], M[t]);
+    mo[t] = (double)H[t] * g;
+  }
+  return true;
+}
+
+__device__ __forceinline__ void gram_of_moments(const double* mo, double* L) {
+  Moments<double> M;
+  M.xx = mo[0]; M.yy = mo[1]; M.zz = mo[2]; M.xy = mo[3]; M.xz = mo[4]; M.yz = mo[5];
+  M.xxx = mo[6]; M.yyy = mo[7]; M.zzz = mo[8]; M.xxy = mo[9]; M.xxz = mo[10]; M.xyy = mo[11];
+  M.yyz = mo[12]; M.xzz = mo[13]; M.yzz = mo[14]; M.xyz = mo[15];
+  M.xxxx = mo[16]; M.yyyy = mo[17]; M.zzzz = mo[18]; M.xxxy = mo[19]; M.xxxz = mo[20];
+  M.xyyy = mo[21]; M.yyyz = mo[22]; M.xzzz = mo[23]; M.yzzz = mo[24]; M.xxyy = mo[25];
+  M.xxzz = mo[26]; M.yyzz = mo[27]; M.xxyz = mo[28]; M.xyyz = mo[29]; M.xyzz = mo[30];
+  M.gram(L);
+}
+
+// Right-hand sides A^T b of NF fields in column order, in units of the lattice
+// spacing; sgn: the factor (-1, 0, 1) of a field at a floor mirror; GH: bG is
+// the right-hand side of a flagged entry's ghost row. False: a field does not
+// fit (the caller queues the particle).
+template <int NF, bool PER, bool GH>
+__device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const int* sgn,
+                                       const double* bG, double (*R9)[kNB]) {
+  const int n = A.n;
+  const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
+  const StepConsts& K = A.K;
+  // the scale of each field: its largest difference in this stencil, in FP32
+  unsigned mx[NF];
+  float mf[NF];
+  {
+    const float4 v = A.fs[s];
+    const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      mf[f] = vv[f];
+      mx[f] = 0u;
+      if (GH) mx[f] = __float_as_uint(fx_float(bG[f])) & 0x7fffffffu;
+    }
+  }
+  constexpr int kChunk = 4;
+  for (int k0 = 0; k0 < m; k0 += kChunk) {
+    uint32_t cd[kChunk];
+    float4 v[kChunk];
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t)
+      cd[t] = k0 + t < m ? (uint32_t)A.nbr[(int64_t)(k0 + t) * n + s] : kIndexMask;
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t) {
+      const uint32_t j = cd[t] & kIndexMask;
+      v[t] = A.fs[j < (uint32_t)n ? j : (uint32_t)s];
+    }
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t) {
+      if ((cd[t] & kIndexMask) >= (uint32_t)n) continue;
+      const float vv[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
+      const bool mir = cd[t] >> 31;
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        const float d = (mir ? (float)sgn[f] * vv[f] : vv[f]) - mf[f];
+        mx[f] = max(mx[f], __float_as_uint(d) & 0x7fffffffu);
+      }
+    }
+  }
+  int kb[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    // a bound on the FP64 differences: the FP32 copies err by 2^-24 each
+    float B = __fmaf_rn(fabsf(mf[f]), 0x1p-22f, __uint_as_float(mx[f]) * (1.f + 0x1p-20f));
+    if (GH && K.free_surface) B *= 2.f;  // b +- bG
+    if (!(B < 0x1p120f) || (B > 0.f && B < 0x1p-90f)) return false;
+    const int e = (int)((__float_as_uint(B) + 0x007fffffu) >> 23) - 127;
+    kb[f] = B > 0.f ? 60 - e : 0;
+  }
+  FxRec me;
+  fx_rec_pos(me, R, s);
+  unsigned long long U[NF], G[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    U[f] = fx_of(R[s].f[f], kb[f]);
+    G[f] = GH ? fx_of(bG[f], kb[f]) : 0ull;
+  }
+  long long H[NF][kNB];
+  float M[NF][kNB];
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) { H[f][q] = 0; M[f][q] = 0.f; }
+  uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
+  uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
+  FxPosLoad P;
+  double uj[NF];
+  auto fetch = [&](uint32_t c) {
+    P.fetch(R, c, n, s);
+    const uint32_t j = c & kIndexMask;
+    const FxRec* r = R + (j < (uint32_t)n ? j : (uint32_t)s);
+    const double2 a = *reinterpret_cast<const double2*>(&r->f[0]);
+    uj[0] = a.x;
+    if (NF > 1) uj[1 % NF] = a.y;
+    if (NF > 2) uj[2 % NF] = r->f[2];
+  };
+  fetch(code);
+  for (int k = 0; k < m; ++k) {
+    const uint32_t c0 = code;
+    const FxPosLoad p = P;
+    double u0[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) u0[f] = uj[f];
+    if (k + 1 < m) {
+      code = nxt;
+      fetch(code);
+      if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
+    }
+    if ((c0 & kIndexMask) >= (uint32_t)n) continue;  // stale or corrupt stencil entry
+    const bool mir = c0 >> 31;
+    unsigned long long D[3];
+    fx_offsets<PER>(K, me, p.xy.x, p.xy.y, p.zf.x, p.xf(), p.yf(), mir, D);
+    FxV a[kNB];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) a[t] = fx_split(D[t]);
+    a[3] = fx_quad(fx_mul(a[0], a[0]), K.fx_sq, K.fx_qs);
+    a[4] = fx_quad(fx_mul(a[1], a[1]), K.fx_sq, K.fx_qs);
+    a[5] = fx_quad(fx_mul(a[2], a[2]), K.fx_sq, K.fx_qs);
+    a[6] = fx_quad(fx_mul(a[0], a[1]), K.fx_sq, K.fx_qs);
+    a[7] = fx_quad(fx_mul(a[0], a[2]), K.fx_sq, K.fx_qs);
+    a[8] = fx_quad(fx_mul(a[1], a[2]), K.fx_sq, K.fx_qs);
+    const bool twin = GH && (c0 & kGhostBit);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      unsigned long long u = fx_of(u0[f], kb[f]);
+      if (mir) u = sgn[f] < 0 ? 0ull - u : (sgn[f] ? u : 0ull);
+      const unsigned long long d = u - U[f];
+      // a ghost row is T(-offset) with right-hand side bG: with the entry's own
+      // row, linear terms take b - bG and quadratic ones b + bG
+      const FxV bl = fx_split(twin ? d - G[f] : d);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) fx_acc(H[f][q], M[f][q], bl, a[q]);
+      const FxV bq = GH ? fx_split(twin ? d + G[f] : d) : bl;
+#pragma unroll
+      for (int q = 3; q < kNB; ++q) fx_acc(H[f][q], M[f][q], bq, a[q]);
+    }
+    if (fx_flush_at(k)) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int q = 0; q < kNB; ++q) fx_flush(H[f][q], M[f][q]);
+    }
+  }
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    const double ub = pow2_of(32 - kb[f]);
+    const double ul = ub * K.fx_lin, uq = ub * K.fx_quad;
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) {
+      fx_flush(H[f][q], M[f][q]);
+      R9[f][q] = (double)H[f][q] * (q < 3 ? ul : (q < 6 ? 0.5 * uq : uq));
+    }
+  }
+  return true;
+}
+
+}  // namespace lp

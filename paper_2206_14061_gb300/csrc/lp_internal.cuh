@@ -77,6 +77,15 @@ struct StepConsts {
   float ih_h, ih_l, ih2_h, ih2_l;  // 1/h and 1/h^2 as float-float
   float phic_h, phic_l;            // phi_c as float-float
   float rho;                       // bound on |offset| / h of a stencil entry (r/h, rounded up)
+  // fixed-point rows (fixed_rows.cuh): positions are x 2^fx_k, products of two
+  // offsets are cut by 2^fx_sq (fx_qs = 2^-fx_sq), fx_lim bounds the integer
+  // part of an offset; factors from integer sums of degree 2, 3, 4 (moments)
+  // and 1, 2 (right-hand sides) to units of h; the mirror plane and the
+  // periods in fixed point; half periods (infinite without)
+  int fx_k, fx_sq, fx_lim;
+  float fx_qs, fx_hLx, fx_hLy;
+  double fx_g2, fx_g3, fx_g4, fx_lin, fx_quad;
+  unsigned long long fx_F2, fx_Lx, fx_Ly;
   long long ghost_PX, ghost_PY;
   double ghost_grid, ghost_hk, ghost_V, ghost_num;
   long long ghost_R2, ghost_clear2;
@@ -276,7 +285,11 @@ struct StepArgs {
   // into hi and lo floats (w = mirror height), velocities split likewise,
   // |gdot| and V^{n+1} split (hi, lo, hi, lo), Gram matrices in float-float
   const GridCol* grids;
-  FF8* XU;  // split positions and velocities
+  FF8* XU;  // split positions and velocities (FP64: the fixed-point records, FxRec)
+  float4* fs;           // FP64: FP32 copies of the fields of the pass
+  int32_t* slow;        // FP64: particles queued for the plain FP64 rows (pass 1, then pass 2)
+  int* slow_count;      // their numbers in pass 1 and pass 2
+  uint8_t* kx;          // FP64: 1 where the offsets do not fit the fixed-point rows
   float2* R1;   // LP_MIXED_FF: pass 1's right-hand sides (27 float-float, k-major)
   float2* P1s;  // LP_MIXED_FF: gdot (6) and ld (3) of pass 1 as float-float, k-major
                 // (null in the other modes)
@@ -401,19 +414,21 @@ struct Closure {
 };
 __device__ __forceinline__ Closure closure_at(double phi, const ColMui& m, double phi_c,
                                               double phi_min) {
-  const double a = phi_c - phi_min;
-  const double w = phi_c - phi;
-  const double k = 4.0 * a * a * m.d * m.d;
+  // (multiply-adds written out: the same bits in every kernel)
+  const double a = __dsub_rn(phi_c, phi_min);
+  const double w = __dsub_rn(phi_c, phi);
+  const double k = __dmul_rn(__dmul_rn(__dmul_rn(__dmul_rn(4.0, a), a), m.d), m.d);
   Closure c;
   const double iw = 1.0 / w;
-  c.M = -k * iw * iw;
-  const double den = a * m.I0 + w;
-  const double iden = 1.0 / den;
-  c.mu = (a * m.mu_s * m.I0 + m.mu_2 * w) * iden;
-  c.N = -c.M * c.mu;
-  c.S = -2.0 * k * iw * iw * iw;
-  const double dmu = -(a * m.I0 * (m.mu_2 - m.mu_s)) * iden * iden;
-  c.R = -c.S * c.mu - c.M * dmu;
+  const double kw2 = __dmul_rn(__dmul_rn(k, iw), iw);
+  c.M = -kw2;
+  const double aI0 = __dmul_rn(a, m.I0);
+  const double iden = 1.0 / __dadd_rn(aI0, w);
+  c.mu = __dmul_rn(__fma_rn(m.mu_2, w, __dmul_rn(__dmul_rn(a, m.mu_s), m.I0)), iden);
+  c.N = __dmul_rn(kw2, c.mu);
+  c.S = __dmul_rn(__dmul_rn(-2.0, kw2), iw);
+  const double dmu = -__dmul_rn(__dmul_rn(__dmul_rn(aI0, __dsub_rn(m.mu_2, m.mu_s)), iden), iden);
+  c.R = __fma_rn(kw2, dmu, -__dmul_rn(c.S, c.mu));
   return c;
 }
 
@@ -462,6 +477,67 @@ __device__ __forceinline__ void chol9_solve(const T* L, TB* b) {
 #pragma unroll
     for (int k = i + 1; k < kNB; ++k) s -= TB(L[tri(k, i)]) * b[k];
     b[i] = s * TB(L[tri(i, i)]);
+  }
+}
+
+// The same factor and solve for the fixed-point rows of LP_FP64, whose kernels
+// are bound by the FP64 pipe: multiply-adds written out (every kernel gets the
+// same bits), one call per column (as a loop over the columns the factor is not
+// unrolled and lives in local memory), and 1/sqrt in 5 operations.
+//
+// 1 / sqrt(v) for a positive normal v: the hardware's approximation (about 20
+// bits) and one step of Halley's third-order iteration y (1 + e/2 + 3 e^2/8),
+// e = 1 - v y^2, which leaves the rounding of the step itself (about 1 ulp).
+__device__ __forceinline__ double inv_sqrt(double v) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+  const double e = __fma_rn(-__dmul_rn(v, y), y, 1.0);
+  return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
+}
+template <int J>
+__device__ __forceinline__ bool fx_chol9_column(double* a, double rel_tol) {
+  double d = a[tri(J, J)];
+  const double d0 = d;
+#pragma unroll
+  for (int k = 0; k < J; ++k) d = __fma_rn(-a[tri(J, k)], a[tri(J, k)], d);
+  const bool good = d > rel_tol * d0;
+  const double inv = good ? inv_sqrt(d) : 0.0;
+  a[tri(J, J)] = inv;
+#pragma unroll
+  for (int i = J + 1; i < kNB; ++i) {
+    double s = a[tri(i, J)];
+#pragma unroll
+    for (int k = 0; k < J; ++k) s = __fma_rn(-a[tri(i, k)], a[tri(J, k)], s);
+    a[tri(i, J)] = __dmul_rn(s, inv);
+  }
+  return good;
+}
+__device__ __forceinline__ bool fx_chol9(double* a, double rel_tol) {
+  bool ok = fx_chol9_column<0>(a, rel_tol);
+  ok = fx_chol9_column<1>(a, rel_tol) && ok;
+  ok = fx_chol9_column<2>(a, rel_tol) && ok;
+  ok = fx_chol9_column<3>(a, rel_tol) && ok;
+  ok = fx_chol9_column<4>(a, rel_tol) && ok;
+  ok = fx_chol9_column<5>(a, rel_tol) && ok;
+  ok = fx_chol9_column<6>(a, rel_tol) && ok;
+  ok = fx_chol9_column<7>(a, rel_tol) && ok;
+  ok = fx_chol9_column<8>(a, rel_tol) && ok;
+  return ok;
+}
+__device__ __forceinline__ void fx_chol9_solve(const double* L, double* b) {
+#pragma unroll
+  for (int i = 0; i < kNB; ++i) {
+    double s = b[i];
+#pragma unroll
+    for (int k = 0; k < i; ++k) s = __fma_rn(-L[tri(i, k)], b[k], s);
+    b[i] = __dmul_rn(s, L[tri(i, i)]);
+  }
+#pragma unroll
+  for (int i = kNB - 1; i >= 0; --i) {
+    double s = b[i];
+#pragma unroll
+    for (int k = i + 1; k < kNB; ++k) s = __fma_rn(-L[tri(k, i)], b[k], s);
+    b[i] = __dmul_rn(s, L[tri(i, i)]);
   }
 }
 

@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(kBlock, PREC == LP_MIXED_FF ? 4 : 3)
     phase_stamp(P, LP_PHASE_NEIGHBORS);
   }
   if (tid == 0) *S.fb_count = 0;
+  if (PREC == LP_FP64 && tid == 0) S.slow_count[0] = S.slow_count[1] = 0;
   if (P.save_y0) {  // Heun's method: the state at the start of the step
     const double* src[7] = {S.x, S.y, S.z, S.u, S.v, S.w, S.V};
     for (int s = tid; s < n; s += nth)
@@ -205,7 +206,20 @@ __global__ void __launch_bounds__(kBlock, PREC == LP_MIXED_FF ? 4 : 3)
   }
   if (PREC == LP_MIXED_FF)
     for (int s = tid; s < n; s += nth) split_state_body(S, s);
+  if (PREC == LP_FP64)
+    for (int s = tid; s < n; s += nth) fx_split_state_body(S, s);
   LP_SYNC_OR_LEAVE();
+  if (PREC == LP_FP64) {  // fixed-point rows, then the particles they left (the factor of a
+                          // particle is read back by the thread that stored it)
+    for (int s = tid; s < n; s += nth) {
+      gram_fx_body<true, true>(S, s);
+      pass1_fx_body<true>(S, s);
+    }
+    LP_SYNC_OR_LEAVE();
+    const int nsl = min(S.slow_count[0], n);
+    for (int t = tid; t < nsl; t += nth) pass1_body<LP_FP64, true>(S, S.slow[t]);
+    LP_SYNC_OR_LEAVE();
+  }
   if (PREC == LP_MIXED_FF) {
     for (int s = tid; s < n; s += nth) {
       if (S.K.free_surface) gram_twins_body<true>(S, s);  // read back by the same thread
@@ -213,8 +227,10 @@ __global__ void __launch_bounds__(kBlock, PREC == LP_MIXED_FF ? 4 : 3)
     }
     LP_SYNC_OR_LEAVE();
   }
-  for (int s = tid; s < n; s += nth) pass1_body<PREC, true>(S, s);
-  LP_SYNC_OR_LEAVE();
+  if (PREC != LP_FP64) {
+    for (int s = tid; s < n; s += nth) pass1_body<PREC, true>(S, s);
+    LP_SYNC_OR_LEAVE();
+  }
   const int nfb = min(*S.fb_count, S.fb_cap);
   for (int t = tid; t < nfb; t += nth) pass1_fallback_item(S, t);
   if (tid == 0 && nfb > 0) atomicAdd(&S.dg->n_fallback, (unsigned long long)nfb);
@@ -224,12 +240,24 @@ __global__ void __launch_bounds__(kBlock, PREC == LP_MIXED_FF ? 4 : 3)
     for (int s = tid; s < n; s += nth) split_p1_body(S, s);
     LP_SYNC_OR_LEAVE();
   }
+  if (PREC == LP_FP64) {
+    for (int s = tid; s < n; s += nth) fx_split_p1_body(S, s);
+    LP_SYNC_OR_LEAVE();
+  }
   for (int t = tid; t < nfb; t += nth) pass2_fallback_item(S, t);
   LP_SYNC_OR_LEAVE();
   for (int base = 0; base < n; base += nth) {
     const int s = base + tid;
     if (PREC == LP_MIXED_FF && S.K.free_surface && s < n) pass2_twins_body<true>(S, s);
-    pass2_body<PREC, true>(S, s, s < n);
+    pass2_body<PREC == LP_FP64 ? kFixedRows : PREC, true>(S, s, s < n);
+  }
+  if (PREC == LP_FP64) {  // the particles the fixed-point rows left, a warp at a time
+    LP_SYNC_OR_LEAVE();
+    const int nsl = min(S.slow_count[1], n);
+    for (int b = tid & ~31; b < nsl; b += nth) {
+      const int t = b + (threadIdx.x & 31);
+      pass2_body<LP_FP64, true>(S, t < nsl ? S.slow[t] : 0, t < nsl);
+    }
   }
   if (P.phase_ns) {  // profiling: close pass 2
     LP_SYNC_OR_LEAVE();
