@@ -22,8 +22,9 @@
 // for the stencil radius r: the conversion is exact for all but the last bits
 // of tiny coordinates, and differences of neighbours are exact whatever the
 // distance from the origin (the modular wrap cancels). Field values (u, v, w;
-// |gdot|, V) are converted per stencil row with the exponent of the stencil's
-// largest difference, found in a first walk over FP32 copies.
+// |gdot|, V) are aligned per stencil to its largest value, and their differences
+// shifted up to fill the range; the scales come from a first walk over FP32
+// copies.
 //
 // What does not fit (offsets beyond about the radius, which only stencils held
 // fixed over several steps can have; fields whose differences are not finite
@@ -53,19 +54,36 @@ __host__ __device__ __forceinline__ unsigned long long fx_of(double v, int k) {
   return (b >> 63) ? 0ull - r : r;
 }
 
-// one particle of the rows: fixed-point position (with the FP32 coordinates
+// One particle of the rows: fixed-point position (with the FP32 coordinates
 // that choose the nearest image; xf is NaN for a non-finite position) and the
-// FP64 field values of the pass
+// field values of the pass as signed significands (53 bits, the top one at bit
+// 58) with their exponents, so that a row aligns a value to its stencil's scale
+// with one shift. A value is m 2^(e - 58).
 struct __align__(64) FxRec {
   unsigned long long X, Y, Z;
   float xf, yf;
-  double f[4];
+  long long m[3];
+  short e[4];
 };
+__device__ __forceinline__ void fx_field(double v, long long* m, short* e) {
+  const long long b = __double_as_longlong(v);
+  const int x = (int)((b >> 52) & 0x7ff);
+  // (subnormal values count as 0: they are queued by the scale walk)
+  const long long t = x ? ((b & 0xfffffffffffffll) | 0x10000000000000ll) << 6 : 0ll;
+  *m = b < 0 ? -t : t;
+  *e = (short)(x - 1023);
+}
 
 struct FxV {  // value h + l; hf = float(h)
   int h;
   float hf, l;
 };
+// (multiply-adds on 64-bit sums as one instruction each)
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
 __device__ __forceinline__ FxV fx_split(unsigned long long D) {
   FxV v;
   v.h = (int)((D + 0x80000000ull) >> 32);
@@ -76,7 +94,7 @@ __device__ __forceinline__ FxV fx_split(unsigned long long D) {
 // product of two values, rounded to an integer in units of h h
 __device__ __forceinline__ long long fx_mul(const FxV& a, const FxV& b) {
   const float c = __fmaf_rn(a.l, b.hf, __fmul_rn(a.hf, b.l));
-  return (long long)a.h * b.h + (long long)__float2int_rn(c);
+  return fx_mad(a.h, b.h, (long long)__float2int_rn(c));
 }
 // a product as a factor again: units 2^sq
 __device__ __forceinline__ FxV fx_quad(long long Q, int sq, float qs) {
@@ -87,14 +105,14 @@ __device__ __forceinline__ FxV fx_quad(long long Q, int sq, float qs) {
   return v;
 }
 __device__ __forceinline__ void fx_acc(long long& H, float& M, const FxV& a, const FxV& b) {
-  H += (long long)a.h * b.h;
+  H = fx_mad(a.h, b.h, H);
   M = __fmaf_rn(a.hf, b.l, M);
   M = __fmaf_rn(a.l, b.hf, M);
 }
 // M, rounded to an integer, moves into H: every fourth row (and after a row
 // that counts twice), so that |M| < 2^31 and its rounding stays small
 __device__ __forceinline__ void fx_flush(long long& H, float& M) {
-  H += (long long)__float2int_rn(M);
+  H = fx_mad(__float2int_rn(M), 1, H);
   M = 0.f;
 }
 __device__ __forceinline__ bool fx_flush_at(int k) { return (k & 3) == 3; }
@@ -164,15 +182,26 @@ __device__ __forceinline__ void fx_split_state_body(const StepArgs& A, int s) {
   const bool fin = isfinite(x) && isfinite(y) && isfinite(z);
   r.xf = fin ? __double2float_rn(x) : __int_as_float(0x7fffffff);
   r.yf = __double2float_rn(y);
-  r.f[0] = A.u[s]; r.f[1] = A.v[s]; r.f[2] = A.w[s]; r.f[3] = 0.0;
+  const double u = A.u[s], v = A.v[s], w = A.w[s];
+  fx_field(u, &r.m[0], &r.e[0]);
+  fx_field(v, &r.m[1], &r.e[1]);
+  fx_field(w, &r.m[2], &r.e[2]);
+  r.e[3] = 0;
   R[s] = r;
-  A.fs[s] = make_float4(fx_float(r.f[0]), fx_float(r.f[1]), fx_float(r.f[2]), 0.f);
+  A.fs[s] = make_float4(fx_float(u), fx_float(v), fx_float(w), 0.f);
 }
 // fields of pass 2: |gdot|^n and the V of its fit
 __device__ __forceinline__ void fx_split_p1_body(const StepArgs& A, int s) {
   FxRec* R = reinterpret_cast<FxRec*>(A.XU);
   const double g = A.p1[P1_GN * A.n + s], v = A.K.euler ? A.V[s] : A.p1[P1_VN * A.n + s];
-  *reinterpret_cast<double2*>(&R[s].f[0]) = make_double2(g, v);
+  longlong2 m;
+  long long mg, mv;
+  short eg, ev;
+  fx_field(g, &mg, &eg);
+  fx_field(v, &mv, &ev);
+  m.x = mg; m.y = mv;
+  *reinterpret_cast<longlong2*>(&R[s].m[0]) = m;
+  *reinterpret_cast<short2*>(&R[s].e[0]) = make_short2(eg, ev);
   A.fs[s] = make_float4(fx_float(g), fx_float(v), 0.f, 0.f);
 }
 
@@ -199,16 +228,16 @@ __device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, doub
   P.fetch(R, code, n, s);
   for (int k = 0; k < m; ++k) {
     const uint32_t c0 = code;
-    const FxPosLoad p = P;
-    if (k + 1 < m) {
+    const bool live = (c0 & kIndexMask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
+    unsigned long long D[3];
+    fx_offsets<PER>(K, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), c0 >> 31, D);
+    bad = bad || (live && !(P.xf() == P.xf()));
+    if (k + 1 < m) {  // (the position is taken: its registers hold the next one)
       code = nxt;
       P.fetch(R, code, n, s);
       if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
     }
-    if ((c0 & kIndexMask) >= (uint32_t)n) continue;  // stale or corrupt stencil entry
-    unsigned long long D[3];
-    fx_offsets<PER>(K, me, p.xy.x, p.xy.y, p.zf.x, p.xf(), p.yf(), c0 >> 31, D);
-    bad = bad || !(p.xf() == p.xf());
+    if (!live) continue;
     FxV d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -322,22 +351,29 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       }
     }
   }
-  int kb[NF];
+  // kb: differences are held as b 2^kb; et: values as v 2^(58 - et), exact for
+  // all but values far below the largest; lsh: from the second to the first
+  int kb[NF], et[NF], lsh[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     // a bound on the FP64 differences: the FP32 copies err by 2^-24 each
-    float B = __fmaf_rn(fabsf(mf[f]), 0x1p-22f, __uint_as_float(mx[f]) * (1.f + 0x1p-20f));
+    const float d = __uint_as_float(mx[f]) * (1.f + 0x1p-20f);
+    float B = __fmaf_rn(fabsf(mf[f]), 0x1p-22f, d);
+    const float V = __fmaf_rn(fabsf(mf[f]), 1.f + 0x1p-20f, d);  // and on the values
     if (GH && K.free_surface) B *= 2.f;  // b +- bG
     if (!(B < 0x1p120f) || (B > 0.f && B < 0x1p-90f)) return false;
-    const int e = (int)((__float_as_uint(B) + 0x007fffffu) >> 23) - 127;
-    kb[f] = B > 0.f ? 60 - e : 0;
+    const int eb = (int)((__float_as_uint(B) + 0x007fffffu) >> 23) - 127;
+    const int ev = (int)((__float_as_uint(V) + 0x007fffffu) >> 23) - 127;
+    kb[f] = B > 0.f ? 60 - eb : 0;
+    et[f] = B > 0.f ? ev : 0;
+    lsh[f] = B > 0.f ? ev - eb + 2 : 0;  // (>= 0: B <= 4 V)
   }
   FxRec me;
   fx_rec_pos(me, R, s);
   unsigned long long U[NF], G[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    U[f] = fx_of(R[s].f[f], kb[f]);
+    U[f] = (unsigned long long)(R[s].m[f] >> min(max(et[f] - R[s].e[f], 0), 63));
     G[f] = GH ? fx_of(bG[f], kb[f]) : 0ull;
   }
   long long H[NF][kNB];
@@ -349,32 +385,38 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
   uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
   uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
   FxPosLoad P;
-  double uj[NF];
+  longlong2 f01, f23;  // m[0], m[1]; m[2], exponents
   auto fetch = [&](uint32_t c) {
     P.fetch(R, c, n, s);
     const uint32_t j = c & kIndexMask;
-    const FxRec* r = R + (j < (uint32_t)n ? j : (uint32_t)s);
-    const double2 a = *reinterpret_cast<const double2*>(&r->f[0]);
-    uj[0] = a.x;
-    if (NF > 1) uj[1 % NF] = a.y;
-    if (NF > 2) uj[2 % NF] = r->f[2];
+    const longlong2* r = reinterpret_cast<const longlong2*>(&R[j < (uint32_t)n ? j : (uint32_t)s].m[0]);
+    f01 = r[0];
+    f23 = r[1];
   };
   fetch(code);
   for (int k = 0; k < m; ++k) {
     const uint32_t c0 = code;
-    const FxPosLoad p = P;
-    double u0[NF];
+    const bool live = (c0 & kIndexMask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
+    const bool mir = c0 >> 31;
+    unsigned long long D[3], u[NF];
+    fx_offsets<PER>(K, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), mir, D);
+    {
+      const long long mj[3] = {f01.x, f01.y, f23.x};
+      const int ej[3] = {(int)(short)f23.y, (int)f23.y >> 16, (int)(short)(f23.y >> 32)};
 #pragma unroll
-    for (int f = 0; f < NF; ++f) u0[f] = uj[f];
+      for (int f = 0; f < NF; ++f)
+        u[f] = (unsigned long long)(mj[f] >> min(max(et[f] - ej[f], 0), 63));
+    }
     if (k + 1 < m) {
       code = nxt;
       fetch(code);
       if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
     }
-    if ((c0 & kIndexMask) >= (uint32_t)n) continue;  // stale or corrupt stencil entry
-    const bool mir = c0 >> 31;
-    unsigned long long D[3];
-    fx_offsets<PER>(K, me, p.xy.x, p.xy.y, p.zf.x, p.xf(), p.yf(), mir, D);
+    if (!live) continue;
+    if (mir) {
+#pragma unroll
+      for (int f = 0; f < NF; ++f) u[f] = sgn[f] < 0 ? 0ull - u[f] : (sgn[f] ? u[f] : 0ull);
+    }
     FxV a[kNB];
 #pragma unroll
     for (int t = 0; t < 3; ++t) a[t] = fx_split(D[t]);
@@ -387,9 +429,7 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     const bool twin = GH && (c0 & kGhostBit);
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      unsigned long long u = fx_of(u0[f], kb[f]);
-      if (mir) u = sgn[f] < 0 ? 0ull - u : (sgn[f] ? u : 0ull);
-      const unsigned long long d = u - U[f];
+      const unsigned long long d = (u[f] - U[f]) << lsh[f];
       // a ghost row is T(-offset) with right-hand side bG: with the entry's own
       // row, linear terms take b - bG and quadratic ones b + bG
       const FxV bl = fx_split(twin ? d - G[f] : d);
