@@ -582,15 +582,16 @@ void launch_gather_fields(int n, const int32_t* idx, const double* const* src, d
 }
 
 void launch_adjoint_step(const AdjArgs& A, cudaStream_t st) {
-  const int nb = (A.n + kBlock - 1) / kBlock;
-  k_adj_prepare<<<nb, kBlock, 0, st>>>(A);
-  k_adj_accel<<<nb, kBlock, 0, st>>>(A);
-  k_adj_split<true><<<nb, kBlock, 0, st>>>(A);
-  if (A.K.periodic) k_adj_pass2<true><<<nb, kBlock, 0, st>>>(A);
-  else k_adj_pass2<false><<<nb, kBlock, 0, st>>>(A);
-  k_adj_split<false><<<nb, kBlock, 0, st>>>(A);
-  if (A.K.periodic) k_adj_pass1<true><<<nb, kBlock, 0, st>>>(A);
-  else k_adj_pass1<false><<<nb, kBlock, 0, st>>>(A);
+  const int bs = spread_block(A.n, kBlock);
+  const int nb = (A.n + bs - 1) / bs;
+  k_adj_prepare<<<nb, bs, 0, st>>>(A);
+  k_adj_accel<<<nb, bs, 0, st>>>(A);
+  k_adj_split<true><<<nb, bs, 0, st>>>(A);
+  if (A.K.periodic) k_adj_pass2<true><<<nb, bs, 0, st>>>(A);
+  else k_adj_pass2<false><<<nb, bs, 0, st>>>(A);
+  k_adj_split<false><<<nb, bs, 0, st>>>(A);
+  if (A.K.periodic) k_adj_pass1<true><<<nb, bs, 0, st>>>(A);
+  else k_adj_pass1<false><<<nb, bs, 0, st>>>(A);
 }
 
 }  // namespace lp

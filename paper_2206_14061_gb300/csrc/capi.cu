@@ -22,14 +22,14 @@ void launch_keys(int n, const double* x, const double* y, const double* z, const
 void exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t* tile_sum, int64_t n,
                     cudaStream_t st);
 int64_t scan_tiles(int64_t n);
+int scan_launches(int64_t n);
 void launch_scatter(int n, const uint32_t* key, const uint32_t* start, uint32_t* fill,
                     int32_t* tmp, cudaStream_t st, const int* search = nullptr);
-void launch_cell_sort(int64_t ncell, const uint32_t* start, int32_t* tmp, const int32_t* ids,
-                      cudaStream_t st, const int* search = nullptr);
-void launch_gather(int n, const int32_t* tmp, const double* const* src, double* const* dst,
-                   int nsrc, const int32_t* ids_in, int32_t* ids_out, const int32_t* col_in,
+void launch_gather(int n, const int32_t* tmp, const uint32_t* key, const uint32_t* start,
+                   int64_t ncell, const double* const* src, double* const* dst, int nsrc,
+                   const int32_t* ids_in, int32_t* ids_out, const int32_t* col_in,
                    int32_t* col_out, const GridCol* grids, float4* pf, cudaStream_t st,
-                   const int32_t* iota = nullptr, const int* search = nullptr);
+                   const int* search = nullptr);
 void launch_neighbors(int keep, int n, const double* x, const double* y, const double* z,
                       const float4* pf, const int32_t* colid, const int32_t* ids,
                       const GridCol* grids, const uint32_t* start, const double* radius,
@@ -388,14 +388,14 @@ void sort_particles(lp_ctx* c, int n, int kind, int nsrc, cudaStream_t st,
   // cells 0..ncell-1, the bucket of non-finite particles (ncell), the total
   exclusive_scan(count, start, c->tile, c->ncell + 2, st);
   launch_scatter(n, c->key, start, fill, c->tmp, st, search);
-  launch_cell_sort(c->ncell, start, c->tmp, c->ids[c->ci], st, search);
   const double* const* src = (const double* const*)(c->d_tab + ((d * 2 + kind) * 2 + 0) * kTabFields);
   double* const* dst = c->d_tab + ((d * 2 + kind) * 2 + 1) * kTabFields;
-  launch_gather(n, c->tmp, src, dst, nsrc, c->ids[c->ci], c->ids[1 - c->ci], c->colid[c->ci],
-                c->colid[1 - c->ci], c->d_grids, c->pf, st, c->iota, search);
+  launch_gather(n, c->tmp, c->key, start, c->ncell, src, dst, nsrc, c->ids[c->ci],
+                c->ids[1 - c->ci], c->colid[c->ci], c->colid[1 - c->ci], c->d_grids, c->pf, st,
+                search);
   c->cx ^= 1;
   c->ci ^= 1;
-  c->launches += 7;
+  c->launches += scan_launches(c->ncell + 2) + 3;
 }
 
 // Filter skipping between searches (VerletSkip); off with free-surface ghosts,

@@ -549,10 +549,12 @@ __global__ void k_mui_stress(int64_t n, ColMui mui, double phi_c, double phi_min
 // ------------------------------------------------------------- launchers
 
 void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
+  bs = spread_block(A.n, bs);
+  const int sb = spread_block(A.n, 256);  // of the splitting kernels
   const int nb = (A.n + bs - 1) / bs;
   const bool per = A.K.periodic != 0;
   if (prec == LP_FP64) {
-    k_fx_split<<<(A.n + 255) / 256, 256, 0, st>>>(A);
+    k_fx_split<<<(A.n + sb - 1) / sb, sb, 0, st>>>(A);
     if (A.perm) k_row_order<<<(A.n + kRowGroup - 1) / kRowGroup, kRowGroup, 0, st>>>(A.n, A.cnt, const_cast<int32_t*>(A.perm));
     const int b = bs < kFxBlock ? bs : kFxBlock;
     const int nf = (A.n + b - 1) / b;
@@ -571,7 +573,7 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
     if (per) k_pass1<LP_MIXED, true><<<nb, bs, 0, st>>>(A);
     else k_pass1<LP_MIXED, false><<<nb, bs, 0, st>>>(A);
   } else {
-    k_split_state<<<(A.n + 255) / 256, 256, 0, st>>>(A);
+    k_split_state<<<(A.n + sb - 1) / sb, sb, 0, st>>>(A);
     if (A.perm) k_row_order<<<(A.n + kRowGroup - 1) / kRowGroup, kRowGroup, 0, st>>>(A.n, A.cnt, const_cast<int32_t*>(A.perm));
     const int b = bs < kFFBlock ? bs : kFFBlock;
     const int nf = (A.n + b - 1) / b;
@@ -584,19 +586,21 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
       k_gram_ff<false><<<nf, b, 0, st>>>(A);
       k_pass1_ff_rows<false><<<nf, b, 0, st>>>(A);
     }
-    k_pass1_ff_solve<<<(A.n + kFFBlock - 1) / kFFBlock, kFFBlock, 0, st>>>(A);
+    k_pass1_ff_solve<<<nf, b, 0, st>>>(A);
   }
   k_pass1_fallback<<<152, 64, 0, st>>>(A);
 }
 void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
+  bs = spread_block(A.n, bs);
+  const int sb = spread_block(A.n, 256);  // of the splitting kernels
   if (prec == LP_MIXED_FF) {
-    k_split_p1<<<(A.n + 255) / 256, 256, 0, st>>>(A);
+    k_split_p1<<<(A.n + sb - 1) / sb, sb, 0, st>>>(A);
     if (A.K.free_surface) {
       if (A.K.periodic) k_pass2_twins<true><<<kTwinBlocks, 128, 0, st>>>(A);
       else k_pass2_twins<false><<<kTwinBlocks, 128, 0, st>>>(A);
     }
   }
-  if (prec == LP_FP64) k_fx_split_p1<<<(A.n + 255) / 256, 256, 0, st>>>(A);
+  if (prec == LP_FP64) k_fx_split_p1<<<(A.n + sb - 1) / sb, sb, 0, st>>>(A);
   k_pass2_fallback<<<152, 64, 0, st>>>(A);
   const int nb = (A.n + bs - 1) / bs;
   const bool per = A.K.periodic != 0;
@@ -622,16 +626,16 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
   }
 }
 void launch_fit(int prec, const FitArgs& F, cudaStream_t st) {
-  const int nb = (F.n + kBlock - 1) / kBlock;
+  const int bs = spread_block(F.n, kBlock);
+  const int nb = (F.n + bs - 1) / bs;
   if (prec == LP_FP64) {
-    k_fit<LP_FP64><<<nb, kBlock, 0, st>>>(F);
+    k_fit<LP_FP64><<<nb, bs, 0, st>>>(F);
   } else if (prec == LP_MIXED) {
-    k_fit<LP_MIXED><<<nb, kBlock, 0, st>>>(F);
+    k_fit<LP_MIXED><<<nb, bs, 0, st>>>(F);
   } else {
-    const int nf = (F.n + 127) / 128;
     k_fit_split_ff<<<(F.n + 255) / 256, 256, 0, st>>>(F);
-    k_fit_gram_ff<<<nf, 128, 0, st>>>(F);
-    for (int f0 = 0; f0 < F.nf; f0 += 2) k_fit_rhs_ff<2><<<nf, 128, 0, st>>>(F, f0);
+    k_fit_gram_ff<<<nb, bs, 0, st>>>(F);
+    for (int f0 = 0; f0 < F.nf; f0 += 2) k_fit_rhs_ff<2><<<nb, bs, 0, st>>>(F, f0);
   }
   k_fit_fallback<<<152, 64, 0, st>>>(F);
 }

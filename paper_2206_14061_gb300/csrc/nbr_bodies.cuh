@@ -93,8 +93,43 @@ __device__ __forceinline__ void cell_sort_body(int64_t c, const uint32_t* __rest
   }
 }
 
+// Sorted slot of the particle in arrival slot t of its cell: its rank by
+// original index among the cell's particles (the order cell_sort_body gives).
+// A cell crowded beyond kSortCap and the bucket of non-finite particles keep
+// their arrival order.
+__device__ __forceinline__ int rank_slot(int t, int s, uint32_t ncell,
+                                         const uint32_t* __restrict__ key,
+                                         const uint32_t* __restrict__ start,
+                                         const int32_t* __restrict__ tmp,
+                                         const int32_t* __restrict__ ids) {
+  const uint32_t c = key[s];
+  if (c >= ncell) return t;
+  const uint32_t b = start[c], e = start[c + 1];
+  if (e - b > kSortCap) return t;
+  const int32_t k = ids[s];
+  int r = 0;
+  for (uint32_t j = b; j < e; ++j) r += ids[tmp[j]] < k;
+  return (int)b + r;
+}
+
 // Gather the state into the new order; FP32 origin-relative positions for the
-// prefilter.
+// prefilter. Particle s of the old order goes to slot t of the new one.
+__device__ __forceinline__ void gather_to(int t, int s, const double* const* __restrict__ src,
+                                          double* const* __restrict__ dst, int nsrc,
+                                          const int32_t* __restrict__ ids_in,
+                                          int32_t* __restrict__ ids_out,
+                                          const int32_t* __restrict__ col_in,
+                                          int32_t* __restrict__ col_out,
+                                          const GridCol* __restrict__ grids,
+                                          float4* __restrict__ pf) {
+  for (int f = 0; f < nsrc; ++f) dst[f][t] = src[f][s];
+  ids_out[t] = ids_in[s];
+  const int c = col_in[s];
+  col_out[t] = c;
+  const GridCol g = grids[c];
+  pf[t] = make_float4(__double2float_rn(src[0][s] - g.ox), __double2float_rn(src[1][s] - g.oy),
+                      __double2float_rn(src[2][s] - g.oz), 0.f);
+}
 __device__ __forceinline__ void gather_body(int t, int n, const int32_t* __restrict__ tmp,
                                             const double* const* __restrict__ src,
                                             double* const* __restrict__ dst, int nsrc,
@@ -106,13 +141,7 @@ __device__ __forceinline__ void gather_body(int t, int n, const int32_t* __restr
                                             float4* __restrict__ pf) {
   int s = tmp[t];
   if ((unsigned)s >= (unsigned)n) s = t;  // stay inside the buffers whatever tmp holds
-  for (int f = 0; f < nsrc; ++f) dst[f][t] = src[f][s];
-  ids_out[t] = ids_in[s];
-  const int c = col_in[s];
-  col_out[t] = c;
-  const GridCol g = grids[c];
-  pf[t] = make_float4(__double2float_rn(src[0][s] - g.ox), __double2float_rn(src[1][s] - g.oy),
-                      __double2float_rn(src[2][s] - g.oz), 0.f);
+  gather_to(t, s, src, dst, nsrc, ids_in, ids_out, col_in, col_out, grids, pf);
 }
 
 // FP32 offset along an axis of period L (float), nearest image; with L = 0
