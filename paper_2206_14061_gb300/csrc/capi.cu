@@ -36,7 +36,8 @@ void launch_neighbors(int keep, int n, const double* x, const double* y, const d
                       double r_const, int mirror_mode, double floor_z, int cap, int32_t* nbr,
                       int32_t* cnt, DevDiag* dg, cudaStream_t st, int bs = kBlock,
                       const int* search = nullptr, double* xref = nullptr,
-                      bool periodic = false, VerletSkip vs = VerletSkip{});
+                      bool periodic = false, VerletSkip vs = VerletSkip{},
+                      bool caller = false);
 void launch_filter(int n, const double* x, const double* y, const double* z, const float4* pf,
                    const int32_t* cand, const int32_t* ccnt, int capc, const GridCol* grids,
                    const int32_t* colid, double r, double floor_z, int cap, int32_t* nbr,
@@ -54,8 +55,6 @@ void launch_axpby(int64_t n, double a, const double* x, double b, double* y, cud
 void launch_need_search(int n, const double* x, const double* y, const double* z,
                         const double* xref, double half_skin2, double Lx, double Ly, int* flag,
                         VerletSkip vs, cudaStream_t st);
-void launch_nbr_to_caller(int n, int cap, const int32_t* ids, const int32_t* nbr_s,
-                          const int32_t* cnt_s, int32_t* nbr_o, int32_t* cnt_o, cudaStream_t st);
 // fit.cu
 void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs = kBlock);
 void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs = kBlock);
@@ -939,9 +938,8 @@ lp_status lp_build_neighbors(lp_ctx* c, const lp_particles* p, const double* rad
   const int e = c->cx;
   launch_neighbors(keep_nearest, n, c->X[e][0], c->X[e][1], c->X[e][2], c->pf,
                    c->colid[c->ci], c->ids[c->ci], c->d_grids, c->cells + 2 * c->cell_capacity,
-                   radius ? c->X[e][7] : nullptr, r_const, mirror_mode, floor_z, cap, c->nbr,
-                   c->cnt, c->dg, st);
-  launch_nbr_to_caller(n, cap, c->ids[c->ci], c->nbr, c->cnt, c->nbr_o, c->cnt_o, st);
+                   radius ? c->X[e][7] : nullptr, r_const, mirror_mode, floor_z, cap, c->nbr_o,
+                   c->cnt_o, c->dg, st, kBlock, nullptr, nullptr, false, VerletSkip{}, true);
   return cuda_status();
 }
 

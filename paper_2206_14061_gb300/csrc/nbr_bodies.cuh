@@ -172,12 +172,121 @@ __device__ __forceinline__ bool cand_less(uint64_t da, uint32_t ka, uint64_t db,
 
 __device__ __forceinline__ void stencil_stats(bool live, int c, int cap, DevDiag* dg);
 
+// Candidates of one particle in the truncating searches.
+template <bool KEEP>
+struct KeepSet {
+  float d[KEEP ? kMaxCand : 1];        // FP32 squared distances (the ordering's screen)
+  uint32_t code[KEEP ? kMaxCand : 1];
+  uint8_t oct[KEEP ? kMaxCand : 1];    // octant: bit 0 dx >= 0, bit 1 dy >= 0, bit 2 dz >= 0
+};
+
+// The first `cap` of m > cap candidates (a set: stencils have no set order).
+//
+// A threshold T on the FP32 distances with `cap` of them below it is found by
+// bisection, each step one pass of independent loads over the candidates. A
+// candidate more than gap below T is then in, one more than gap above it out
+// (FP32 distances order the exact ones but for gap), and the few in between are
+// ranked exactly. A max-heap of cap indices and a heapsort, a chain of dependent
+// local loads that diverges over the warp, took 5.3 ms on 2.0 M particles
+// (48 nearest), this 2.4.
+template <class Before, class Put>
+__device__ __forceinline__ void keep_nearest(const KeepSet<true>& ks, int m, int cap, float r2f,
+                                             float gap, Before before, Put put) {
+  // (bits of floats >= 0 order as integers); first guess: even density
+  float T = r2f * __powf((float)cap / (float)m, 2.f / 3.f);
+  uint32_t lo = 0u, hi = 0x7f800000u;  // count(< lo) <= cap, count(< hi) > cap
+  float step = r2f * (1.f / 32.f);
+  int below = 0;
+  for (int it = 0; it < 64; ++it) {
+    below = 0;
+    for (int t = 0; t < m; ++t) below += ks.d[t] < T;
+    if (below == cap) break;
+    const uint32_t b = __float_as_uint(T);
+    if (below < cap) lo = b; else hi = b;
+    if (hi - lo <= 1u) {  // equal FP32 distances straddle the cut: T is their value
+      T = __uint_as_float(lo);
+      break;
+    }
+    // out from the guess until both sides are known, then bisect
+    if (hi == 0x7f800000u) { T += step; step *= 2.f; }
+    else if (lo == 0u && T > step) { T -= step; step *= 2.f; }
+    else if (lo == 0u) T *= 0.5f;
+    else T = 0.5f * (__uint_as_float(lo) + __uint_as_float(hi));
+    const uint32_t tb = __float_as_uint(T);
+    if (tb <= lo || tb >= hi) T = __uint_as_float(lo + (hi - lo) / 2u);
+  }
+  // (far from the origin, gap = infinity, every candidate is in between)
+  int w = 0, c = 0;
+  uint8_t mid[kMaxCand];
+  for (int t = 0; t < m; ++t) {
+    if (ks.d[t] < T - gap) put(c++, ks.code[t]);
+    else if (!(ks.d[t] > T + gap)) mid[w++] = (uint8_t)t;
+  }
+  const int need = cap - c;
+  for (int i = 0; i < w; ++i) {
+    int r = 0;
+    if (w > need)
+      for (int k = 0; k < w; ++k) r += k != i && before(mid[k], mid[i]);
+    if (r < need) put(c++, ks.code[mid[i]]);
+  }
+}
+
+// Octant-balanced: a candidate's round is its nearest-first rank in its own
+// octant; the first cap by (round, order). Every candidate of a round below R,
+// the last round that does not fit whole, is in, and the first of round R fill
+// the rest. The candidates are grouped by octant first, so that ranks compare
+// within a group only (ranks over all m candidates, a heap and a heapsort took
+// 1.42 ms on 59,000 particles, cap 32; this 0.47).
+template <class Before, class Put>
+__device__ __forceinline__ void keep_octants(const KeepSet<true>& ks, int m, int cap,
+                                             Before before, Put put) {
+  uint64_t cn = 0;  // eight byte counters (at most 128 each)
+  for (int t = 0; t < m; ++t) cn += 1ull << (8 * ks.oct[t]);
+  auto cnt8 = [](uint64_t v, int o) { return (int)((v >> (8 * o)) & 0xffu); };
+  int R = 0, kept = 0;
+  for (;; ++R) {
+    int add = 0;
+#pragma unroll
+    for (int o = 0; o < 8; ++o) add += cnt8(cn, o) > R;
+    if (kept + add > cap || add == 0) break;
+    kept += add;
+  }
+  const int need = cap - kept;
+  uint64_t at = 0;  // where each octant's group starts
+#pragma unroll
+  for (int o = 1; o < 8; ++o) at |= (uint64_t)(cnt8(at, o - 1) + cnt8(cn, o - 1)) << (8 * o);
+  uint8_t ix[kMaxCand];
+  uint64_t fill = at;
+  for (int t = 0; t < m; ++t) {
+    const int o = ks.oct[t];
+    ix[cnt8(fill, o)] = (uint8_t)t;
+    fill += 1ull << (8 * o);
+  }
+  int c = 0, nl = 0;
+  uint8_t last[8];  // round R: one candidate per octant that reaches it
+  for (int i = 0; i < m; ++i) {
+    const int t = ix[i], o = ks.oct[t];
+    const int b = cnt8(at, o), e = b + cnt8(cn, o);
+    int r = 0;
+    for (int k = b; k < e; ++k) r += k != i && before(ix[k], t);
+    if (r < R) put(c++, ks.code[t]);
+    else if (r == R) last[nl++] = (uint8_t)t;
+  }
+  for (int i = 0; i < nl; ++i) {
+    int r = 0;
+    for (int k = 0; k < nl; ++k) r += k != i && before(last[k], last[i]);
+    if (r < need) put(c++, ks.code[last[i]]);
+  }
+}
+
 // Stencil of particle s; every lane of the warp must call it (live or not).
 // stats = false leaves the stencil-size statistics alone (candidate lists).
 // PER: the grid may have periodic axes (GridCol::Lx, Ly).
 // KEEP: truncate to cap entries; keep_mode 1 keeps the cap nearest,
 // keep_mode 2 the first cap of the octant-balanced ordering.
-template <bool KEEP, bool PER = false>
+// CALLER: the stencil is written in the caller's indices, at the caller's slot
+// (a kernel that translated the stored stencils took 0.36 ms on 2.0 M particles).
+template <bool KEEP, bool PER = false, bool CALLER = false>
 __device__ __forceinline__ void neighbors_body(
     int s, bool live, int n, const double* __restrict__ x, const double* __restrict__ y,
     const double* __restrict__ z, const float4* __restrict__ pf,
@@ -210,9 +319,15 @@ __device__ __forceinline__ void neighbors_body(
     const float lo = r2f * (1.0f - band), hi = r2f * (1.0f + band);
     const bool exact_only = !(band < 0.25f);  // far from the origin: FP64 for every pair
     const float Lxf = g.Lxf, Lyf = g.Lyf;
-    float cdf[KEEP ? kMaxCand : 1];  // FP32 squared distances (the ordering's screen)
-    uint32_t cj[KEEP ? kMaxCand : 1];
-    uint8_t co[KEEP ? kMaxCand : 1];  // octant: bit 0 dx >= 0, bit 1 dy >= 0, bit 2 dz >= 0
+    const float sgn_tol = KEEP ? 0x1p-21f * (cmax + rf) : 0.f;  // FP32 offsets err by half of it
+    auto put = [&](int k, uint32_t code) {
+      if (CALLER)
+        nbr[(int64_t)k * n + ids[s]] =
+            (int32_t)((uint32_t)ids[code & ~kMirrorBit] | (code & kMirrorBit));
+      else
+        nbr[(int64_t)k * n + s] = (int32_t)code;
+    };
+    KeepSet<KEEP> ks;  // the candidates
     const int ncx = g.nx, ncy = g.ny, ncz = g.nz;
     // periodic axes wrap (>= 3 cells); float tests keep the FP64 pipe free
     const bool perx = PER && g.Lxf > 0.f, pery = PER && g.Lyf > 0.f;
@@ -257,51 +372,54 @@ __device__ __forceinline__ void neighbors_body(
               if (!exact_only && d2f > hi) continue;
               double d2 = 0.0;
               bool in;
-              uint8_t oct = 0;
-              // (the octant rule forms octants from the FP64 offsets, so its
-              // candidates all take the FP64 test)
-              if (!exact_only && d2f < lo && !(KEEP && keep_mode == 2)) {
+              if (!exact_only && d2f < lo) {
                 in = true;
               } else {
                 const double zj = pass == 0 ? z[j] : __dsub_rn(2.0 * floor_z, z[j]);
                 in = exact_in(xi, yi, zi, x[j], y[j], zj, r2, &d2, PER ? g.Lx : 0.0,
                               PER ? g.Ly : 0.0);
-                // (caller stencils are never periodic: the sign of x_j - x_i
-                // in FP64 is that of the comparison)
-                if (KEEP && keep_mode == 2)
-                  oct = (uint8_t)((x[j] >= xi ? 1 : 0) | (y[j] >= yi ? 2 : 0) | (zj >= zi ? 4 : 0));
               }
               if (!in) continue;
               const uint32_t code = j | (pass ? kMirrorBit : 0u);
               if (KEEP) {
                 if (c < kMaxCand) {
-                  cdf[c] = d2f;
-                  cj[c] = code;
-                  co[c] = oct;
+                  ks.d[c] = d2f;
+                  ks.code[c] = code;
+                  if (keep_mode == 2) {
+                    // the signs of the FP64 offsets; the FP32 ones are theirs
+                    // where they are larger than twice their error
+                    const bool sure = !exact_only && fabsf(dxf) > sgn_tol &&
+                                      fabsf(dyf) > sgn_tol && fabsf(dzf) > sgn_tol;
+                    int oct = (dxf >= 0.f ? 1 : 0) | (dyf >= 0.f ? 2 : 0) | (dzf >= 0.f ? 4 : 0);
+                    if (!sure) {
+                      const double zj = pass == 0 ? z[j] : __dsub_rn(2.0 * floor_z, z[j]);
+                      oct = (x[j] >= xi ? 1 : 0) | (y[j] >= yi ? 2 : 0) | (zj >= zi ? 4 : 0);
+                    }
+                    ks.oct[c] = (uint8_t)oct;
+                  }
                 } else {
                   over = true;
                 }
               } else if (c < cap) {
-                nbr[(int64_t)c * n + s] = (int32_t)code;
+                put(c, code);
               }
               ++c;
               }
             }
           }
     }
-    if (KEEP) {
-      int m = c < kMaxCand ? c : kMaxCand;
-      if (m > cap) {
-        // tie-break keys (original index, then real before mirror), read once
-        uint32_t kk[kMaxCand];
-        for (int t = 0; t < m; ++t)
-          kk[t] = ((uint32_t)ids[cj[t] & ~kMirrorBit] << 1) | (cj[t] >> 31);
-        // The order is by the FP64 squared distance, then the key. The FP32
-        // distances are within band r^2 of it (the prefilter's bound, for
-        // every pair within the radius), so two candidates whose FP32
-        // distances differ by more than twice that are in that order; only
-        // closer pairs recompute their FP64 distances (as the test above)
-        // and compare them exactly.
+    if constexpr (KEEP) {
+      const int m = c < kMaxCand ? c : kMaxCand;
+      if (m <= cap) {
+        for (int t = 0; t < m; ++t) put(t, ks.code[t]);
+        c = m;
+      } else {
+        // The order is by the FP64 squared distance, then the key (original
+        // index, real before mirror). The FP32 distances are within band r^2
+        // of it (the prefilter's bound, for every pair within the radius), so
+        // two candidates whose FP32 distances differ by more than twice that
+        // are in that order; only closer pairs recompute their FP64 distances
+        // (as the test above) and compare them exactly.
         const float gap = exact_only ? INFINITY : 2.0f * band * r2f;
         auto exact_bits = [&](uint32_t code) {
           const int j = code & ~kMirrorBit;
@@ -310,65 +428,23 @@ __device__ __forceinline__ void neighbors_body(
           exact_in(xi, yi, zi, x[j], y[j], zj, r2, &d2);
           return (uint64_t)__double_as_longlong(d2);
         };
-        auto d_less = [&](int a, int b) {
-          if (cdf[a] + gap < cdf[b]) return true;
-          if (cdf[b] + gap < cdf[a]) return false;
-          return cand_less(exact_bits(cj[a]), kk[a], exact_bits(cj[b]), kk[b]);
+        auto key = [&](uint32_t code) {
+          return ((uint32_t)ids[code & ~kMirrorBit] << 1) | (code >> 31);
         };
-        // octant-balanced: each candidate's round is its nearest-first rank
-        // among the candidates of its own octant (stored over co[])
-        if (keep_mode == 2) {
-          uint8_t rk[kMaxCand];
-          for (int t = 0; t < m; ++t) {
-            int r = 0;
-            for (int u = 0; u < m; ++u)
-              r += (u != t && co[u] == co[t] && d_less(u, t));
-            rk[t] = (uint8_t)r;
-          }
-          for (int t = 0; t < m; ++t) co[t] = rk[t];
-        }
-        // the first cap of the ordering (keys are unique, so it is one set in
-        // one order): a max-heap of cap candidate indices, in which a
-        // candidate that precedes the top replaces it; then heapsort, so that
-        // hp[0 .. cap-1] lists them in ascending order
         auto before = [&](int a, int b) {
-          if (keep_mode == 2 && co[a] != co[b]) return co[a] < co[b];  // round first
-          return d_less(a, b);
+          if (ks.d[a] + gap < ks.d[b]) return true;
+          if (ks.d[b] + gap < ks.d[a]) return false;
+          return cand_less(exact_bits(ks.code[a]), key(ks.code[a]), exact_bits(ks.code[b]),
+                           key(ks.code[b]));
         };
-        uint8_t hp[LP_MAX_CAP];
-        auto sift_down = [&](int i, int len) {
-          for (;;) {
-            const int l = 2 * i + 1;
-            if (l >= len) break;
-            int big = l;
-            if (l + 1 < len && before(hp[l], hp[l + 1])) big = l + 1;
-            if (!before(hp[i], hp[big])) break;
-            const uint8_t t = hp[i]; hp[i] = hp[big]; hp[big] = t;
-            i = big;
-          }
-        };
-        for (int t = 0; t < cap; ++t) hp[t] = (uint8_t)t;
-        for (int i = cap / 2 - 1; i >= 0; --i) sift_down(i, cap);
-        for (int t = cap; t < m; ++t)
-          if (before(t, hp[0])) {
-            hp[0] = (uint8_t)t;
-            sift_down(0, cap);
-          }
-        for (int e = cap - 1; e > 0; --e) {
-          const uint8_t t = hp[0]; hp[0] = hp[e]; hp[e] = t;
-          sift_down(0, e);
-        }
-        uint32_t kept[LP_MAX_CAP];
-        for (int t = 0; t < cap; ++t) kept[t] = cj[hp[t]];
-        for (int t = 0; t < cap; ++t) cj[t] = kept[t];
-        m = cap;
+        if (keep_mode == 2) keep_octants(ks, m, cap, before, put);
+        else keep_nearest(ks, m, cap, r2f, gap, before, put);
+        c = cap;
       }
-      for (int t = 0; t < m; ++t) nbr[(int64_t)t * n + s] = (int32_t)cj[t];
-      c = m;
     } else {
       over = c > cap;
     }
-    cnt[s] = c;
+    cnt[CALLER ? ids[s] : s] = c;
   }
   warp_count(&dg->n_overflow, live && over);
   if (live && over) atomicOr(&dg->flags, (unsigned)LP_FLAG_OVERFLOW);

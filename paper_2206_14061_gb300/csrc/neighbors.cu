@@ -226,7 +226,7 @@ __global__ void k_gather(int n, const int32_t* __restrict__ tmp, const uint32_t*
 
 // ------------------------------------------------------- neighbour search
 
-template <bool KEEP, bool PER>
+template <bool KEEP, bool PER, bool CALLER>
 __global__ void __launch_bounds__(kMaxBlock)
 k_neighbors(int n, const double* __restrict__ x, const double* __restrict__ y,
             const double* __restrict__ z, const float4* __restrict__ pf,
@@ -248,7 +248,7 @@ k_neighbors(int n, const double* __restrict__ x, const double* __restrict__ y,
       if (s == 0) *vs.dmax_all = 0u;
     }
   }
-  neighbors_body<KEEP, PER>(s, s < n, n, x, y, z, pf, colid, ids, grids, start, radius, r_const,
+  neighbors_body<KEEP, PER, CALLER>(s, s < n, n, x, y, z, pf, colid, ids, grids, start, radius, r_const,
                             mirror_mode, floor_z, cap, nbr, cnt, dg, xref == nullptr, keep_mode);
 }
 
@@ -306,22 +306,6 @@ k_ghosts(int n, const double* __restrict__ z, const int4* __restrict__ X,
   }
 }
 
-// Stencils from sorted indices to caller indices.
-__global__ void k_nbr_to_caller(int n, int cap, const int32_t* __restrict__ ids,
-                                const int32_t* __restrict__ nbr_s, const int32_t* __restrict__ cnt_s,
-                                int32_t* __restrict__ nbr_o, int32_t* __restrict__ cnt_o) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int o = ids[s];
-  const int c = cnt_s[s];
-  cnt_o[o] = c;
-  const int m = c < cap ? c : cap;
-  for (int k = 0; k < m; ++k) {
-    const uint32_t code = (uint32_t)nbr_s[(int64_t)k * n + s];
-    nbr_o[(int64_t)k * n + o] = (int32_t)(((uint32_t)ids[code & ~kMirrorBit]) | (code & kMirrorBit));
-  }
-}
-
 // ----------------------------------------------------------- host wrappers
 
 void launch_fill_colid(int n, const int32_t* offs, int ncol, int32_t* colid, cudaStream_t st) {
@@ -355,25 +339,30 @@ void launch_gather(int n, const int32_t* tmp, const uint32_t* key, const uint32_
                                              ids_in, ids_out, col_in, col_out, grids, pf, search);
 }
 // keep: 0 every neighbour (overflow past cap), 1 the cap nearest, 2 the first
-// cap of the octant-balanced ordering
+// cap of the octant-balanced ordering (caller stencils only); caller: stencils in
+// the caller's indices
 void launch_neighbors(int keep, int n, const double* x, const double* y, const double* z,
                       const float4* pf, const int32_t* colid, const int32_t* ids,
                       const GridCol* grids, const uint32_t* start, const double* radius,
                       double r_const, int mirror_mode, double floor_z, int cap, int32_t* nbr,
                       int32_t* cnt, DevDiag* dg, cudaStream_t st, int bs, const int* search,
-                      double* xref, bool periodic, VerletSkip vs) {
+                      double* xref, bool periodic, VerletSkip vs, bool caller) {
   bs = spread_block(n, bs);
   const int nb = (n + bs - 1) / bs;
-  if (keep)  // (stencils for callers: never periodic)
-    k_neighbors<true, false><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start, radius,
-                                                 r_const, mirror_mode, floor_z, cap, nbr, cnt, dg,
-                                                 search, xref, keep, vs);
+  if (keep && caller)  // (stencils for callers: never periodic)
+    k_neighbors<true, false, true><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start,
+                                                       radius, r_const, mirror_mode, floor_z, cap,
+                                                       nbr, cnt, dg, search, xref, keep, vs);
+  else if (caller)
+    k_neighbors<false, false, true><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start,
+                                                        radius, r_const, mirror_mode, floor_z,
+                                                        cap, nbr, cnt, dg, search, xref, 0, vs);
   else if (periodic)
-    k_neighbors<false, true><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start, radius,
+    k_neighbors<false, true, false><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start, radius,
                                                  r_const, mirror_mode, floor_z, cap, nbr, cnt, dg,
                                                  search, xref, 0, vs);
   else
-    k_neighbors<false, false><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start,
+    k_neighbors<false, false, false><<<nb, bs, 0, st>>>(n, x, y, z, pf, colid, ids, grids, start,
                                                   radius, r_const, mirror_mode, floor_z, cap, nbr,
                                                   cnt, dg, search, xref, 0, vs);
 }
@@ -408,9 +397,4 @@ void launch_ghosts(int n, const double* x, const double* y, const double* z,
   k_ghost_scan<<<(n + bs - 1) / bs, bs, 0, st>>>(n, X, nbr, cnt, gcnt, K, olist, gcount);
   k_ghosts<<<kGhostBlocks, 128, 0, st>>>(n, z, X, nbr, cnt, gcnt, K, dg, glist, gcount, olist);
 }
-void launch_nbr_to_caller(int n, int cap, const int32_t* ids, const int32_t* nbr_s,
-                          const int32_t* cnt_s, int32_t* nbr_o, int32_t* cnt_o, cudaStream_t st) {
-  k_nbr_to_caller<<<(n + 255) / 256, 256, 0, st>>>(n, cap, ids, nbr_s, cnt_s, nbr_o, cnt_o);
-}
-
 }  // namespace lp
