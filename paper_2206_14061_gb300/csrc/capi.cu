@@ -96,6 +96,7 @@ struct lp_ctx {
   int32_t* cnt = nullptr;
   int32_t* nbr_o = nullptr;
   int32_t* cnt_o = nullptr;
+  double nbr_rmax = 0.0;      // largest radius of the stencils in nbr_o (0: none)
   double* p1 = nullptr;
   double* fac = nullptr;
   float* facf = nullptr;
@@ -137,9 +138,11 @@ struct lp_ctx {
   int32_t* olist = nullptr;   // particles with one-sided stencils (compact, any order)
   int* gcount = nullptr;      // the two lists' lengths
   int32_t* perm = nullptr;    // fit thread -> particle (LP_MIXED_FF, LP_FP64)
-  float4* fs = nullptr;       // FP32 copies of the fields (fixed-point rows of LP_FP64)
-  int32_t* slow = nullptr;    // particles left to the plain FP64 rows
-  uint8_t* kx = nullptr;      // 1: offsets outside the fixed-point range
+  // fixed-point rows of LP_FP64 (in P1s): FP32 copies of the fields, particles
+  // left to the plain FP64 rows, 1 where offsets are outside the range
+  float4* fs = nullptr;
+  int32_t* slow = nullptr;
+  uint8_t* kx = nullptr;
   float *Tg = nullptr, *T2 = nullptr;  // twin sums (allocated on first free-surface step)
   double* Y0[7] = {};                  // Heun: state at the start of the step (on first use)
   double* stage = nullptr;             // lp_step on host arrays: 7 x cap_n (on first use)
@@ -666,6 +669,32 @@ bool valid_params(const lp_params* q, const lp_eos* e, double dt) {
   return true;
 }
 
+// Scales of the fixed-point rows (fixed_rows.cuh) for the stencil radius r:
+// r 2^k = f 2^60 with f in (1/2, 1], so an offset's integer part is at most
+// f 2^28, and products are cut to at most 2^28 as well. fx_lim leaves a tenth
+// of the radius for stencils that are held while the particles move.
+// shifted: the rows shift a particle's offsets to its own largest one (up to
+// 2^12), and leave room for offsets beyond r.
+void fixed_consts(StepConsts& K, bool shifted = false) {
+  int e;
+  const double f = std::frexp(K.radius, &e);  // radius = f 2^e, f in [1/2, 1)
+  K.fx_k = (shifted ? 58 : 60) - e;
+  K.fx_mask = kIndexMask;
+  K.fx_sq = shifted || f * f <= 0.5 ? 27 : 28;
+  K.fx_qs = (float)std::ldexp(1.0, -K.fx_sq);
+  K.fx_lim = (int)((K.fx_sq == 27 ? 0.777 : 1.1) * 0x1p28);
+  const double unit = std::ldexp(1.0, 32 - K.fx_k);  // of an offset's integer part
+  const double l = unit * K.inv_h;
+  const double q = l * l * std::ldexp(1.0, K.fx_sq);  // of a product as a factor
+  K.fx_g2 = l * l; K.fx_g3 = l * q; K.fx_g4 = q * q;
+  K.fx_lin = l; K.fx_quad = q;
+  K.fx_F2 = fx_of(2.0 * K.floor_z, K.fx_k);
+  K.fx_Lx = fx_of(K.Lx, K.fx_k);
+  K.fx_Ly = fx_of(K.Ly, K.fx_k);
+  K.fx_hLx = K.Lx > 0.0 ? (float)(0.5 * K.Lx) : INFINITY;
+  K.fx_hLy = K.Ly > 0.0 ? (float)(0.5 * K.Ly) : INFINITY;
+}
+
 }  // namespace
 
 // ================================================================= C ABI
@@ -733,6 +762,11 @@ lp_status lp_ctx_create(const lp_ctx_desc* desc, lp_ctx** out) {
   if (s == LP_OK) s = dalloc(c, &c->bar, 2);
   if (s == LP_OK) s = dalloc(c, &c->XU, n);
   if (s == LP_OK) s = dalloc(c, &c->P1s, n * 9);
+  if (s == LP_OK) {  // FP64 passes use the float-float passes' block (72 B per particle)
+    c->fs = (float4*)c->P1s;
+    c->slow = (int32_t*)(c->fs + n);
+    c->kx = (uint8_t*)(c->slow + n);
+  }
   if (s == LP_OK) s = dalloc(c, &c->R1, n * 27);
   if (s == LP_OK) s = dalloc(c, &c->Lff, n * kTri);
   if (s == LP_OK) s = dalloc(c, &c->Xfix, n);
@@ -741,9 +775,6 @@ lp_status lp_ctx_create(const lp_ctx_desc* desc, lp_ctx** out) {
   if (s == LP_OK) s = dalloc(c, &c->olist, n);
   if (s == LP_OK) s = dalloc(c, &c->gcount, 2);
   if (s == LP_OK) s = dalloc(c, &c->perm, n);
-  if (s == LP_OK) s = dalloc(c, &c->fs, n);
-  if (s == LP_OK) s = dalloc(c, &c->slow, n);
-  if (s == LP_OK) s = dalloc(c, &c->kx, n);
   c->capc = std::min(c->cap + 32, 96);
   if (s == LP_OK) s = dalloc(c, &c->cand, n * c->capc);
   if (s == LP_OK) s = dalloc(c, &c->ccnt, n);
@@ -934,6 +965,7 @@ lp_status lp_build_neighbors(lp_ctx* c, const lp_particles* p, const double* rad
     if (!finite_pos(rmax)) return LP_ERR_INVALID_ARG;
   }
   LP_TRY(setup_grids(c, p->ncolumns, rmax, st));
+  c->nbr_rmax = rmax;
   sort_particles(c, n, 1, radius ? 4 : 3, st);
   const int e = c->cx;
   launch_neighbors(keep_nearest, n, c->X[e][0], c->X[e][1], c->X[e][2], c->pf,
@@ -1013,7 +1045,28 @@ lp_status lp_fit_derivatives(lp_ctx* c, const lp_particles* p, const lp_neighbor
     if (!c->fit_fs) LP_TRY(dalloc(c, &c->fit_fs, (size_t)kMaxFields * c->cap_n));
     F.xs = c->XU; F.fs = c->fit_fs; F.lf = c->Lff;
   }
-  cudaMemsetAsync(c->fb_count, 0, sizeof(int32_t), st);
+  if (LP_ROW_ORDER) F.perm = c->perm;
+  // FP64: rows in fixed point, the range laid out for the largest radius of the
+  // stencils where the context built them, else for four lattice spacings, and
+  // shifted to each particle's offsets. Offsets beyond three times that, or
+  // below a thousandth of it, take the plain rows, and so do mirror factors other
+  // than -1, 0 and 1.
+  StepArgs A{};
+  bool unit_signs = true;
+  for (int f = 0; f < nf; ++f)
+    unit_signs = unit_signs && (mirror_sign[f] == 0.0 || std::fabs(mirror_sign[f]) == 1.0);
+  if (precision == LP_FP64 && unit_signs) {
+    A.n = F.n; A.cap = F.cap; A.nbr = F.nbr; A.cnt = F.cnt;
+    A.XU = c->XU; A.fs = c->fs; A.slow = c->slow; A.slow_count = c->fb_count + 1; A.kx = c->kx;
+    A.fac = c->fac; A.dg = c->dg;
+    A.K.inv_h = F.inv_h;
+    A.K.floor_z = floor_z;
+    A.K.radius = nb->nbr == c->nbr_o && c->nbr_rmax > 0.0 ? c->nbr_rmax : 4.0 * h;
+    fixed_consts(A.K, true);
+    A.K.fx_mask = ~kMirrorBit;
+    F.rows = &A;
+  }
+  cudaMemsetAsync(c->fb_count, 0, 3 * sizeof(int32_t), st);
   launch_fit(precision, F, st);
   return cuda_status();
 }
@@ -1032,29 +1085,6 @@ lp_status lp_mui_stress(lp_ctx* c, const lp_mui* mui, const lp_eos* eos, int64_t
 }
 
 namespace {
-// Scales of the fixed-point rows (fixed_rows.cuh) for the stencil radius r:
-// r 2^k = f 2^60 with f in (1/2, 1], so an offset's integer part is at most
-// f 2^28, and products are cut to at most 2^28 as well. fx_lim leaves a tenth
-// of the radius for stencils that are held while the particles move.
-void fixed_consts(StepConsts& K) {
-  int e;
-  const double f = std::frexp(K.radius, &e);  // radius = f 2^e, f in [1/2, 1)
-  K.fx_k = 60 - e;
-  K.fx_sq = f * f <= 0.5 ? 27 : 28;
-  K.fx_qs = (float)std::ldexp(1.0, -K.fx_sq);
-  K.fx_lim = (int)((K.fx_sq == 27 ? 0.777 : 1.1) * 0x1p28);
-  const double unit = std::ldexp(1.0, 32 - K.fx_k);  // of an offset's integer part
-  const double l = unit * K.inv_h;
-  const double q = l * l * std::ldexp(1.0, K.fx_sq);  // of a product as a factor
-  K.fx_g2 = l * l; K.fx_g3 = l * q; K.fx_g4 = q * q;
-  K.fx_lin = l; K.fx_quad = q;
-  K.fx_F2 = fx_of(2.0 * K.floor_z, K.fx_k);
-  K.fx_Lx = fx_of(K.Lx, K.fx_k);
-  K.fx_Ly = fx_of(K.Ly, K.fx_k);
-  K.fx_hLx = K.Lx > 0.0 ? (float)(0.5 * K.Lx) : INFINITY;
-  K.fx_hLy = K.Ly > 0.0 ? (float)(0.5 * K.Ly) : INFINITY;
-}
-
 StepConsts step_consts(const lp_eos* eos, const lp_params* q, double dt, int cap) {
   StepConsts K{};
   K.phi_c = eos->phi_c; K.phi_min = eos->phi_min; K.phi_max = eos->phi_max;

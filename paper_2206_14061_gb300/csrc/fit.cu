@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_pass2_fx(const StepArgs A) {
   pass2_body<kFixedRows, PER, GH>(A, s, s < A.n);
 }
 // the particles that the fixed-point rows left to the plain FP64 rows
+constexpr int kSlowBlocks = 4 * 152;
 template <bool PER>
 __global__ void __launch_bounds__(64) k_pass1_slow(const StepArgs A) {
   const int cnt = min(A.slow_count[0], A.n);
@@ -207,9 +208,7 @@ __device__ __forceinline__ void write_coeffs(const FitArgs& F, int s, int f, con
 
 // fields are processed in groups of 4 right-hand sides per sweep
 template <int PREC>
-__global__ void __launch_bounds__(kBlock) k_fit(const FitArgs F) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= F.n) return;
+__device__ __forceinline__ void fit_body(const FitArgs& F, int s) {
   const int n = F.n;
   const int m = min(F.cnt[s], F.cap);
   const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
@@ -309,6 +308,109 @@ __global__ void __launch_bounds__(kBlock) k_fit(const FitArgs F) {
     for (int f = 0; f < nf; ++f) write_coeffs(F, s, f0 + f, c[f]);
   }
 }
+template <int PREC>
+__global__ void __launch_bounds__(kBlock) k_fit(const FitArgs F) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < F.n) fit_body<PREC>(F, s);
+}
+__device__ __forceinline__ int fit_thread(const FitArgs& F) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  return (F.perm && t < F.n) ? F.perm[t] : t;
+}
+
+// ---- lp_fit_derivatives in FP64 with the rows in fixed point (as the step's
+// pass 1, fixed_rows.cuh): records of the positions, moments and factor, then
+// the fields in groups of up to three. 170,000 particles, three fields: 1.61 ms
+// with FP64 rows, 0.40 now.
+constexpr uint8_t kFxSlow = 255;
+__global__ void k_fit_fx_split(const FitArgs F, const StepArgs A) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= F.n) return;
+  FxRec* R = reinterpret_cast<FxRec*>(A.XU);
+  fx_position(F.x[s], F.y[s], F.z[s], A.K.fx_k, R[s]);
+}
+__global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, const StepArgs A) {
+  const int s = fit_thread(F);
+  if (s >= F.n) return;
+  const int64_t n = F.n;
+  const int m = min(F.cnt[s], F.cap);
+  double L[kTri];
+  int rows = 0;
+  const int sh = fx_shift(A, s, m);
+  bool fits = sh >= 0;
+  if (fits) {
+    double mo[31];
+    fits = fx_moments<false, false, true>(A, s, m, mo, &rows, sh);
+    if (fits) gram_of_moments(mo, L);
+  }
+  bool ill = false;
+  const bool ok = fits && fx_chol9(L, 1e-9, &ill) && rows >= kNB;
+  A.kx[s] = ok && !ill ? sh : kFxSlow;
+  if (!fits) {
+    fx_push(A, s, 0);
+    return;
+  }
+  if (!ok || ill) {
+    // poorly conditioned stencils take the QR fit: rounding of the normal
+    // equations is amplified by 1 / pivot^2 there (2.5e-11 of the largest
+    // derivative for a stencil of nine entries), and the sweep lattice has 0.15 %
+    // of them. Those the normal equations refuse in every mode count as fallbacks.
+    const int slot = atomicAdd(F.fb_count, 1);
+    if (slot < F.fb_cap) F.fb_list[slot] = ok ? s | (int)kMirrorBit : s;
+    else atomicOr(&F.dg->flags, (unsigned)LP_FLAG_OVERFLOW);
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < kTri; ++k) A.fac[k * n + s] = L[k];
+}
+// the group's fields as records
+template <int NF>
+__global__ void k_fit_fx_fields(const FitArgs F, const StepArgs A, int f0) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= F.n) return;
+  FxRec& r = reinterpret_cast<FxRec*>(A.XU)[s];
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    const double w = F.fields[f0 + f][s];
+    fx_field(w, &r.m[f], &r.e[f]);
+    v[f] = fx_float(w);
+  }
+  A.fs[s] = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <int NF>
+__global__ void __launch_bounds__(kFxBlock, 3) k_fit_rhs_fx(const FitArgs F, const StepArgs A,
+                                                            int f0) {
+  const int s = fit_thread(F);
+  if (s >= F.n) return;
+  const int sh = A.kx[s];
+  if (sh == kFxSlow) return;  // queued for the plain rows or the QR fit
+  const int64_t n = F.n;
+  const int m = min(F.cnt[s], F.cap);
+  int sgn[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) sgn[f] = (int)F.msign[f0 + f];
+  double R[NF][kNB];
+  if (!fx_rhs<NF, false, false, true>(A, s, m, sgn, nullptr, R, sh)) {
+    A.kx[s] = kFxSlow;  // (all of its fields)
+    fx_push(A, s, 0);
+    return;
+  }
+  {
+    double L[kTri];
+#pragma unroll
+    for (int k = 0; k < kTri; ++k) L[k] = A.fac[k * n + s];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) fx_chol9_solve(L, R[f]);
+  }
+#pragma unroll
+  for (int f = 0; f < NF; ++f) write_coeffs(F, s, f0 + f, R[f]);
+}
+__global__ void __launch_bounds__(64) k_fit_slow(const FitArgs F, const StepArgs A) {
+  const int cnt = min(A.slow_count[0], F.n);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x)
+    fit_body<LP_FP64>(F, A.slow[t]);
+}
 
 // ---- lp_fit_derivatives in float-float (LP_MIXED_FF): positions relative
 // to the first particle in units of h (with the floor-mirror height) and the
@@ -330,7 +432,7 @@ __global__ void k_fit_split_ff(const FitArgs F) {
 }
 
 __global__ void __launch_bounds__(128, 4) k_fit_gram_ff(const FitArgs F) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = fit_thread(F);
   if (s >= F.n) return;
   const int n = F.n;
   const int m = min(F.cnt[s], F.cap);
@@ -368,9 +470,14 @@ __global__ void __launch_bounds__(128, 4) k_fit_gram_ff(const FitArgs F) {
   ff_gram_fo(mo, G);
 #pragma unroll
   for (int k = 0; k < kTri; ++k) G[k] = ff_norm(G[k]);
-  if (!(ff_chol9(G, 1e-4f) && rows >= kNB)) {
+  bool ill = false;
+  const bool ok = ff_chol9(G, 1e-4f, &ill) && rows >= kNB;
+  // poorly conditioned stencils take the QR fit, as in FP64, but at 2^-10 (about
+  // one in 100,000 of the sweep lattice; at 2^-7 the QR fits of 2.0 M particles
+  // cost 0.5 ms)
+  if (!ok || ill) {
     const int slot = atomicAdd(F.fb_count, 1);
-    if (slot < F.fb_cap) F.fb_list[slot] = s;
+    if (slot < F.fb_cap) F.fb_list[slot] = ok ? s | (int)kMirrorBit : s;
     else atomicOr(&F.dg->flags, (unsigned)LP_FLAG_OVERFLOW);
     F.lf[s] = make_float2(-1.f, 0.f);  // 1/L_00 > 0 for a factored stencil
     return;
@@ -388,7 +495,7 @@ __global__ void __launch_bounds__(128, 4) k_fit_gram_ff(const FitArgs F) {
 // solve runs on zero sums; 3 blocks of 168 registers, as at 128 the sums spill)
 template <int NG>
 __global__ void __launch_bounds__(128, 3) k_fit_rhs_ff(const FitArgs F, int f0) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = fit_thread(F);
   if (s >= F.n) return;
   if (!(F.lf[s].x > 0.f)) return;  // queued for the pivoted-QR fit
   const int n = F.n;
@@ -461,48 +568,153 @@ __global__ void __launch_bounds__(128, 3) k_fit_rhs_ff(const FitArgs F, int f0) 
   }
 }
 
+// Pivoted-QR fits of the queued particles, a warp for each: a lane holds rows
+// lane and lane + 32 of [A | B] in registers, and every column norm and
+// reflection is a warp sum. The same algorithm as qr_pivoted_solve (pivot: the
+// largest remaining norm, ties to the lower column; rank by 1e-8; basic
+// solution). One thread per particle with its matrix in local memory took 205 us
+// for the few hundred of the 2.0 M-particle sweep, a chain of dependent loads.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+template <int K>
+__device__ __forceinline__ bool qr_column(double (*a)[kNB], double (*b)[4], int* perm,
+                                          double* rdiag, int lane) {
+  // row index of a[h]: lane + 32 h; rows above K are done
+  const bool in = lane >= K;
+  int best = K;
+  double bestn = -1.0;
+#pragma unroll
+  for (int j = K; j < kNB; ++j) {
+    const double s = warp_sum((in ? a[0][j] * a[0][j] : 0.0) + a[1][j] * a[1][j]);
+    if (s > bestn) { bestn = s; best = j; }
+  }
+  const double alpha = sqrt(bestn);
+  if (alpha == 0.0 || !(bestn >= 0.0)) {  // (a NaN norm never wins: all columns are NaN)
+    rdiag[K] = bestn >= 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+    return false;
+  }
+#pragma unroll
+  for (int j = K + 1; j < kNB; ++j)
+    if (j == best) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) { const double t = a[h][K]; a[h][K] = a[h][j]; a[h][j] = t; }
+      const int t = perm[K]; perm[K] = perm[j]; perm[j] = t;
+    }
+  const double akk = __shfl_sync(0xffffffffu, a[0][K], K);
+  const double sgn = akk >= 0.0 ? 1.0 : -1.0;
+  const double v0 = lane == K ? akk + sgn * alpha : (in ? a[0][K] : 0.0), v1 = a[1][K];
+  const double f = 1.0 / (bestn + fabs(akk) * alpha);  // 2 / v.v
+#pragma unroll
+  for (int j = K + 1; j < kNB; ++j) {
+    const double t = f * warp_sum(v0 * a[0][j] + v1 * a[1][j]);
+    a[0][j] -= t * v0;
+    a[1][j] -= t * v1;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double t = f * warp_sum(v0 * b[0][q] + v1 * b[1][q]);
+    b[0][q] -= t * v0;
+    b[1][q] -= t * v1;
+  }
+  rdiag[K] = -sgn * alpha;
+  return true;
+}
 __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
   const int cnt = min(*F.fb_count, F.fb_cap);
-  double Am[LP_MAX_CAP * kNB], Bm[LP_MAX_CAP * 4], C[4 * kNB], Acopy[LP_MAX_CAP * kNB];
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x) {
-    const int s = F.fb_list[t];
+  const int lane = threadIdx.x & 31;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < cnt; t += nw) {
+    const int e = F.fb_list[t], s = e & ~kMirrorBit;
     const int n = F.n;
     const int m = min(F.cnt[s], F.cap);
     const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
-    // rows are packed: an entry whose index is out of range is dropped, as in
-    // the Cholesky path, and the rows after it move up
+    // rows are packed: an entry whose index is out of range is dropped and the
+    // rows after it move up; lanes past the last row hold zeros
+    __shared__ uint32_t packed[2][LP_MAX_CAP];
+    uint32_t* pk = packed[threadIdx.x >> 5];
+    pk[lane] = pk[lane + 32] = ~kMirrorBit;
+    __syncwarp();
     int rows = 0;
-    for (int k = 0; k < m; ++k) {
-      const uint32_t code = (uint32_t)F.nbr[(int64_t)k * n + s];
-      const int j = code & ~kMirrorBit;
-      if ((unsigned)j >= (unsigned)n) continue;  // stale or corrupt stencil entry
-      const double zj = (code >> 31) ? F.f2 - F.z[j] : F.z[j];
-      taylor_row((F.x[j] - xi) * F.inv_h, (F.y[j] - yi) * F.inv_h, (zj - zi) * F.inv_h,
-                 &Acopy[rows * kNB]);
-      ++rows;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = lane + 32 * h;
+      const uint32_t c = k < m ? (uint32_t)F.nbr[(int64_t)k * n + s] : ~kMirrorBit;
+      const bool in = (c & ~kMirrorBit) < (uint32_t)n;
+      const unsigned all = __ballot_sync(0xffffffffu, in);
+      if (in) pk[rows + __popc(all & ((1u << lane) - 1u))] = c;
+      rows += __popc(all);
+    }
+    __syncwarp();
+    uint32_t code[2];
+    double row[2][kNB];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      code[h] = pk[lane + 32 * h];
+      const int j = code[h] & ~kMirrorBit;
+#pragma unroll
+      for (int q = 0; q < kNB; ++q) row[h][q] = 0.0;
+      if ((unsigned)j < (unsigned)n) {
+        const double zj = (code[h] >> 31) ? F.f2 - F.z[j] : F.z[j];
+        taylor_row((F.x[j] - xi) * F.inv_h, (F.y[j] - yi) * F.inv_h, (zj - zi) * F.inv_h, row[h]);
+      }
     }
     for (int f0 = 0; f0 < F.nf; f0 += 4) {
       const int nf = min(4, F.nf - f0);
-      int r = 0;
-      for (int k = 0; k < m; ++k) {
-        const uint32_t code = (uint32_t)F.nbr[(int64_t)k * n + s];
-        const int j = code & ~kMirrorBit;
-        if ((unsigned)j >= (unsigned)n) continue;  // stale or corrupt stencil entry
-        const bool mir = code >> 31;
-        for (int q = 0; q < kNB; ++q) Am[r * kNB + q] = Acopy[r * kNB + q];
-        for (int f = 0; f < nf; ++f) {
-          double vj = F.fields[f0 + f][j];
-          if (mir) vj *= F.msign[f0 + f];
-          Bm[r * nf + f] = vj - F.fields[f0 + f][s];
+      double a[2][kNB], b[2][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int j = code[h] & ~kMirrorBit;
+#pragma unroll
+        for (int q = 0; q < kNB; ++q) a[h][q] = row[h][q];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          b[h][f] = 0.0;
+          if (f < nf && (unsigned)j < (unsigned)n) {
+            double vj = F.fields[f0 + f][j];
+            if (code[h] >> 31) vj *= F.msign[f0 + f];
+            b[h][f] = vj - F.fields[f0 + f][s];
+          }
         }
-        ++r;
       }
-      qr_pivoted_solve(rows, Am, nf, Bm, C);
-      for (int f = 0; f < nf; ++f) write_coeffs(F, s, f0 + f, C + f * kNB);
+      int perm[kNB];
+      double rd[kNB];
+#pragma unroll
+      for (int q = 0; q < kNB; ++q) { perm[q] = q; rd[q] = 0.0; }
+      qr_column<0>(a, b, perm, rd, lane) && qr_column<1>(a, b, perm, rd, lane) &&
+          qr_column<2>(a, b, perm, rd, lane) && qr_column<3>(a, b, perm, rd, lane) &&
+          qr_column<4>(a, b, perm, rd, lane) && qr_column<5>(a, b, perm, rd, lane) &&
+          qr_column<6>(a, b, perm, rd, lane) && qr_column<7>(a, b, perm, rd, lane) &&
+          qr_column<8>(a, b, perm, rd, lane);
+      int rank = 0;
+      bool run = true;
+#pragma unroll
+      for (int q = 0; q < kNB; ++q) {
+        run = run && !(fabs(rd[q]) <= 1e-8 * fabs(rd[0]));  // (NaN: full rank, NaN results)
+        rank += run;
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        double y[kNB], mine = 0.0;
+#pragma unroll
+        for (int k = kNB - 1; k >= 0; --k) {
+          double v = __shfl_sync(0xffffffffu, b[0][f], k);
+#pragma unroll
+          for (int j = k + 1; j < kNB; ++j)
+            v -= __shfl_sync(0xffffffffu, a[0][j], k) * y[j];
+          y[k] = k < rank ? v / rd[k] : 0.0;
+          if (perm[k] == lane) mine = y[k];
+        }
+        if (f < nf && lane < kNB)
+          F.coeffs[((int64_t)s * F.nf + f0 + f) * kNB + lane] =
+              mine * (lane < 3 ? F.inv_h : F.inv_h * F.inv_h);
+      }
     }
+    if (lane == 0 && e >= 0) atomicAdd(&F.dg->n_fallback, 1ull);
+    __syncwarp();  // (pk is reused)
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0)
-    atomicAdd(&F.dg->n_fallback, (unsigned long long)cnt);
 }
 
 // ---------------------------------------------------------- lp_mui_stress
@@ -562,12 +774,12 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
       if (A.K.free_surface) k_gram_fx<true, true><<<nf, b, 0, st>>>(A);
       else k_gram_fx<true, false><<<nf, b, 0, st>>>(A);
       k_pass1_fx<true><<<nf, b, 0, st>>>(A);
-      k_pass1_slow<true><<<152, 64, 0, st>>>(A);
+      k_pass1_slow<true><<<kSlowBlocks, 64, 0, st>>>(A);
     } else {
       if (A.K.free_surface) k_gram_fx<false, true><<<nf, b, 0, st>>>(A);
       else k_gram_fx<false, false><<<nf, b, 0, st>>>(A);
       k_pass1_fx<false><<<nf, b, 0, st>>>(A);
-      k_pass1_slow<false><<<152, 64, 0, st>>>(A);
+      k_pass1_slow<false><<<kSlowBlocks, 64, 0, st>>>(A);
     }
   } else if (prec == LP_MIXED) {
     if (per) k_pass1<LP_MIXED, true><<<nb, bs, 0, st>>>(A);
@@ -610,11 +822,11 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
     if (per) {
       if (A.K.free_surface) k_pass2_fx<true, true><<<nf, b, 0, st>>>(A);
       else k_pass2_fx<true, false><<<nf, b, 0, st>>>(A);
-      k_pass2_slow<true><<<152, 64, 0, st>>>(A);
+      k_pass2_slow<true><<<kSlowBlocks, 64, 0, st>>>(A);
     } else {
       if (A.K.free_surface) k_pass2_fx<false, true><<<nf, b, 0, st>>>(A);
       else k_pass2_fx<false, false><<<nf, b, 0, st>>>(A);
-      k_pass2_slow<false><<<152, 64, 0, st>>>(A);
+      k_pass2_slow<false><<<kSlowBlocks, 64, 0, st>>>(A);
     }
   } else if (prec == LP_MIXED) {
     if (per) k_pass2<LP_MIXED, true><<<nb, bs, 0, st>>>(A);
@@ -628,7 +840,30 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
 void launch_fit(int prec, const FitArgs& F, cudaStream_t st) {
   const int bs = spread_block(F.n, kBlock);
   const int nb = (F.n + bs - 1) / bs;
-  if (prec == LP_FP64) {
+  if (F.perm && (prec == LP_MIXED_FF || F.rows))
+    k_row_order<<<(F.n + kRowGroup - 1) / kRowGroup, kRowGroup, 0, st>>>(
+        F.n, F.cnt, const_cast<int32_t*>(F.perm));
+  if (prec == LP_FP64 && F.rows) {
+    const StepArgs& A = *F.rows;
+    const int sb = spread_block(F.n, 256), ns = (F.n + sb - 1) / sb;
+    k_fit_fx_split<<<ns, sb, 0, st>>>(F, A);
+    k_fit_gram_fx<<<nb, bs, 0, st>>>(F, A);
+    for (int f0 = 0; f0 < F.nf;) {
+      const int left = F.nf - f0, g = left == 4 ? 2 : (left < 3 ? left : 3);
+      if (g == 3) {
+        k_fit_fx_fields<3><<<ns, sb, 0, st>>>(F, A, f0);
+        k_fit_rhs_fx<3><<<nb, bs, 0, st>>>(F, A, f0);
+      } else if (g == 2) {
+        k_fit_fx_fields<2><<<ns, sb, 0, st>>>(F, A, f0);
+        k_fit_rhs_fx<2><<<nb, bs, 0, st>>>(F, A, f0);
+      } else {
+        k_fit_fx_fields<1><<<ns, sb, 0, st>>>(F, A, f0);
+        k_fit_rhs_fx<1><<<nb, bs, 0, st>>>(F, A, f0);
+      }
+      f0 += g;
+    }
+    k_fit_slow<<<kSlowBlocks, 64, 0, st>>>(F, A);
+  } else if (prec == LP_FP64) {
     k_fit<LP_FP64><<<nb, bs, 0, st>>>(F);
   } else if (prec == LP_MIXED) {
     k_fit<LP_MIXED><<<nb, bs, 0, st>>>(F);
@@ -637,7 +872,7 @@ void launch_fit(int prec, const FitArgs& F, cudaStream_t st) {
     k_fit_gram_ff<<<nb, bs, 0, st>>>(F);
     for (int f0 = 0; f0 < F.nf; f0 += 2) k_fit_rhs_ff<2><<<nb, bs, 0, st>>>(F, f0);
   }
-  k_fit_fallback<<<152, 64, 0, st>>>(F);
+  k_fit_fallback<<<2 * 152, 64, 0, st>>>(F);
 }
 void launch_mui_stress(int64_t n, const ColMui& m, const lp_eos& e, const double* V,
                        const double* gu, double* gdot, double* gnorm, double* P, double* eta,

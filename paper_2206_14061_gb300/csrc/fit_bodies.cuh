@@ -247,26 +247,28 @@ __device__ __forceinline__ void pass1_body(const StepArgs& A, int s) {
 // Pass 1 of LP_FP64 with the rows in fixed point (fixed_rows.cuh), in two
 // kernels: the moments and the FP64 factor, then the right-hand sides, solves
 // and derived values. 31 or 27 sums of three registers each are live, so one
-// kernel for both would not fit. A particle whose rows do not fit is queued
-// for pass1_body<LP_FP64>.
+// kernel for both would not fit. A particle whose rows do not fit, or whose
+// factor has a relative pivot below 2^-7, is queued for pass1_body<LP_FP64>
+// (which queues for the QR fit): there rounding is amplified ten-thousandfold,
+// and they keep the plain rows' results. None of a column's or cube's particles is
+// below it.
 template <bool PER, bool GH>
 __device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
   const int64_t n = A.n;
   const int m = min(A.cnt[s], A.cap);
   double L[kTri];
+  bool fits;
   {
     double mo[31];
-    const bool fits = fx_moments<PER, GH>(A, s, m, mo);
-    A.kx[s] = fits ? 0 : 1;
-    if (!fits) {
-      fx_push(A, s, 0);
-      return;
-    }
-    gram_of_moments(mo, L);
+    int rows;
+    fits = fx_moments<PER, GH>(A, s, m, mo, &rows);
+    if (fits) gram_of_moments(mo, L);
   }
-  const bool ok = fx_chol9(L, 1e-9) && m >= kNB;
-  if (!ok) {
-    push_fallback(A, s);
+  bool ill;
+  fits = fits && fx_chol9(L, 1e-9, &ill) && m >= kNB && !ill;
+  A.kx[s] = fits ? 0 : 1;
+  if (!fits) {
+    fx_push(A, s, 0);
     return;
   }
   A.fbslot[s] = -1;
@@ -583,7 +585,8 @@ __device__ __forceinline__ void ff_gram_fo(const ff* mo, ff* g) {
 // Same pivot test as chol9: the Schur complement of column j must stay above
 // rel_tol times the original diagonal entry, else the stencil is too
 // ill-conditioned for the normal equations.
-__device__ __forceinline__ bool ff_chol9(ff* a, float rel_tol) {
+// ill (optional): a relative pivot below 2^-10.
+__device__ __forceinline__ bool ff_chol9(ff* a, float rel_tol, bool* ill = nullptr) {
   bool ok = true;
 #pragma unroll
   for (int j = 0; j < kNB; ++j) {
@@ -594,6 +597,7 @@ __device__ __forceinline__ bool ff_chol9(ff* a, float rel_tol) {
     d = ff_norm(d);
     const bool good = d.h > rel_tol * d0;
     ok = ok && good;
+    if (ill && !(d.h > 0x1p-10f * d0)) *ill = true;
     const ff inv = good ? ff_rsqrt(d) : ff{0.f, 0.f};
     a[tri(j, j)] = inv;
 #pragma unroll

@@ -9,14 +9,15 @@
 // factor and solves stay FP64.
 //
 // A factor v is held as h + l, h a 28-bit integer and l the rest of it in
-// units of h, |l| <= 1/2, as a float. A sum of products a b is
-//   H += a.h b.h            exact, one 32 x 32 + 64-bit multiply-add
-//   M += a.h b.l + a.l b.h  two FP32 multiply-adds (a.l b.l is below 2^-56),
-//                           moved into H every four rows
-// so a sum errs by about 2^-51 of its largest possible term, less than an FP64
-// sum over the same rows, which rounds at 2^-53 of the running sum (36 rows) in
-// each row; 64 rows of 2^56 cannot overflow H. 7.0 cycles per accumulation and
-// scheduler, measured; an FP64 multiply-add takes about 75.
+// units of h, |l| <= 1/2, as a float. A product a b enters its sum as
+//   a.h b.h                       exact, one 32 x 32 + 64-bit multiply-add
+//   round(a.h b.l + a.l b.h)      FP32, to an integer (a.l b.l is below 1/4)
+// so a term errs by about 2^-54 of the largest possible one, less than an FP64
+// sum, which rounds at 2^-53 of the running sum in every row. The sums are
+// exact, so their order does not matter, and 64 rows of 2^56 cannot overflow
+// them. (Keeping the second part as a float sum, moved into the integer one
+// every fourth row, is as fast and errs by 2^-50.) About 8 cycles per
+// accumulation and scheduler; an FP64 multiply-add takes about 75.
 //
 // Positions are integers X = x 2^k modulo 2^64, with r 2^k in (2^59, 2^60]
 // for the stencil radius r: the conversion is exact for all but the last bits
@@ -104,25 +105,18 @@ __device__ __forceinline__ FxV fx_quad(long long Q, int sq, float qs) {
   v.l = __fmul_rn((float)(int)((unsigned)Q - ((unsigned)v.h << sq)), qs);
   return v;
 }
-__device__ __forceinline__ void fx_acc(long long& H, float& M, const FxV& a, const FxV& b) {
-  H = fx_mad(a.h, b.h, H);
-  M = __fmaf_rn(a.hf, b.l, M);
-  M = __fmaf_rn(a.l, b.hf, M);
+__device__ __forceinline__ void fx_acc(long long& H, const FxV& a, const FxV& b) {
+  const int c = __float2int_rn(__fmaf_rn(a.l, b.hf, __fmul_rn(a.hf, b.l)));
+  H = fx_mad(a.h, b.h, H) + (long long)c;
 }
-// M, rounded to an integer, moves into H: every fourth row (and after a row
-// that counts twice), so that |M| < 2^31 and its rounding stays small
-__device__ __forceinline__ void fx_flush(long long& H, float& M) {
-  H = fx_mad(__float2int_rn(M), 1, H);
-  M = 0.f;
-}
-__device__ __forceinline__ bool fx_flush_at(int k) { return (k & 3) == 3; }
 __device__ __forceinline__ double pow2_of(int e) {  // 2^e, a normal double
   return __longlong_as_double((long long)(1023 + e) << 52);
 }
 
 // offsets of entry j of a particle at `me` (PER: nearest images)
-template <bool PER>
-__device__ __forceinline__ void fx_offsets(const StepConsts& K, const FxRec& me,
+// (SH: shifted up by sh)
+template <bool PER, bool SH>
+__device__ __forceinline__ void fx_offsets(const StepConsts& K, int sh, const FxRec& me,
                                            unsigned long long Xj, unsigned long long Yj,
                                            unsigned long long Zj, float xf, float yf, bool mir,
                                            unsigned long long* D) {
@@ -134,15 +128,18 @@ __device__ __forceinline__ void fx_offsets(const StepConsts& K, const FxRec& me,
     if (fabsf(dx) > K.fx_hLx) D[0] -= dx > 0.f ? K.fx_Lx : 0ull - K.fx_Lx;
     if (fabsf(dy) > K.fx_hLy) D[1] -= dy > 0.f ? K.fx_Ly : 0ull - K.fx_Ly;
   }
+  if (SH) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) D[a] <<= sh;
+  }
 }
 
 // row loop state: the neighbour's position one row ahead, its code two rows ahead
 struct FxPosLoad {
   ulonglong2 xy;
   ulonglong2 zf;  // Z and the two floats
-  __device__ __forceinline__ void fetch(const FxRec* R, uint32_t code, int n, int s) {
-    int j = code & kIndexMask;
-    if ((unsigned)j >= (unsigned)n) j = s;  // never read outside the arrays (row skipped)
+  __device__ __forceinline__ void fetch(const FxRec* R, uint32_t j, int n, int s) {
+    if (j >= (uint32_t)n) j = (uint32_t)s;  // never read outside the arrays (row skipped)
     const ulonglong2* p = reinterpret_cast<const ulonglong2*>(R + j);
     xy = p[0];
     zf = p[1];
@@ -172,16 +169,18 @@ __device__ __forceinline__ float fx_float(double v) {
   return (fabsf(f) < 0x1p-100f && (b << 1)) ? copysignf(0x1p-100f, (b >> 63) ? -1.f : 1.f) : f;
 }
 
-// records of pass 1: positions, u, v, w
-__device__ __forceinline__ void fx_split_state_body(const StepArgs& A, int s) {
-  FxRec* R = reinterpret_cast<FxRec*>(A.XU);
-  const double x = A.x[s], y = A.y[s], z = A.z[s];
-  const int k = A.K.fx_k;
-  FxRec r;
+// the position half of a record
+__device__ __forceinline__ void fx_position(double x, double y, double z, int k, FxRec& r) {
   r.X = fx_of(x, k); r.Y = fx_of(y, k); r.Z = fx_of(z, k);
   const bool fin = isfinite(x) && isfinite(y) && isfinite(z);
   r.xf = fin ? __double2float_rn(x) : __int_as_float(0x7fffffff);
   r.yf = __double2float_rn(y);
+}
+// records of pass 1: positions, u, v, w
+__device__ __forceinline__ void fx_split_state_body(const StepArgs& A, int s) {
+  FxRec* R = reinterpret_cast<FxRec*>(A.XU);
+  FxRec r;
+  fx_position(A.x[s], A.y[s], A.z[s], A.K.fx_k, r);
   const double u = A.u[s], v = A.v[s], w = A.w[s];
   fx_field(u, &r.m[0], &r.e[0]);
   fx_field(v, &r.m[1], &r.e[1]);
@@ -205,39 +204,86 @@ __device__ __forceinline__ void fx_split_p1_body(const StepArgs& A, int s) {
   A.fs[s] = make_float4(fx_float(g), fx_float(v), 0.f, 0.f);
 }
 
+// Stencils whose radius is not known (lp_fit_derivatives): the shift that
+// brings a particle's largest offset into (fx_lim / 2, fx_lim], from a walk over
+// the positions; -1 if the offsets are too large, or so small that the shift
+// would reach below the positions' resolution.
+__device__ __forceinline__ int fx_shift(const StepArgs& A, int s, int m) {
+  const int n = A.n;
+  const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
+  FxRec me;
+  fx_rec_pos(me, R, s);
+  unsigned big = 0;
+  constexpr int kChunk = 4;
+  for (int k0 = 0; k0 < m; k0 += kChunk) {
+    uint32_t cd[kChunk];
+    FxPosLoad p[kChunk];
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t)
+      cd[t] = k0 + t < m ? (uint32_t)A.nbr[(int64_t)(k0 + t) * n + s] : ~kMirrorBit;
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t) p[t].fetch(R, cd[t] & A.K.fx_mask, n, s);
+#pragma unroll
+    for (int t = 0; t < kChunk; ++t) {
+      if ((cd[t] & A.K.fx_mask) >= (uint32_t)n) continue;
+      unsigned long long D[3];
+      fx_offsets<false, false>(A.K, 0, me, p[t].xy.x, p[t].xy.y, p[t].zf.x, 0.f, 0.f,
+                               cd[t] >> 31, D);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int h = (int)(D[a] >> 32);
+        big = max(big, (unsigned)(h ^ (h >> 31)));
+      }
+    }
+  }
+  // (+ 1: the integer parts are rounded)
+  const unsigned lim = (unsigned)A.K.fx_lim;
+  if (big + 1u > lim) return -1;
+  int sh = max(__clz((int)(big + 1u)) - __clz((int)lim), 0);
+  if (((big + 1u) << sh) > lim) --sh;
+  return sh <= 12 ? sh : -1;
+}
+
 // The 31 moments of a stencil (order of ff_moments_add) in units of the
 // lattice spacing. GH: flagged entries (kGhostBit) also stand for their point
 // reflection, so they add their even moments twice and no odd ones. False: the
 // row does not fit the fixed-point range.
-template <bool PER, bool GH>
-__device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo) {
+// rows: the entries with an index in range. SH: offsets are shifted up by sh,
+// which fx_shift chose for the particle's largest one.
+template <bool PER, bool GH, bool SH = false>
+__device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo,
+                                           int* rows, int sh = 0) {
   const int n = A.n;
   const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
   const StepConsts& K = A.K;
+  const uint32_t mask = K.fx_mask;
   FxRec me;
   fx_rec_pos(me, R, s);
   long long H[31];
-  float M[31];  // (degree 2 needs no M)
 #pragma unroll
-  for (int q = 0; q < 31; ++q) { H[q] = 0; M[q] = 0.f; }
-  unsigned big = 0;  // OR of the offsets' magnitudes
+  for (int q = 0; q < 31; ++q) H[q] = 0;
+  unsigned big = 0;  // the largest magnitude of an offset
+  int in_range = m;
   bool bad = !(me.xf == me.xf);
   uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
   uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
   FxPosLoad P;
-  P.fetch(R, code, n, s);
+  P.fetch(R, code & mask, n, s);
   for (int k = 0; k < m; ++k) {
     const uint32_t c0 = code;
-    const bool live = (c0 & kIndexMask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
+    const bool live = (c0 & mask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
     unsigned long long D[3];
-    fx_offsets<PER>(K, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), c0 >> 31, D);
+    fx_offsets<PER, SH>(K, sh, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), c0 >> 31, D);
     bad = bad || (live && !(P.xf() == P.xf()));
     if (k + 1 < m) {  // (the position is taken: its registers hold the next one)
       code = nxt;
-      P.fetch(R, code, n, s);
+      P.fetch(R, code & mask, n, s);
       if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
     }
-    if (!live) continue;
+    if (!live) {
+      --in_range;
+      continue;
+    }
     FxV d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -265,29 +311,31 @@ __device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, doub
       for (int a = 0; a < 3; ++a) d[a] = FxV{0, 0.f, 0.f};
     }
     // q: 0 xx, 1 yy, 2 zz, 3 xy, 4 xz, 5 yz
-    fx_acc(H[6], M[6], d[0], q[0]);   fx_acc(H[7], M[7], d[1], q[1]);
-    fx_acc(H[8], M[8], d[2], q[2]);   fx_acc(H[9], M[9], d[1], q[0]);
-    fx_acc(H[10], M[10], d[2], q[0]); fx_acc(H[11], M[11], d[0], q[1]);
-    fx_acc(H[12], M[12], d[2], q[1]); fx_acc(H[13], M[13], d[0], q[2]);
-    fx_acc(H[14], M[14], d[1], q[2]); fx_acc(H[15], M[15], d[2], q[3]);
-    fx_acc(H[16], M[16], w[0], q[0]); fx_acc(H[17], M[17], w[1], q[1]);
-    fx_acc(H[18], M[18], w[2], q[2]); fx_acc(H[19], M[19], w[0], q[3]);
-    fx_acc(H[20], M[20], w[0], q[4]); fx_acc(H[21], M[21], w[1], q[3]);
-    fx_acc(H[22], M[22], w[1], q[5]); fx_acc(H[23], M[23], w[2], q[4]);
-    fx_acc(H[24], M[24], w[2], q[5]); fx_acc(H[25], M[25], w[0], q[1]);
-    fx_acc(H[26], M[26], w[0], q[2]); fx_acc(H[27], M[27], w[1], q[2]);
-    fx_acc(H[28], M[28], w[0], q[5]); fx_acc(H[29], M[29], w[1], q[4]);
-    fx_acc(H[30], M[30], w[2], q[3]);
-    if (fx_flush_at(k) || twin) {
-#pragma unroll
-      for (int t = 6; t < 31; ++t) fx_flush(H[t], M[t]);
-    }
+    fx_acc(H[6], d[0], q[0]);   fx_acc(H[7], d[1], q[1]);
+    fx_acc(H[8], d[2], q[2]);   fx_acc(H[9], d[1], q[0]);
+    fx_acc(H[10], d[2], q[0]); fx_acc(H[11], d[0], q[1]);
+    fx_acc(H[12], d[2], q[1]); fx_acc(H[13], d[0], q[2]);
+    fx_acc(H[14], d[1], q[2]); fx_acc(H[15], d[2], q[3]);
+    fx_acc(H[16], w[0], q[0]); fx_acc(H[17], w[1], q[1]);
+    fx_acc(H[18], w[2], q[2]); fx_acc(H[19], w[0], q[3]);
+    fx_acc(H[20], w[0], q[4]); fx_acc(H[21], w[1], q[3]);
+    fx_acc(H[22], w[1], q[5]); fx_acc(H[23], w[2], q[4]);
+    fx_acc(H[24], w[2], q[5]); fx_acc(H[25], w[0], q[1]);
+    fx_acc(H[26], w[0], q[2]); fx_acc(H[27], w[1], q[2]);
+    fx_acc(H[28], w[0], q[5]); fx_acc(H[29], w[1], q[4]);
+    fx_acc(H[30], w[2], q[3]);
   }
+  *rows = in_range;
   if (bad || big > (unsigned)K.fx_lim) return false;
+  double g2 = K.fx_g2, g3 = K.fx_g3, g4 = K.fx_g4;
+  if (SH) {
+    g2 *= pow2_of(-2 * sh);
+    g3 *= pow2_of(-3 * sh);
+    g4 *= pow2_of(-4 * sh);
+  }
 #pragma unroll
   for (int t = 0; t < 31; ++t) {
-    const double g = t < 6 ? K.fx_g2 : (t < 16 ? K.fx_g3 : K.fx_g4);
-    if (t >= 6) fx_flush(H[t], M[t]);
+    const double g = t < 6 ? g2 : (t < 16 ? g3 : g4);
     mo[t] = (double)H[t] * g;
   }
   return true;
@@ -308,12 +356,13 @@ __device__ __forceinline__ void gram_of_moments(const double* mo, double* L) {
 // spacing; sgn: the factor (-1, 0, 1) of a field at a floor mirror; GH: bG is
 // the right-hand side of a flagged entry's ghost row. False: a field does not
 // fit (the caller queues the particle).
-template <int NF, bool PER, bool GH>
+template <int NF, bool PER, bool GH, bool SH = false>
 __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const int* sgn,
-                                       const double* bG, double (*R9)[kNB]) {
+                                       const double* bG, double (*R9)[kNB], int sh = 0) {
   const int n = A.n;
   const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
   const StepConsts& K = A.K;
+  const uint32_t mask = K.fx_mask;
   // the scale of each field: its largest difference in this stencil, in FP32
   unsigned mx[NF];
   float mf[NF];
@@ -333,15 +382,15 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     float4 v[kChunk];
 #pragma unroll
     for (int t = 0; t < kChunk; ++t)
-      cd[t] = k0 + t < m ? (uint32_t)A.nbr[(int64_t)(k0 + t) * n + s] : kIndexMask;
+      cd[t] = k0 + t < m ? (uint32_t)A.nbr[(int64_t)(k0 + t) * n + s] : ~kMirrorBit;
 #pragma unroll
     for (int t = 0; t < kChunk; ++t) {
-      const uint32_t j = cd[t] & kIndexMask;
+      const uint32_t j = cd[t] & mask;
       v[t] = A.fs[j < (uint32_t)n ? j : (uint32_t)s];
     }
 #pragma unroll
     for (int t = 0; t < kChunk; ++t) {
-      if ((cd[t] & kIndexMask) >= (uint32_t)n) continue;
+      if ((cd[t] & mask) >= (uint32_t)n) continue;
       const float vv[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
       const bool mir = cd[t] >> 31;
 #pragma unroll
@@ -377,18 +426,17 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     G[f] = GH ? fx_of(bG[f], kb[f]) : 0ull;
   }
   long long H[NF][kNB];
-  float M[NF][kNB];
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
-    for (int q = 0; q < kNB; ++q) { H[f][q] = 0; M[f][q] = 0.f; }
+    for (int q = 0; q < kNB; ++q) H[f][q] = 0;
   uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
   uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
   FxPosLoad P;
   longlong2 f01, f23;  // m[0], m[1]; m[2], exponents
   auto fetch = [&](uint32_t c) {
-    P.fetch(R, c, n, s);
-    const uint32_t j = c & kIndexMask;
+    const uint32_t j = c & mask;
+    P.fetch(R, j, n, s);
     const longlong2* r = reinterpret_cast<const longlong2*>(&R[j < (uint32_t)n ? j : (uint32_t)s].m[0]);
     f01 = r[0];
     f23 = r[1];
@@ -396,10 +444,10 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
   fetch(code);
   for (int k = 0; k < m; ++k) {
     const uint32_t c0 = code;
-    const bool live = (c0 & kIndexMask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
+    const bool live = (c0 & mask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
     const bool mir = c0 >> 31;
     unsigned long long D[3], u[NF];
-    fx_offsets<PER>(K, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), mir, D);
+    fx_offsets<PER, SH>(K, sh, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), mir, D);
     {
       const long long mj[3] = {f01.x, f01.y, f23.x};
       const int ej[3] = {(int)(short)f23.y, (int)f23.y >> 16, (int)(short)(f23.y >> 32)};
@@ -434,25 +482,22 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       // row, linear terms take b - bG and quadratic ones b + bG
       const FxV bl = fx_split(twin ? d - G[f] : d);
 #pragma unroll
-      for (int q = 0; q < 3; ++q) fx_acc(H[f][q], M[f][q], bl, a[q]);
+      for (int q = 0; q < 3; ++q) fx_acc(H[f][q], bl, a[q]);
       const FxV bq = GH ? fx_split(twin ? d + G[f] : d) : bl;
 #pragma unroll
-      for (int q = 3; q < kNB; ++q) fx_acc(H[f][q], M[f][q], bq, a[q]);
-    }
-    if (fx_flush_at(k)) {
-#pragma unroll
-      for (int f = 0; f < NF; ++f)
-#pragma unroll
-        for (int q = 0; q < kNB; ++q) fx_flush(H[f][q], M[f][q]);
+      for (int q = 3; q < kNB; ++q) fx_acc(H[f][q], bq, a[q]);
     }
   }
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const double ub = pow2_of(32 - kb[f]);
-    const double ul = ub * K.fx_lin, uq = ub * K.fx_quad;
+    double ul = ub * K.fx_lin, uq = ub * K.fx_quad;
+    if (SH) {
+      ul *= pow2_of(-sh);
+      uq *= pow2_of(-2 * sh);
+    }
 #pragma unroll
     for (int q = 0; q < kNB; ++q) {
-      fx_flush(H[f][q], M[f][q]);
       R9[f][q] = (double)H[f][q] * (q < 3 ? ul : (q < 6 ? 0.5 * uq : uq));
     }
   }

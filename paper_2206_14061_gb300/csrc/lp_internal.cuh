@@ -94,6 +94,7 @@ struct StepConsts {
   // and 1, 2 (right-hand sides) to units of h; the mirror plane and the
   // periods in fixed point; half periods (infinite without)
   int fx_k, fx_sq, fx_lim;
+  uint32_t fx_mask;  // index bits of a stencil code (the ghost flag is not one in a step)
   float fx_qs, fx_hLx, fx_hLy;
   double fx_g2, fx_g3, fx_g4, fx_lin, fx_quad;
   unsigned long long fx_F2, fx_Lx, fx_Ly;
@@ -301,6 +302,7 @@ struct StepArgs {
   int32_t* slow;        // FP64: particles queued for the plain FP64 rows (pass 1, then pass 2)
   int* slow_count;      // their numbers in pass 1 and pass 2
   uint8_t* kx;          // FP64: 1 where the offsets do not fit the fixed-point rows
+                        // (lp_fit_derivatives: the particle's shift, kFxSlow there)
   float2* R1;   // LP_MIXED_FF: pass 1's right-hand sides (27 float-float, k-major)
   float2* P1s;  // LP_MIXED_FF: gdot (6) and ld (3) of pass 1 as float-float, k-major
                 // (null in the other modes)
@@ -341,6 +343,10 @@ struct FitArgs {
   int32_t* fb_count;
   int fb_cap;
   DevDiag* dg;
+  const int32_t* perm;  // particle of each thread (rows sorted within groups of 128), or NULL
+  // LP_FP64 with fixed-point rows (a context's workspace): the rows' arguments;
+  // NULL: plain FP64 rows
+  const StepArgs* rows;
 };
 
 // arguments of the persistent step kernel (persistent.cu)
@@ -505,13 +511,16 @@ __device__ __forceinline__ double inv_sqrt(double v) {
   const double e = __fma_rn(-__dmul_rn(v, y), y, 1.0);
   return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
 }
+constexpr int kFxIllBits = 7;
 template <int J>
-__device__ __forceinline__ bool fx_chol9_column(double* a, double rel_tol) {
+__device__ __forceinline__ bool fx_chol9_column(double* a, double rel_tol, bool* ill) {
   double d = a[tri(J, J)];
   const double d0 = d;
 #pragma unroll
   for (int k = 0; k < J; ++k) d = __fma_rn(-a[tri(J, k)], a[tri(J, k)], d);
   const bool good = d > rel_tol * d0;
+  // (compared as high words: the exponents and 20 bits)
+  *ill = *ill || __double2hiint(d) + (kFxIllBits << 20) <= __double2hiint(d0);
   const double inv = good ? inv_sqrt(d) : 0.0;
   a[tri(J, J)] = inv;
 #pragma unroll
@@ -523,16 +532,18 @@ __device__ __forceinline__ bool fx_chol9_column(double* a, double rel_tol) {
   }
   return good;
 }
-__device__ __forceinline__ bool fx_chol9(double* a, double rel_tol) {
-  bool ok = fx_chol9_column<0>(a, rel_tol);
-  ok = fx_chol9_column<1>(a, rel_tol) && ok;
-  ok = fx_chol9_column<2>(a, rel_tol) && ok;
-  ok = fx_chol9_column<3>(a, rel_tol) && ok;
-  ok = fx_chol9_column<4>(a, rel_tol) && ok;
-  ok = fx_chol9_column<5>(a, rel_tol) && ok;
-  ok = fx_chol9_column<6>(a, rel_tol) && ok;
-  ok = fx_chol9_column<7>(a, rel_tol) && ok;
-  ok = fx_chol9_column<8>(a, rel_tol) && ok;
+// (ill: a relative pivot below 2^-kFxIllBits)
+__device__ __forceinline__ bool fx_chol9(double* a, double rel_tol, bool* ill) {
+  *ill = false;
+  bool ok = fx_chol9_column<0>(a, rel_tol, ill);
+  ok = fx_chol9_column<1>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<2>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<3>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<4>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<5>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<6>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<7>(a, rel_tol, ill) && ok;
+  ok = fx_chol9_column<8>(a, rel_tol, ill) && ok;
   return ok;
 }
 __device__ __forceinline__ void fx_chol9_solve(const double* L, double* b) {
