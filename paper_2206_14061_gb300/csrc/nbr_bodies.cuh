@@ -727,15 +727,13 @@ __device__ __forceinline__ void ghost_scan_body(int s, bool live, int n,
   }
 }
 
-// glist (optional): every particle with ghosts is appended, in no set order,
-// at glist[(*gcount)++], so that the twin kernels need visit only those.
+// Flags the entries of particle s whose reflections are ghosts, one thread per
+// particle (the persistent launch; ghost_group below gives the same flags).
 __device__ __forceinline__ void ghost_body(int s, bool live, int n, const double* __restrict__ z,
                                            const int4* __restrict__ X,
                                            int32_t* __restrict__ nbr, const int32_t* __restrict__ cnt,
                                            int32_t* __restrict__ gcnt, const StepConsts& K,
-                                           DevDiag* __restrict__ dg,
-                                           int32_t* __restrict__ glist = nullptr,
-                                           int* __restrict__ gcount = nullptr) {
+                                           DevDiag* __restrict__ dg) {
   int twins = 0;
   bool over = false;
   if (live) {
@@ -785,21 +783,142 @@ __device__ __forceinline__ void ghost_body(int s, bool live, int n, const double
     }
     gcnt[s] = twins;
   }
-  if (glist) {  // one atomic per warp for the warp's particles with ghosts
-    const unsigned has = __ballot_sync(0xffffffffu, live && twins > 0);
-    if (has) {
-      const int lane = threadIdx.x & 31;
-      int base = 0;
-      if (lane == 0) base = atomicAdd(gcount, __popc(has));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (live && twins > 0) glist[base + __popc(has & ((1u << lane) - 1u))] = s;
-    }
-  }
   unsigned long long a = (unsigned long long)twins;
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   if ((threadIdx.x & 31) == 0 && a) atomicAdd(&dg->n_ghosts, a);
   warp_count(&dg->n_overflow, live && over);
   if (live && over) atomicOr(&dg->flags, (unsigned)LP_FLAG_OVERFLOW);
+}
+
+// The same for a list of one-sided particles, kGhostLanes lanes to a particle.
+// One thread per particle holds its offsets in local memory (6 bytes an entry):
+// 512 threads of an SM need 196 KB of it, more than the L1 keeps, and the
+// check of a reflection against the entries loads it over and over. Four lanes
+// share one copy in shared memory (8 bytes an entry, 24 KB a block with the
+// codes), each gathers and tests a quarter of the entries.
+// slot: the particle's column of the shared arrays; sub: the lane within the
+// particle. Every lane of the warp must call it (live or not). A particle with
+// ghosts is appended, in no set order, at glist[(*gcount)++].
+constexpr int kGhostLanes = 4;
+constexpr int kGhostBlock = 128;
+constexpr int kGhostSlots = kGhostBlock / kGhostLanes;
+struct GhostShared {
+  int2 o[LP_MAX_CAP][kGhostSlots];  // offsets: x and y (16 bits each), z
+  int32_t code[LP_MAX_CAP][kGhostSlots];
+};
+__device__ __forceinline__ void ghost_group(int s, bool live, int slot, int sub, GhostShared& sh,
+                                            int n, const double* __restrict__ z,
+                                            const int4* __restrict__ X,
+                                            int32_t* __restrict__ nbr,
+                                            const int32_t* __restrict__ cnt,
+                                            int32_t* __restrict__ gcnt, const StepConsts& K,
+                                            DevDiag* __restrict__ dg,
+                                            int32_t* __restrict__ glist,
+                                            int* __restrict__ gcount) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int m = live ? min(cnt[s], K.cap) : 0;
+  const int R2 = (int)K.ghost_R2;
+  const int PX = (int)K.ghost_PX, PY = (int)K.ghost_PY;
+  const int4 xi = live ? X[s] : make_int4(0, 0, 0, 0);
+  long long S0 = 0, S1 = 0, S2 = 0, W = 0;
+  int ok = m > 0;
+  for (int k = sub; k < m; k += kGhostLanes) {
+    const uint32_t code = (uint32_t)nbr[(int64_t)k * n + s];
+    if ((code & kIndexMask) >= (uint32_t)n || (code & kGhostBit)) { ok = 0; break; }
+    const int4 xj = X[code & kIndexMask];
+    const int o0 = wrap_fix(xj.x - xi.x, PX), o1 = wrap_fix(xj.y - xi.y, PY);
+    const int o2 = ((code & kMirrorBit) ? xj.w : xj.z) - xi.z;
+    sh.o[k][slot] = make_int2((o0 & 0xffff) | (o1 << 16), (int)(short)o2);
+    sh.code[k][slot] = (int32_t)code;
+    const int q = (o0 * o0 + o1 * o1) + o2 * o2;
+    const int w = q < R2 ? R2 - q : 0;
+    S0 += (long long)w * o0;
+    S1 += (long long)w * o1;
+    S2 += (long long)w * o2;
+    W += w;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int d = 1; d < kGhostLanes; d <<= 1) {  // (whole numbers: any order gives the same sums)
+    S0 += __shfl_xor_sync(kAll, S0, d);
+    S1 += __shfl_xor_sync(kAll, S1, d);
+    S2 += __shfl_xor_sync(kAll, S2, d);
+    W += __shfl_xor_sync(kAll, W, d);
+    ok &= __shfl_xor_sync(kAll, ok, d);
+  }
+  double s2;
+  const bool side = ghost_one_sided(S0, S1, S2, W, K, &s2);
+  unsigned long long cand = 0ull;  // entries whose reflection is on the open side
+  if (ok && side) {
+    const double dep = __dmul_rn(0.5, K.ghost_hk);
+    const double dep2s2 = __dmul_rn(__dmul_rn(dep, dep), s2);
+    const double zi = z[s];
+    const double f2 = __dmul_rn(2.0, K.floor_z);
+    for (int k = sub; k < m; k += kGhostLanes) {
+      const int2 o = sh.o[k][slot];
+      const int o0 = (int)(short)o.x, o1 = o.x >> 16, o2 = o.y;
+      const double ds = (double)(((long long)o0 * S0 + (long long)o1 * S1) + (long long)o2 * S2);
+      if (!(ds > 0.0 && __dmul_rn(ds, ds) >= dep2s2)) continue;
+      if (K.mirror_mode != LP_MIRROR_NONE) {
+        const uint32_t code = (uint32_t)sh.code[k][slot];
+        const int j = code & kIndexMask;
+        const double zk = (code & kMirrorBit) ? __dsub_rn(f2, z[j]) : z[j];
+        if (__dsub_rn(__dadd_rn(zi, zi), zk) < K.floor_z) continue;
+      }
+      cand |= 1ull << k;
+    }
+  }
+#pragma unroll
+  for (int d = 1; d < kGhostLanes; d <<= 1) cand |= __shfl_xor_sync(kAll, cand, d);
+  // a candidate at a time, the particle's lanes each against a quarter of the
+  // entries: a ghost if none lies within h/2 of the reflection
+  const int clear2 = (int)K.ghost_clear2;
+  const unsigned group = ((1u << kGhostLanes) - 1u) << (lane & ~(kGhostLanes - 1));
+  unsigned long long tw = 0ull;
+  while (__any_sync(kAll, cand != 0ull)) {
+    const int k = cand ? __ffsll((long long)cand) - 1 : 0;
+    int hits = 0;
+    if (cand) {
+      const int2 c = sh.o[k][slot];
+      const int c0 = (int)(short)c.x, c1 = c.x >> 16, c2 = c.y;
+#pragma unroll 4
+      for (int l = sub; l < m; l += kGhostLanes) {
+        const int2 o = sh.o[l][slot];
+        const int e0 = (int)(short)o.x + c0, e1 = (o.x >> 16) + c1, e2 = o.y + c2;
+        hits += (e0 * e0 + e1 * e1) + e2 * e2 < clear2;
+      }
+    }
+    const bool hit = __ballot_sync(kAll, hits != 0) & group;
+    if (cand && !hit) tw |= 1ull << k;
+    cand &= cand - 1ull;
+  }
+  const int twins = __popcll(tw);
+  // entries without a ghost first (in their order), then the flagged ones
+  if (twins) {
+    for (int k = sub; k < m; k += kGhostLanes) {
+      const unsigned long long below = tw & ((1ull << k) - 1ull);
+      const bool f = (tw >> k) & 1ull;
+      const int w = f ? m - twins + __popcll(below) : k - __popcll(below);
+      const uint32_t code = (uint32_t)sh.code[k][slot];
+      nbr[(int64_t)w * n + s] = (int32_t)(f ? code | kGhostBit : code);
+    }
+  }
+  __syncwarp();  // (the next particle overwrites the shared columns)
+  const bool lead = live && sub == 0;
+  if (lead) gcnt[s] = twins;
+  const unsigned has = __ballot_sync(kAll, lead && twins > 0);
+  if (has) {  // one atomic per warp for the warp's particles with ghosts
+    int base = 0;
+    if (lane == 0) base = atomicAdd(gcount, __popc(has));
+    base = __shfl_sync(kAll, base, 0);
+    if (lead && twins > 0) glist[base + __popc(has & ((1u << lane) - 1u))] = s;
+  }
+  const bool over = lead && twins > 0 && m + twins > K.cap;
+  const unsigned a = __reduce_add_sync(kAll, lead ? (unsigned)twins : 0u);
+  if (lane == 0 && a) atomicAdd(&dg->n_ghosts, (unsigned long long)a);
+  warp_count(&dg->n_overflow, over);
+  if (over) atomicOr(&dg->flags, (unsigned)LP_FLAG_OVERFLOW);
 }
 
 }  // namespace lp

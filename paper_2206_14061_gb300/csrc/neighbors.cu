@@ -288,21 +288,27 @@ k_ghost_scan(int n, const int4* __restrict__ X, const int32_t* __restrict__ nbr,
   ghost_scan_body(s, s < n, n, X, nbr, cnt, gcnt, K, olist, gcount + 1);
 }
 
-// second half: the one-sided particles of the list, in full warps (a fixed
-// grid strides over the list a warp at a time, so every lane calls the body)
-constexpr int kGhostBlocks = 4 * 152;
-__global__ void __launch_bounds__(128)
+// second half: the one-sided particles of the list, kGhostLanes lanes each. A
+// fixed grid strides over the list eight particles (a warp) at a time, the
+// first warps of all blocks before the second ones, so that a short list
+// occupies every SM.
+constexpr int kGhostBlocks = 6 * 152;
+__global__ void __launch_bounds__(kGhostBlock)
 k_ghosts(int n, const double* __restrict__ z, const int4* __restrict__ X,
          int32_t* __restrict__ nbr, const int32_t* __restrict__ cnt, int32_t* __restrict__ gcnt,
          const StepConsts K, DevDiag* __restrict__ dg, int32_t* __restrict__ glist,
          int* __restrict__ gcount, const int32_t* __restrict__ olist) {
+  __shared__ GhostShared sh;
   const int m = min(gcount[1], n);
-  const int lane = threadIdx.x & 31;
-  const int stride = gridDim.x * blockDim.x;
-  for (int base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < m; base += stride) {
-    const int t = base + lane;
+  constexpr int kWarps = kGhostBlock / 32, kItems = 32 / kGhostLanes;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int item = lane / kGhostLanes, sub = lane % kGhostLanes;
+  for (int base = (warp * gridDim.x + blockIdx.x) * kItems; base < m;
+       base += gridDim.x * kWarps * kItems) {
+    const int t = base + item;
     const bool live = t < m;
-    ghost_body(live ? olist[t] : 0, live, n, z, X, nbr, cnt, gcnt, K, dg, glist, gcount);
+    ghost_group(live ? olist[t] : 0, live, warp * kItems + item, sub, sh, n, z, X, nbr, cnt, gcnt,
+                K, dg, glist, gcount);
   }
 }
 
@@ -395,6 +401,6 @@ void launch_ghosts(int n, const double* x, const double* y, const double* z,
                                                X, gcount);
   bs = spread_block(n, bs);
   k_ghost_scan<<<(n + bs - 1) / bs, bs, 0, st>>>(n, X, nbr, cnt, gcnt, K, olist, gcount);
-  k_ghosts<<<kGhostBlocks, 128, 0, st>>>(n, z, X, nbr, cnt, gcnt, K, dg, glist, gcount, olist);
+  k_ghosts<<<kGhostBlocks, kGhostBlock, 0, st>>>(n, z, X, nbr, cnt, gcnt, K, dg, glist, gcount, olist);
 }
 }  // namespace lp
