@@ -96,9 +96,15 @@ __device__ __forceinline__ int fit_particle(const StepArgs& A) {
 // moments and factor 0.71 ms, right-hand sides and solves 0.97 ms, pass 2
 // 0.85 ms; with the rows in FP64, on whose pipe they were bound (91 % busy),
 // pass 1 took 5.58 and pass 2 2.66 ms. 3 blocks of 128 threads at 168
-// registers: at 128 registers (4 blocks) the sums spill (the column's four
-// steps 12.1 -> 13.2 ms).
+// registers, or WIDE: 4 blocks at 128 registers, whose few spilled values (8
+// to 156 bytes a thread) cost less than the fourth block gives once there are
+// more particles than 3 blocks per SM take at a time. LP_FP64 steps with 3 and
+// with 4 blocks: 8,000 particles 944 and 977 us (4 steps), 17,000 964 and 976,
+// 64,000 1640 and 1573, 227,000 3789 and 3585, 402,000 6017 and 5591. The
+// right-hand sides of pass 1 stay at 3: 27 sums and the solve of three fields
+// spill 430 bytes (402,000: 5641 with 4).
 constexpr int kFxBlock = 128;
+constexpr int kFxWide = 3 * 152 * kFxBlock;  // particles that 3 blocks per SM hold
 __global__ void k_fx_split(const StepArgs A) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < A.n) fx_split_state_body(A, s);
@@ -107,8 +113,8 @@ __global__ void k_fx_split_p1(const StepArgs A) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < A.n) fx_split_p1_body(A, s);
 }
-template <bool PER, bool GH>
-__global__ void __launch_bounds__(kFxBlock, 3) k_gram_fx(const StepArgs A) {
+template <bool PER, bool GH, bool WIDE>
+__global__ void __launch_bounds__(kFxBlock, WIDE ? 4 : 3) k_gram_fx(const StepArgs A) {
   const int s = fit_particle(A);
   if (s < A.n) gram_fx_body<PER, GH>(A, s);
 }
@@ -117,10 +123,20 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_pass1_fx(const StepArgs A) {
   const int s = fit_particle(A);
   if (s < A.n) pass1_fx_body<PER>(A, s);
 }
-template <bool PER, bool GH>
-__global__ void __launch_bounds__(kFxBlock, 3) k_pass2_fx(const StepArgs A) {
+template <bool PER, bool GH, bool WIDE>
+__global__ void __launch_bounds__(kFxBlock, WIDE ? 4 : 3) k_pass2_fx(const StepArgs A) {
   const int s = fit_particle(A);
   pass2_body<kFixedRows, PER, GH>(A, s, s < A.n);
+}
+template <bool PER, bool GH>
+void launch_gram_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
+  if (A.n > kFxWide) k_gram_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
+  else k_gram_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
+}
+template <bool PER, bool GH>
+void launch_pass2_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
+  if (A.n > kFxWide) k_pass2_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
+  else k_pass2_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
 }
 // the particles that the fixed-point rows left to the plain FP64 rows
 constexpr int kSlowBlocks = 4 * 152;
@@ -771,13 +787,13 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
     const int b = bs < kFxBlock ? bs : kFxBlock;
     const int nf = (A.n + b - 1) / b;
     if (per) {
-      if (A.K.free_surface) k_gram_fx<true, true><<<nf, b, 0, st>>>(A);
-      else k_gram_fx<true, false><<<nf, b, 0, st>>>(A);
+      if (A.K.free_surface) launch_gram_fx<true, true>(A, nf, b, st);
+      else launch_gram_fx<true, false>(A, nf, b, st);
       k_pass1_fx<true><<<nf, b, 0, st>>>(A);
       k_pass1_slow<true><<<kSlowBlocks, 64, 0, st>>>(A);
     } else {
-      if (A.K.free_surface) k_gram_fx<false, true><<<nf, b, 0, st>>>(A);
-      else k_gram_fx<false, false><<<nf, b, 0, st>>>(A);
+      if (A.K.free_surface) launch_gram_fx<false, true>(A, nf, b, st);
+      else launch_gram_fx<false, false>(A, nf, b, st);
       k_pass1_fx<false><<<nf, b, 0, st>>>(A);
       k_pass1_slow<false><<<kSlowBlocks, 64, 0, st>>>(A);
     }
@@ -820,12 +836,12 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
     const int b = bs < kFxBlock ? bs : kFxBlock;
     const int nf = (A.n + b - 1) / b;
     if (per) {
-      if (A.K.free_surface) k_pass2_fx<true, true><<<nf, b, 0, st>>>(A);
-      else k_pass2_fx<true, false><<<nf, b, 0, st>>>(A);
+      if (A.K.free_surface) launch_pass2_fx<true, true>(A, nf, b, st);
+      else launch_pass2_fx<true, false>(A, nf, b, st);
       k_pass2_slow<true><<<kSlowBlocks, 64, 0, st>>>(A);
     } else {
-      if (A.K.free_surface) k_pass2_fx<false, true><<<nf, b, 0, st>>>(A);
-      else k_pass2_fx<false, false><<<nf, b, 0, st>>>(A);
+      if (A.K.free_surface) launch_pass2_fx<false, true>(A, nf, b, st);
+      else launch_pass2_fx<false, false>(A, nf, b, st);
       k_pass2_slow<false><<<kSlowBlocks, 64, 0, st>>>(A);
     }
   } else if (prec == LP_MIXED) {
