@@ -74,29 +74,105 @@ __device__ __forceinline__ double usign_adj(int mode, int a) {
   return mode == LP_MIRROR_NOSLIP ? -1.0 : (mode == LP_MIRROR_FREESLIP && a == 2 ? -1.0 : 1.0);
 }
 
-// adjoint of the Taylor row: dbar = J^T abar
-__device__ __forceinline__ void row_adjoint(double dx, double dy, double dz, const double* ab,
-                                            double* db) {
-  db[0] = ab[0] + dx * ab[3] + dy * ab[6] + dz * ab[7];
-  db[1] = ab[1] + dy * ab[4] + dx * ab[6] + dz * ab[8];
-  db[2] = ab[2] + dz * ab[5] + dx * ab[7] + dy * ab[8];
-}
-// the same in float-float
-__device__ __forceinline__ void ff_row_adjoint(ff dx, ff dy, ff dz, const ff* ab, ff* db) {
-  db[0] = ab[0];
-  ff_acc(db[0], dx, ab[3]);
-  ff_acc(db[0], dy, ab[6]);
-  ff_acc(db[0], dz, ab[7]);
-  db[1] = ab[1];
-  ff_acc(db[1], dy, ab[4]);
-  ff_acc(db[1], dx, ab[6]);
-  ff_acc(db[1], dz, ab[8]);
-  db[2] = ab[2];
-  ff_acc(db[2], dz, ab[5]);
-  ff_acc(db[2], dx, ab[7]);
-  ff_acc(db[2], dy, ab[8]);
+// The rows of both adjoints, kAdjLanes lanes to a particle: each takes every
+// kAdjLanes-th row, and the particle's own sums are added over the lanes in
+// FP64. One thread per particle needed 248 registers for its four or six
+// 9-vectors in float-float, so 8 warps at most fit on an SM (26,000 particles
+// put 5 there), all waiting for the dependent operations of their rows. The
+// lanes of a particle share the vectors in shared memory (14 KB a block), which
+// leaves 127 registers: 16 warps. 26,000 particles with ghosts, pass-1 and
+// pass-2 rows: 259 and 160 us with a thread each, 215 and 114 with four lanes
+// and the vectors in registers, 155 and 104 so.
+constexpr int kAdjLanes = 4;
+
+// A fit's quadratic p(d) = v . T(d) = l . d + d . H d / 2 (l = v[0..2], H from
+// v[3..8]) and its gradient g = J^T v = l + H d at d: the value is
+// d . (l + g) / 2, so neither the Taylor row nor J^T of a 9-vector is formed.
+__device__ __forceinline__ ff ff_half_dot(const ff* v, const ff* g, const ff* d) {
+  ff p = {0.f, 0.f};
 #pragma unroll
-  for (int q = 0; q < 3; ++q) db[q] = ff_norm(db[q]);
+  for (int a = 0; a < 3; ++a) {
+    ff t = two_sum(v[a].h, g[a].h);
+    t.l = __fadd_rn(t.l, __fadd_rn(v[a].l, g[a].l));
+    ff_acc(p, d[a], t);
+  }
+  return ff_scale(ff_norm(p), 0.5f);
+}
+__device__ __forceinline__ ff ff_quadratic(const ff* v, const ff* d, ff* g) {
+  const int H[3][3] = {{3, 6, 7}, {6, 4, 8}, {7, 8, 5}};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    g[a] = v[a];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ff_acc(g[a], d[c], v[H[a][c]]);
+    g[a] = ff_norm(g[a]);
+  }
+  return ff_half_dot(v, g, d);
+}
+// the same at the reflected offset -d, from the gradient at d: l - H d = 2 l - g
+__device__ __forceinline__ ff ff_quadratic_reflected(const ff* v, const ff* d, ff* g) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) g[a] = ff_sub(ff_scale(v[a], 2.f), g[a]);
+  return ff_neg(ff_half_dot(v, g, d));
+}
+// A particle's float-float vectors in shared memory, entry e of slot p at
+// [e][p]; a lane reads the nine entries of one where the row needs them.
+constexpr int kAdjBlock = 128;
+constexpr int kAdjSlots = kAdjBlock / kAdjLanes;
+__device__ __forceinline__ void adj_vector(const float2 (*sh)[kAdjSlots], int e, int slot, ff* v) {
+#pragma unroll
+  for (int q = 0; q < kNB; ++q) {
+    const float2 w = sh[e * kNB + q][slot];
+    v[q] = ff{w.x, w.y};
+  }
+}
+// One field of a row: z and the fit's coefficients c, right-hand side rhs at
+// d; returns b = z . T(d) and adds the row's part of the offset's adjoint,
+// (rhs - c . T) J^T z - b J^T c, to db. With a ghost (the row T(-d), rhs_g),
+// *bg is its b, and its part of the adjoint enters with the opposite sign.
+// ez, ec: the vectors' numbers in shared memory.
+__device__ __forceinline__ ff adj_row_field(const float2 (*sh)[kAdjSlots], int ez, int ec,
+                                            int slot, const ff* d, ff rhs, bool ghost, ff rhs_g,
+                                            ff* bg, ff* db) {
+  ff gz[3], gc[3], z[kNB], c[kNB];
+  adj_vector(sh, ez, slot, z);
+  adj_vector(sh, ec, slot, c);
+  const ff b = ff_quadratic(z, d, gz);
+  const ff r = ff_sub(rhs, ff_quadratic(c, d, gc));
+  const ff nb = ff_neg(b);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    ff_acc(db[a], r, gz[a]);
+    ff_acc(db[a], nb, gc[a]);
+  }
+  if (ghost) {
+    *bg = ff_quadratic_reflected(z, d, gz);
+    const ff nr = ff_sub(ff_quadratic_reflected(c, d, gc), rhs_g);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      ff_acc(db[a], nr, gz[a]);
+      ff_acc(db[a], *bg, gc[a]);
+    }
+  }
+  return b;
+}
+// sum over the lanes of a particle
+__device__ __forceinline__ double adj_lane_sum(unsigned group, double v) {
+#pragma unroll
+  for (int o = 1; o < kAdjLanes; o <<= 1) v += __shfl_xor_sync(group, v, o);
+  return v;
+}
+// the offset of a row (ff_row_of without the quadratic terms)
+template <bool PER>
+__device__ __forceinline__ void adj_offset(const float4& hi, const float4& lo, const FF8& rj,
+                                           bool mir, const StepConsts& K, ff* d) {
+  d[0] = ff_diff(rj.xh.x, rj.xl.x, hi.x, lo.x);
+  d[1] = ff_diff(rj.xh.y, rj.xl.y, hi.y, lo.y);
+  if (PER) {
+    d[0] = ff_min_image(d[0], K.Lhx_h, K.Lhx_l);
+    d[1] = ff_min_image(d[1], K.Lhy_h, K.Lhy_l);
+  }
+  d[2] = mir ? ff_diff(rj.xh.w, rj.xl.w, hi.z, lo.z) : ff_diff(rj.xh.z, rj.xl.z, hi.z, lo.z);
 }
 
 // ---------------------------------------------------------------- R0
@@ -272,23 +348,26 @@ __global__ void __launch_bounds__(kBlock) k_adj_accel(const AdjArgs A) {
 // rows of the pass-2 adjoint: to the neighbours' |gdot| and V^{n+1}, and to
 // the positions
 template <bool PER>
-__global__ void __launch_bounds__(kBlock) k_adj_pass2(const AdjArgs A) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kAdjBlock, 4) k_adj_pass2(const AdjArgs A) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = t / kAdjLanes, sub = t % kAdjLanes;
   if (s >= A.n || !A.ok[s]) return;
+  const unsigned group = ((1u << kAdjLanes) - 1u) << ((threadIdx.x & 31) - sub);
   const int n = A.n;
   // z and the forward coefficients c of the two pass-2 fits (|gdot|, V), split once
-  ff zg[kNB], zV[kNB], cg[kNB], cV[kNB];
+  // (0 z of |gdot|, 1 z of V, 2 and 3 their coefficients)
+  __shared__ float2 sh[4 * kNB][kAdjSlots];
+  const int slot = threadIdx.x / kAdjLanes;
   bool any = false;
-#pragma unroll
-  for (int q = 0; q < kNB; ++q) {
-    const double zgq = A.zz[(int64_t)q * n + s], zVq = A.zz[(int64_t)(kNB + q) * n + s];
-    any = any || zgq != 0.0 || zVq != 0.0;
-    zg[q] = ff_of(zgq);
-    zV[q] = ff_of(zVq);
-    cg[q] = ff_of(A.coef2[(int64_t)q * n + s]);
-    cV[q] = ff_of(A.coef2[(int64_t)(kNB + q) * n + s]);
+  for (int e = sub; e < 2 * kNB; e += kAdjLanes) {
+    const double zq = A.zz[(int64_t)e * n + s];
+    any = any || zq != 0.0;
+    const ff z = ff_of(zq), c = ff_of(A.coef2[(int64_t)e * n + s]);
+    sh[e][slot] = make_float2(z.h, z.l);
+    sh[2 * kNB + e][slot] = make_float2(c.h, c.l);
   }
-  if (!any) return;
+  if (!__any_sync(group, any)) return;  // (and the lanes' entries are in place)
+  __syncwarp(group);
   const double* Gn = A.p1 + P1_GN * n;
   // V of the pass-2 fit: V^{n+1}, or V^n in an Euler stage (whose adjoint is lVd)
   const double* Vn = A.K.euler ? A.V : A.p1 + P1_VN * n;
@@ -317,88 +396,48 @@ __global__ void __launch_bounds__(kBlock) k_adj_pass2(const AdjArgs A) {
   ff sg = {0.f, 0.f}, sV = {0.f, 0.f};
   ff sp[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   double og = 0.0, oV = 0.0;  // adjoints of the particle's own gni, Vi from ghost rows
-  for (int k = 0; k < m; ++k) {
+  for (int k = sub; k < m; k += kAdjLanes) {
     const uint32_t code = (uint32_t)A.nbr[(int64_t)k * n + s];
     const int j = code & kIndexMask;
     if ((unsigned)j >= (unsigned)n) continue;  // stale or corrupt stencil entry
-    const bool mir = code >> 31;
+    const bool mir = code >> 31, ghost = code & kGhostBit;
     const FF8& rj = A.XU[j];
-    const FFRow row = ff_row_of<PER>(hi, lo, rj.xh, rj.xl, code, A.K);
-    ff a[kNB];
-    ff_taylor(row, a);
+    ff d[3];
+    adj_offset<PER>(hi, lo, rj, mir, A.K, d);
     const float4 gvj = rj.uh;
-    ff rg = mir ? ff{-gvi.x, -gvi.y} : ff_diff(gvj.x, gvj.y, gvi.x, gvi.y);
-    ff rV = ff_diff(gvj.z, gvj.w, gvi.z, gvi.w), bg = {0.f, 0.f}, bV = {0.f, 0.f};
-#pragma unroll
-    for (int q = 0; q < kNB; ++q) {
-      ff_acc(rg, a[q], ff_neg(cg[q]));
-      ff_acc(rV, a[q], ff_neg(cV[q]));
-      ff_acc(bg, a[q], zg[q]);
-      ff_acc(bV, a[q], zV[q]);
-    }
-    rg = ff_norm(rg);
-    rV = ff_norm(rV);
-    bg = ff_norm(bg);
-    bV = ff_norm(bV);
+    const ff rg = mir ? ff{-gvi.x, -gvi.y} : ff_diff(gvj.x, gvj.y, gvi.x, gvi.y);
+    const ff rV = ff_diff(gvj.z, gvj.w, gvi.z, gvi.w);
+    ff db[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, bgb, bVb;
+    const ff bg = adj_row_field(sh, 0, 2, slot, d, rg, ghost, bgGf, &bgb, db);
+    const ff bV = adj_row_field(sh, 1, 3, slot, d, rV, ghost, bvGf, &bVb, db);
     if (!mir) atomicAdd(&A.lGn[j], ffs_to_double(bg.h) + ffs_to_double(bg.l));
     sg = ff_add(sg, bg);
     atomicAdd(&lVfit[j], ffs_to_double(bV.h) + ffs_to_double(bV.l));  // the mirror of j carries V_j
     sV = ff_add(sV, bV);
-    ff ab[kNB];
-    const ff nbg = ff_neg(bg), nbV = ff_neg(bV);
-#pragma unroll
-    for (int q = 0; q < kNB; ++q) {
-      ab[q] = {0.f, 0.f};
-      ff_acc(ab[q], rg, zg[q]);
-      ff_acc(ab[q], nbg, cg[q]);
-      ff_acc(ab[q], rV, zV[q]);
-      ff_acc(ab[q], nbV, cV[q]);
-    }
-    ff db[3];
-    ff_row_adjoint(row.dx, row.dy, row.dz, ab, db);
-    if (code & kGhostBit) {  // the ghost's row T(-d)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) a[q] = ff_neg(a[q]);  // T(-d): linear terms flip
-      ff rgG = bgGf, rVG = bvGf, bgb = {0.f, 0.f}, bVb = {0.f, 0.f};
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) {
-        ff_acc(rgG, a[q], ff_neg(cg[q]));
-        ff_acc(rVG, a[q], ff_neg(cV[q]));
-        ff_acc(bgb, a[q], zg[q]);
-        ff_acc(bVb, a[q], zV[q]);
-      }
-      rgG = ff_norm(rgG);
-      rVG = ff_norm(rVG);
-      bgb = ff_norm(bgb);
-      bVb = ff_norm(bVb);
+    if (ghost) {  // the ghost's row T(-d)
       const double bgbd = ffs_to_double(bgb.h) + ffs_to_double(bgb.l);
       og += bgbd * dbg_dg;
       oV += bgbd * dbg_dV - (ffs_to_double(bVb.h) + ffs_to_double(bVb.l));
-      const ff nbgb = ff_neg(bgb), nbVb = ff_neg(bVb);
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) {
-        ab[q] = {0.f, 0.f};
-        ff_acc(ab[q], rgG, zg[q]);
-        ff_acc(ab[q], nbgb, cg[q]);
-        ff_acc(ab[q], rVG, zV[q]);
-        ff_acc(ab[q], nbVb, cV[q]);
-      }
-      ff dbG[3];
-      ff_row_adjoint(ff_neg(row.dx), ff_neg(row.dy), ff_neg(row.dz), ab, dbG);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) db[c] = ff_sub(db[c], dbG[c]);
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      const ff g = ff_mul(q == 2 && mir ? ff_neg(db[q]) : db[q], ihf);
-      atomicAdd(&A.l0[q][j], ffs_to_double(g.h) + ffs_to_double(g.l));
-      sp[q] = ff_add(sp[q], ff_mul(db[q], ihf));
+      const ff g = ff_mul(ff_norm(db[q]), ihf);
+      const float sj = q == 2 && mir ? -1.f : 1.f;
+      atomicAdd(&A.l0[q][j], ffs_to_double(sj * g.h) + ffs_to_double(sj * g.l));
+      sp[q] = ff_add(sp[q], g);
     }
   }
-  atomicAdd(&A.lGn[s], og - (ffs_to_double(sg.h) + ffs_to_double(sg.l)));
-  atomicAdd(&lVfit[s], oV - (ffs_to_double(sV.h) + ffs_to_double(sV.l)));
-  for (int c = 0; c < 3; ++c)
-    atomicAdd(&A.l0[c][s], -(ffs_to_double(sp[c].h) + ffs_to_double(sp[c].l)));
+  og = adj_lane_sum(group, og - (ffs_to_double(sg.h) + ffs_to_double(sg.l)));
+  oV = adj_lane_sum(group, oV - (ffs_to_double(sV.h) + ffs_to_double(sV.l)));
+  if (sub == 0) {
+    atomicAdd(&A.lGn[s], og);
+    atomicAdd(&lVfit[s], oV);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double v = adj_lane_sum(group, -(ffs_to_double(sp[c].h) + ffs_to_double(sp[c].l)));
+    if (sub == 0) atomicAdd(&A.l0[c][s], v);
+  }
 }
 
 // ---------------------------------------------------------------- R3
@@ -418,16 +457,18 @@ __global__ void k_adj_split(const AdjArgs A) {
 // pass-1 adjoint: |gdot| and ld to the velocity gradient and Hessians, then
 // the least-squares rows to the neighbours' velocities and the positions
 template <bool PER>
-__global__ void __launch_bounds__(kBlock) k_adj_pass1(const AdjArgs A) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kAdjBlock, 4) k_adj_pass1(const AdjArgs A) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = t / kAdjLanes, sub = t % kAdjLanes;
   if (s >= A.n) return;
+  const unsigned group = ((1u << kAdjLanes) - 1u) << ((threadIdx.x & 31) - sub);
   const int n = A.n;
   const double dt = A.K.dt, ih = A.K.inv_h, ih2 = ih * ih;
   const double lVn = A.lVn[s];
   const double div = A.p1[P1_DIV * n + s];
   const double Vi = A.V[s];
   // V^{n+1} = V + dt V div; an Euler stage's fits and closure read V itself
-  A.l0[6][s] = lVn * (1.0 + dt * div) + (A.K.euler ? A.lVd[s] : 0.0);
+  if (sub == 0) A.l0[6][s] = lVn * (1.0 + dt * div) + (A.K.euler ? A.lVd[s] : 0.0);
   if (!A.ok[s]) return;
   const double ldiv = lVn * dt * Vi;
   const double Gn = A.p1[P1_GN * n + s];
@@ -462,25 +503,33 @@ __global__ void __launch_bounds__(kBlock) k_adj_pass1(const AdjArgs A) {
   for (int f = 0; f < 3; ++f)
     for (int q = 0; q < kNB; ++q) any = any || lc[f][q] != 0.0;
   if (!any) return;
-  {
+  // (0 to 2 z_f, 3 to 5 c_f)
+  __shared__ float2 sh[6 * kNB][kAdjSlots];
+  const int slot = threadIdx.x / kAdjLanes;
+  if (sub < 3) {  // z_f = G^{-1} lc_f, a field to a lane
+    static_assert(kAdjLanes >= 3, "a lane for each field");
     const double* F = factor_of(A, s);
-    double L[kTri];
+    double L[kTri], v[kNB];
 #pragma unroll
     for (int k = 0; k < kTri; ++k) L[k] = F[(int64_t)k * n + s];
-    for (int f = 0; f < 3; ++f) chol9_solve(L, lc[f]);  // lc becomes z_f
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) v[q] = sub == 0 ? lc[0][q] : (sub == 1 ? lc[1][q] : lc[2][q]);
+    chol9_solve(L, v);
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) {
+      const ff z = ff_of(v[q]);
+      sh[sub * kNB + q][slot] = make_float2(z.h, z.l);
+    }
   }
+  for (int e = sub; e < 3 * kNB; e += kAdjLanes) {
+    const ff c = ff_of(A.coef1[(int64_t)e * n + s]);
+    sh[3 * kNB + e][slot] = make_float2(c.h, c.l);
+  }
+  __syncwarp(group);
   // The rows in float-float (the forward step's coefficients c_f and the z_f
   // split once; the offsets and velocity differences from the split state):
   // the rows' residuals, b = a . z and the row adjoints run on the FP32 pipe,
   // and only the scattered sums are FP64, converted exactly from float-float.
-  ff cf[3][kNB], zf[3][kNB];
-#pragma unroll
-  for (int f = 0; f < 3; ++f)
-#pragma unroll
-    for (int q = 0; q < kNB; ++q) {
-      cf[f][q] = ff_of(A.coef1[(int64_t)(f * kNB + q) * n + s]);
-      zf[f][q] = ff_of(lc[f][q]);
-    }
   const int mm = A.K.mirror_mode;
   const float sgn[3] = {(float)usign_adj(mm, 0), (float)usign_adj(mm, 1),
                         (float)usign_adj(mm, 2)};
@@ -489,80 +538,43 @@ __global__ void __launch_bounds__(kBlock) k_adj_pass1(const AdjArgs A) {
   const ff ihf{A.K.ih_h, A.K.ih_l};
   const int m = min(A.cnt[s], A.cap);
   ff su[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, sp[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  for (int k = 0; k < m; ++k) {
+  for (int k = sub; k < m; k += kAdjLanes) {
     const uint32_t code = (uint32_t)A.nbr[(int64_t)k * n + s];
     const int j = code & kIndexMask;
     if ((unsigned)j >= (unsigned)n) continue;  // stale or corrupt stencil entry
-    const bool mir = code >> 31;
+    const bool mir = code >> 31, ghost = code & kGhostBit;
     const FF8& rj = A.XU[j];
-    const FFRow row = ff_row_of<PER>(hi, lo, rj.xh, rj.xl, code, A.K);
-    ff a[kNB];
-    ff_taylor(row, a);
+    ff d[3];
+    adj_offset<PER>(hi, lo, rj, mir, A.K, d);
     const float ujh[3] = {rj.uh.x, rj.uh.y, rj.uh.z}, ujl[3] = {rj.ul.x, rj.ul.y, rj.ul.z};
-    ff ab[kNB];
-#pragma unroll
-    for (int q = 0; q < kNB; ++q) ab[q] = {0.f, 0.f};
+    ff db[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
       const float sj = mir ? sgn[f] : 1.f;
-      ff r = ff_diff(sj * ujh[f], sj * ujl[f], uih[f], uil[f]), b = {0.f, 0.f};
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) {
-        ff_acc(r, a[q], ff_neg(cf[f][q]));
-        ff_acc(b, a[q], zf[f][q]);
-      }
-      r = ff_norm(r);
-      b = ff_norm(b);
+      ff bg;  // (a ghost row's right-hand side is fixed at 0)
+      const ff b = adj_row_field(sh, f, 3 + f, slot, d,
+                                 ff_diff(sj * ujh[f], sj * ujl[f], uih[f], uil[f]), ghost,
+                                 ff{0.f, 0.f}, &bg, db);
       atomicAdd(&A.l0[3 + f][j], ffs_to_double(sj * b.h) + ffs_to_double(sj * b.l));
       su[f] = ff_add(su[f], b);
-      const ff nb = ff_neg(b);
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) {
-        ff_acc(ab[q], r, zf[f][q]);
-        ff_acc(ab[q], nb, cf[f][q]);
-      }
-    }
-    ff db[3];
-    ff_row_adjoint(row.dx, row.dy, row.dz, ab, db);
-    if (code & kGhostBit) {  // the ghost's row T(-d), right-hand sides 0
-      const ff ndx = ff_neg(row.dx), ndy = ff_neg(row.dy), ndz = ff_neg(row.dz);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) a[q] = ff_neg(a[q]);  // T(-d): linear terms flip
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) ab[q] = {0.f, 0.f};
-#pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        ff r = {0.f, 0.f}, b = {0.f, 0.f};
-#pragma unroll
-        for (int q = 0; q < kNB; ++q) {
-          ff_acc(r, a[q], ff_neg(cf[f][q]));
-          ff_acc(b, a[q], zf[f][q]);
-        }
-        r = ff_norm(r);
-        b = ff_norm(b);
-        const ff nb = ff_neg(b);
-#pragma unroll
-        for (int q = 0; q < kNB; ++q) {
-          ff_acc(ab[q], r, zf[f][q]);
-          ff_acc(ab[q], nb, cf[f][q]);
-        }
-      }
-      ff dbG[3];
-      ff_row_adjoint(ndx, ndy, ndz, ab, dbG);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) db[q] = ff_sub(db[q], dbG[q]);
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      const ff g = ff_mul(q == 2 && mir ? ff_neg(db[q]) : db[q], ihf);
-      atomicAdd(&A.l0[q][j], ffs_to_double(g.h) + ffs_to_double(g.l));
-      sp[q] = ff_add(sp[q], ff_mul(db[q], ihf));
+      const ff g = ff_mul(ff_norm(db[q]), ihf);
+      const float sj = q == 2 && mir ? -1.f : 1.f;
+      atomicAdd(&A.l0[q][j], ffs_to_double(sj * g.h) + ffs_to_double(sj * g.l));
+      sp[q] = ff_add(sp[q], g);
     }
   }
-  for (int f = 0; f < 3; ++f)
-    atomicAdd(&A.l0[3 + f][s], -(ffs_to_double(su[f].h) + ffs_to_double(su[f].l)));
-  for (int q = 0; q < 3; ++q)
-    atomicAdd(&A.l0[q][s], -(ffs_to_double(sp[q].h) + ffs_to_double(sp[q].l)));
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const double v = adj_lane_sum(group, -(ffs_to_double(su[f].h) + ffs_to_double(su[f].l)));
+    const double w = adj_lane_sum(group, -(ffs_to_double(sp[f].h) + ffs_to_double(sp[f].l)));
+    if (sub == 0) {
+      atomicAdd(&A.l0[3 + f][s], v);
+      atomicAdd(&A.l0[f][s], w);
+    }
+  }
 }
 
 // dst[f][s] = src[f][idx[s]] (caller order to sorted order)
@@ -584,14 +596,16 @@ void launch_gather_fields(int n, const int32_t* idx, const double* const* src, d
 void launch_adjoint_step(const AdjArgs& A, cudaStream_t st) {
   const int bs = spread_block(A.n, kBlock);
   const int nb = (A.n + bs - 1) / bs;
+  const int64_t lanes = (int64_t)A.n * kAdjLanes;  // threads of the row kernels
+  const int nr = (int)((lanes + kAdjBlock - 1) / kAdjBlock);
   k_adj_prepare<<<nb, bs, 0, st>>>(A);
   k_adj_accel<<<nb, bs, 0, st>>>(A);
   k_adj_split<true><<<nb, bs, 0, st>>>(A);
-  if (A.K.periodic) k_adj_pass2<true><<<nb, bs, 0, st>>>(A);
-  else k_adj_pass2<false><<<nb, bs, 0, st>>>(A);
+  if (A.K.periodic) k_adj_pass2<true><<<nr, kAdjBlock, 0, st>>>(A);
+  else k_adj_pass2<false><<<nr, kAdjBlock, 0, st>>>(A);
   k_adj_split<false><<<nb, bs, 0, st>>>(A);
-  if (A.K.periodic) k_adj_pass1<true><<<nb, bs, 0, st>>>(A);
-  else k_adj_pass1<false><<<nb, bs, 0, st>>>(A);
+  if (A.K.periodic) k_adj_pass1<true><<<nr, kAdjBlock, 0, st>>>(A);
+  else k_adj_pass1<false><<<nr, kAdjBlock, 0, st>>>(A);
 }
 
 }  // namespace lp
