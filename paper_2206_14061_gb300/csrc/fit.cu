@@ -128,14 +128,51 @@ __global__ void __launch_bounds__(kFxBlock, WIDE ? 4 : 3) k_pass2_fx(const StepA
   const int s = fit_particle(A);
   pass2_body<kFixedRows, PER, GH>(A, s, s < A.n);
 }
+// Few particles: four lanes to a particle (k_*_fx_lanes). 8,000 particles, one
+// thread each, are 250 warps, fewer than the chip has schedulers, and each row
+// waits for its gathers; four lanes take a quarter of the rows each. Four
+// LP_FP64 steps with a thread and with four lanes each: 512 particles 869 and
+// 715 us, 2,744 908 and 746, 8,000 939 and 786, 17,000 956 and 1039, 26,000
+// 1074 and 1102. The line: what one wave of the lanes' blocks takes, 3 per SM.
+constexpr int kFxSplit = 3 * 152 * kFxSlots;
+// (particle of rank t, or -1)
+struct FxParticles {
+  const StepArgs& A;
+  __device__ __forceinline__ int operator()(int t) const {
+    return t < A.n ? (A.perm ? A.perm[t] : t) : -1;
+  }
+};
+template <bool PER, bool GH>
+__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_gram_fx_lanes(const StepArgs A) {
+  gram_fx_lanes<PER, GH>(A, FxParticles{A});
+}
+template <bool PER>
+__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_pass1_fx_lanes(const StepArgs A) {
+  pass1_fx_lanes<PER>(A, FxParticles{A});
+}
+template <bool PER, bool GH>
+__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_pass2_fx_lanes(const StepArgs A) {
+  pass2_fx_lanes<PER, GH>(A, FxParticles{A});
+}
+int fx_lane_blocks(int n) { return (n + kFxSlots - 1) / kFxSlots; }
 template <bool PER, bool GH>
 void launch_gram_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
-  if (A.n > kFxWide) k_gram_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
+  if (A.n <= kFxSplit)
+    k_gram_fx_lanes<PER, GH><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  else if (A.n > kFxWide) k_gram_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
   else k_gram_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
+}
+template <bool PER>
+void launch_pass1_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
+  if (A.n <= kFxSplit)
+    k_pass1_fx_lanes<PER><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  else k_pass1_fx<PER><<<nf, b, 0, st>>>(A);
 }
 template <bool PER, bool GH>
 void launch_pass2_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
-  if (A.n > kFxWide) k_pass2_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
+  if (A.n <= kFxSplit)
+    k_pass2_fx_lanes<PER, GH><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  else if (A.n > kFxWide) k_pass2_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
   else k_pass2_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
 }
 // the particles that the fixed-point rows left to the plain FP64 rows
@@ -789,12 +826,12 @@ void launch_pass1(int prec, const StepArgs& A, cudaStream_t st, int bs) {
     if (per) {
       if (A.K.free_surface) launch_gram_fx<true, true>(A, nf, b, st);
       else launch_gram_fx<true, false>(A, nf, b, st);
-      k_pass1_fx<true><<<nf, b, 0, st>>>(A);
+      launch_pass1_fx<true>(A, nf, b, st);
       k_pass1_slow<true><<<kSlowBlocks, 64, 0, st>>>(A);
     } else {
       if (A.K.free_surface) launch_gram_fx<false, true>(A, nf, b, st);
       else launch_gram_fx<false, false>(A, nf, b, st);
-      k_pass1_fx<false><<<nf, b, 0, st>>>(A);
+      launch_pass1_fx<false>(A, nf, b, st);
       k_pass1_slow<false><<<kSlowBlocks, 64, 0, st>>>(A);
     }
   } else if (prec == LP_MIXED) {

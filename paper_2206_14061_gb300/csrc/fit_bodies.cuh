@@ -252,18 +252,11 @@ __device__ __forceinline__ void pass1_body(const StepArgs& A, int s) {
 // (which queues for the QR fit): there rounding is amplified ten-thousandfold,
 // and they keep the plain rows' results. None of a column's or cube's particles is
 // below it.
-template <bool PER, bool GH>
-__device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
+__device__ __forceinline__ void gram_fx_finish(const StepArgs& A, int s, int m, bool fits,
+                                               const double* mo) {
   const int64_t n = A.n;
-  const int m = min(A.cnt[s], A.cap);
   double L[kTri];
-  bool fits;
-  {
-    double mo[31];
-    int rows;
-    fits = fx_moments<PER, GH>(A, s, m, mo, &rows);
-    if (fits) gram_of_moments(mo, L);
-  }
+  if (fits) gram_of_moments(mo, L);
   bool ill;
   fits = fits && fx_chol9(L, 1e-9, &ill) && m >= kNB && !ill;
   A.kx[s] = fits ? 0 : 1;
@@ -275,19 +268,42 @@ __device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
 #pragma unroll
   for (int k = 0; k < kTri; ++k) A.fac[k * n + s] = L[k];
 }
-template <bool PER>
-__device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
-  if (A.kx[s] || A.fbslot[s] != -1) return;  // queued for the plain rows or the QR fit
-  const int64_t n = A.n;
-  const int m = min(A.cnt[s], A.cap);  // ghost rows carry b = 0: no right-hand side
-  const int mm = A.K.mirror_mode;
-  const int sgn[3] = {mm == LP_MIRROR_NOSLIP ? -1 : 1, mm == LP_MIRROR_NOSLIP ? -1 : 1,
-                      mm != LP_MIRROR_NONE ? -1 : 1};
-  double R[3][kNB];
-  if (!fx_rhs<3, PER, false>(A, s, m, sgn, nullptr, R)) {
-    fx_push(A, s, 0);
-    return;
+template <bool PER, bool GH>
+__device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
+  const int m = min(A.cnt[s], A.cap);
+  double mo[31];
+  int rows;
+  const bool fits = fx_moments<PER, GH>(A, s, m, mo, &rows);
+  gram_fx_finish(A, s, m, fits, mo);
+}
+// the same with the rows taken by kFxLanes lanes (a block of kFxLanes * 32
+// threads calls it; particle_of(t): the particle of rank t, or -1)
+template <bool PER, bool GH, class F>
+__device__ __forceinline__ void gram_fx_lanes(const StepArgs& A, F particle_of) {
+  __shared__ FxShared<31> S;
+  {
+    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int s = particle_of(blockIdx.x * kFxSlots + slot);
+    long long H[31];
+    int rows;
+    const bool fits = fx_moment_rows<PER, GH, false, kFxLanes>(
+        A, max(s, 0), s >= 0 ? min(A.cnt[s], A.cap) : 0, sub, H, &rows, 0);
+    fx_lanes_store(S, slot, sub, H, fits);
   }
+  __syncthreads();
+  if (threadIdx.x >= kFxSlots) return;
+  const int s = particle_of(blockIdx.x * kFxSlots + threadIdx.x);
+  if (s < 0) return;
+  long long H[31];
+#pragma unroll
+  for (int q = 0; q < 31; ++q) H[q] = S.H[q][threadIdx.x];
+  double mo[31];
+  fx_moment_values<false>(A.K, H, 0, mo);
+  gram_fx_finish(A, s, min(A.cnt[s], A.cap), S.fits[threadIdx.x], mo);
+}
+
+__device__ __forceinline__ void pass1_fx_finish(const StepArgs& A, int s, double (*R)[kNB]) {
+  const int64_t n = A.n;
   {
     double L[kTri];
 #pragma unroll
@@ -303,6 +319,53 @@ __device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
       for (int q = 0; q < kNB; ++q) A.coef1[(int64_t)(f * kNB + q) * n + s] = R[f][q];
   }
   pass1_finish(A, s, R);
+}
+// (ghost rows carry b = 0: no right-hand side in pass 1)
+__device__ __forceinline__ void pass1_signs(const StepArgs& A, int* sgn) {
+  const int mm = A.K.mirror_mode;
+  sgn[0] = sgn[1] = mm == LP_MIRROR_NOSLIP ? -1 : 1;
+  sgn[2] = mm != LP_MIRROR_NONE ? -1 : 1;
+}
+template <bool PER>
+__device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
+  if (A.kx[s] || A.fbslot[s] != -1) return;  // queued for the plain rows or the QR fit
+  int sgn[3];
+  pass1_signs(A, sgn);
+  double R[3][kNB];
+  if (!fx_rhs<3, PER, false>(A, s, min(A.cnt[s], A.cap), sgn, nullptr, R)) {
+    fx_push(A, s, 0);
+    return;
+  }
+  pass1_fx_finish(A, s, R);
+}
+template <bool PER, class F>
+__device__ __forceinline__ void pass1_fx_lanes(const StepArgs& A, F particle_of) {
+  __shared__ FxShared<3 * kNB> S;
+  auto has_rows = [&](int s) { return s >= 0 && !A.kx[s] && A.fbslot[s] == -1; };
+  {
+    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int s = particle_of(blockIdx.x * kFxSlots + slot);
+    int sgn[3], kb[3];
+    pass1_signs(A, sgn);
+    long long H[3][kNB];
+    const bool fits = fx_rhs_rows<3, PER, false, false, kFxLanes>(
+        A, max(s, 0), has_rows(s) ? min(A.cnt[s], A.cap) : 0, sub, sgn, nullptr, H, kb, 0);
+    fx_lanes_store(S, slot, sub, &H[0][0], fits);
+#pragma unroll
+    for (int f = 0; f < 3; ++f)
+      if (sub == f) S.kb[f][slot] = kb[f];
+  }
+  __syncthreads();
+  if (threadIdx.x >= kFxSlots) return;
+  const int s = particle_of(blockIdx.x * kFxSlots + threadIdx.x);
+  if (!has_rows(s)) return;
+  if (!S.fits[threadIdx.x]) {
+    fx_push(A, s, 0);
+    return;
+  }
+  double R[3][kNB];
+  fx_shared_values(A.K, S, threadIdx.x, R);
+  pass1_fx_finish(A, s, R);
 }
 
 // pivoted-QR fallback of pass 1 (grid-stride over the queued particles)
@@ -1066,8 +1129,10 @@ __device__ __forceinline__ void accel_ff(const StepArgs& A, int s, const ff* gg,
 
 // every lane of the warp must call it (live or not)
 // (GH: the stencils may carry ghosts; only the fixed-point rows ask)
-template <int PREC, bool PER = false, bool GH = true>
-__device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) {
+// (pre, col: the sums of the fixed-point rows, if they are at hand)
+template <int PREC, bool PER = false, bool GH = true, bool PRE = false>
+__device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live,
+                                           const FxShared<2 * kNB>* pre = nullptr, int col = 0) {
   int regime = 1;
   bool overc = false, nonfin = false, below = false;
   float disp = 0.f;  // displacement from the search positions (filter skipping)
@@ -1104,9 +1169,16 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
         for (int q = 0; q < 3; ++q) gg[q] = gV[q] = 0.0;  // set below where needed
       } else if (PREC == kFixedRows) {
         double R[2][kNB], bG[2] = {0.0, 0.0};
-        if (GH && A.K.free_surface) ghost_rhs2(A, gni, Vi, &bG[0], &bG[1]);
-        const int sgn[2] = {0, 1};
-        if (!fx_rhs<2, PER, GH>(A, s, m, sgn, bG, R)) {  // plain FP64 rows
+        bool fits;
+        if (PRE) {
+          fits = pre->fits[col];
+          fx_shared_values(A.K, *pre, col, R);
+        } else {
+          if (GH && A.K.free_surface) ghost_rhs2(A, gni, Vi, &bG[0], &bG[1]);
+          const int sgn[2] = {0, 1};
+          fits = fx_rhs<2, PER, GH>(A, s, m, sgn, bG, R);
+        }
+        if (!fits) {  // plain FP64 rows
           fx_push(A, s, 1);
           live = false;
           break;
@@ -1346,6 +1418,45 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live) 
   }
   if (live && nonfin) atomicOr(&A.dg->flags, (unsigned)LP_FLAG_NONFINITE);
   if (live && below) atomicOr(&A.dg->flags, (unsigned)LP_FLAG_BELOW_FLOOR);
+}
+// LP_FP64 with the rows taken by kFxLanes lanes (as gram_fx_lanes)
+template <bool PER, bool GH, class F>
+__device__ __forceinline__ void pass2_fx_lanes(const StepArgs& A, F particle_of) {
+  __shared__ FxShared<2 * kNB> S;
+  __shared__ double ghost_b[2][kFxSlots];
+  const int first = blockIdx.x * kFxSlots;
+  if (GH) {  // right-hand sides of the ghost rows
+    if (threadIdx.x < kFxSlots) {
+      const int s = particle_of(first + threadIdx.x);
+      double b[2] = {0.0, 0.0};
+      if (s >= 0 && A.K.free_surface)
+        ghost_rhs2(A, A.p1[P1_GN * A.n + s], A.K.euler ? A.V[s] : A.p1[P1_VN * A.n + s], &b[0],
+                   &b[1]);
+      ghost_b[0][threadIdx.x] = b[0];
+      ghost_b[1][threadIdx.x] = b[1];
+    }
+    __syncthreads();
+  }
+  {
+    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int s = particle_of(first + slot);
+    const bool rows = s >= 0 && !A.kx[s] && A.fbslot[s] == -1;
+    double bG[2] = {0.0, 0.0};
+    if (GH) { bG[0] = ghost_b[0][slot]; bG[1] = ghost_b[1][slot]; }
+    const int sgn[2] = {0, 1};
+    int kb[2];
+    long long H[2][kNB];
+    const bool fits = fx_rhs_rows<2, PER, GH, false, kFxLanes>(
+        A, max(s, 0), rows ? min(A.cnt[s], A.cap) : 0, sub, sgn, bG, H, kb, 0);
+    fx_lanes_store(S, slot, sub, &H[0][0], fits);
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+      if (sub == f) S.kb[f][slot] = kb[f];
+  }
+  __syncthreads();
+  if (threadIdx.x >= kFxSlots) return;
+  const int s = particle_of(first + threadIdx.x);
+  pass2_body<kFixedRows, PER, GH, true>(A, max(s, 0), s >= 0, &S, threadIdx.x);
 }
 
 }  // namespace lp

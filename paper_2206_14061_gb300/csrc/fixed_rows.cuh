@@ -250,35 +250,37 @@ __device__ __forceinline__ int fx_shift(const StepArgs& A, int s, int m) {
 // row does not fit the fixed-point range.
 // rows: the entries with an index in range. SH: offsets are shifted up by sh,
 // which fx_shift chose for the particle's largest one.
-template <bool PER, bool GH, bool SH = false>
-__device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo,
-                                           int* rows, int sh = 0) {
+// P lanes of a particle take every P-th entry each (sub: the lane's first
+// one); the sums are whole numbers, so that adding the lanes' sums gives the
+// bits of one lane taking all (P = 1).
+template <bool PER, bool GH, bool SH, int P>
+__device__ __forceinline__ bool fx_moment_rows(const StepArgs& A, int s, int m, int sub,
+                                               long long* H, int* rows, int sh) {
   const int n = A.n;
   const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
   const StepConsts& K = A.K;
   const uint32_t mask = K.fx_mask;
   FxRec me;
   fx_rec_pos(me, R, s);
-  long long H[31];
 #pragma unroll
   for (int q = 0; q < 31; ++q) H[q] = 0;
   unsigned big = 0;  // the largest magnitude of an offset
   int in_range = m;
   bool bad = !(me.xf == me.xf);
-  uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
-  uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
-  FxPosLoad P;
-  P.fetch(R, code & mask, n, s);
-  for (int k = 0; k < m; ++k) {
+  uint32_t code = sub < m ? (uint32_t)A.nbr[(int64_t)sub * n + s] : 0u;
+  uint32_t nxt = sub + P < m ? (uint32_t)A.nbr[(int64_t)(sub + P) * n + s] : 0u;
+  FxPosLoad X;
+  X.fetch(R, code & mask, n, s);
+  for (int k = sub; k < m; k += P) {
     const uint32_t c0 = code;
     const bool live = (c0 & mask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
     unsigned long long D[3];
-    fx_offsets<PER, SH>(K, sh, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), c0 >> 31, D);
-    bad = bad || (live && !(P.xf() == P.xf()));
-    if (k + 1 < m) {  // (the position is taken: its registers hold the next one)
+    fx_offsets<PER, SH>(K, sh, me, X.xy.x, X.xy.y, X.zf.x, X.xf(), X.yf(), c0 >> 31, D);
+    bad = bad || (live && !(X.xf() == X.xf()));
+    if (k + P < m) {  // (the position is taken: its registers hold the next one)
       code = nxt;
-      P.fetch(R, code & mask, n, s);
-      if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
+      X.fetch(R, code & mask, n, s);
+      if (k + 2 * P < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2 * P) * n + s];
     }
     if (!live) {
       --in_range;
@@ -326,7 +328,11 @@ __device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, doub
     fx_acc(H[30], w[2], q[3]);
   }
   *rows = in_range;
-  if (bad || big > (unsigned)K.fx_lim) return false;
+  return !(bad || big > (unsigned)K.fx_lim);
+}
+template <bool SH>
+__device__ __forceinline__ void fx_moment_values(const StepConsts& K, const long long* H, int sh,
+                                                 double* mo) {
   double g2 = K.fx_g2, g3 = K.fx_g3, g4 = K.fx_g4;
   if (SH) {
     g2 *= pow2_of(-2 * sh);
@@ -338,6 +344,13 @@ __device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, doub
     const double g = t < 6 ? g2 : (t < 16 ? g3 : g4);
     mo[t] = (double)H[t] * g;
   }
+}
+template <bool PER, bool GH, bool SH = false>
+__device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo,
+                                           int* rows, int sh = 0) {
+  long long H[31];
+  if (!fx_moment_rows<PER, GH, SH, 1>(A, s, m, 0, H, rows, sh)) return false;
+  fx_moment_values<SH>(A.K, H, sh, mo);
   return true;
 }
 
@@ -356,9 +369,12 @@ __device__ __forceinline__ void gram_of_moments(const double* mo, double* L) {
 // spacing; sgn: the factor (-1, 0, 1) of a field at a floor mirror; GH: bG is
 // the right-hand side of a flagged entry's ghost row. False: a field does not
 // fit (the caller queues the particle).
-template <int NF, bool PER, bool GH, bool SH = false>
-__device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const int* sgn,
-                                       const double* bG, double (*R9)[kNB], int sh = 0) {
+// kb: the fields' scales. P, sub: as in fx_moment_rows; with P > 1 every lane
+// of the warp must call it.
+template <int NF, bool PER, bool GH, bool SH, int P>
+__device__ __forceinline__ bool fx_rhs_rows(const StepArgs& A, int s, int m, int sub,
+                                            const int* sgn, const double* bG, long long (*H)[kNB],
+                                            int* kb, int sh) {
   const int n = A.n;
   const FxRec* R = reinterpret_cast<const FxRec*>(A.XU);
   const StepConsts& K = A.K;
@@ -377,12 +393,12 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     }
   }
   constexpr int kChunk = 4;
-  for (int k0 = 0; k0 < m; k0 += kChunk) {
+  for (int k0 = sub; k0 < m; k0 += kChunk * P) {
     uint32_t cd[kChunk];
     float4 v[kChunk];
 #pragma unroll
     for (int t = 0; t < kChunk; ++t)
-      cd[t] = k0 + t < m ? (uint32_t)A.nbr[(int64_t)(k0 + t) * n + s] : ~kMirrorBit;
+      cd[t] = k0 + t * P < m ? (uint32_t)A.nbr[(int64_t)(k0 + t * P) * n + s] : ~kMirrorBit;
 #pragma unroll
     for (int t = 0; t < kChunk; ++t) {
       const uint32_t j = cd[t] & mask;
@@ -400,9 +416,14 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       }
     }
   }
+#pragma unroll
+  for (int o = 1; o < P; o <<= 1)
+#pragma unroll
+    for (int f = 0; f < NF; ++f) mx[f] = max(mx[f], __shfl_xor_sync(0xffffffffu, mx[f], o));
   // kb: differences are held as b 2^kb; et: values as v 2^(58 - et), exact for
   // all but values far below the largest; lsh: from the second to the first
-  int kb[NF], et[NF], lsh[NF];
+  int et[NF], lsh[NF];
+  bool fits = true;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     // a bound on the FP64 differences: the FP32 copies err by 2^-24 each
@@ -410,12 +431,16 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     float B = __fmaf_rn(fabsf(mf[f]), 0x1p-22f, d);
     const float V = __fmaf_rn(fabsf(mf[f]), 1.f + 0x1p-20f, d);  // and on the values
     if (GH && K.free_surface) B *= 2.f;  // b +- bG
-    if (!(B < 0x1p120f) || (B > 0.f && B < 0x1p-90f)) return false;
+    fits = fits && B < 0x1p120f && !(B > 0.f && B < 0x1p-90f);
     const int eb = (int)((__float_as_uint(B) + 0x007fffffu) >> 23) - 127;
     const int ev = (int)((__float_as_uint(V) + 0x007fffffu) >> 23) - 127;
     kb[f] = B > 0.f ? 60 - eb : 0;
     et[f] = B > 0.f ? ev : 0;
     lsh[f] = B > 0.f ? ev - eb + 2 : 0;  // (>= 0: B <= 4 V)
+  }
+  if (!fits) {
+    if (P == 1) return false;
+    m = 0;  // (the lanes stay together)
   }
   FxRec me;
   fx_rec_pos(me, R, s);
@@ -425,29 +450,28 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
     U[f] = (unsigned long long)(R[s].m[f] >> min(max(et[f] - R[s].e[f], 0), 63));
     G[f] = GH ? fx_of(bG[f], kb[f]) : 0ull;
   }
-  long long H[NF][kNB];
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
     for (int q = 0; q < kNB; ++q) H[f][q] = 0;
-  uint32_t code = m > 0 ? (uint32_t)A.nbr[s] : 0u;
-  uint32_t nxt = m > 1 ? (uint32_t)A.nbr[(int64_t)n + s] : 0u;
-  FxPosLoad P;
+  uint32_t code = sub < m ? (uint32_t)A.nbr[(int64_t)sub * n + s] : 0u;
+  uint32_t nxt = sub + P < m ? (uint32_t)A.nbr[(int64_t)(sub + P) * n + s] : 0u;
+  FxPosLoad X;
   longlong2 f01, f23;  // m[0], m[1]; m[2], exponents
   auto fetch = [&](uint32_t c) {
     const uint32_t j = c & mask;
-    P.fetch(R, j, n, s);
+    X.fetch(R, j, n, s);
     const longlong2* r = reinterpret_cast<const longlong2*>(&R[j < (uint32_t)n ? j : (uint32_t)s].m[0]);
     f01 = r[0];
     f23 = r[1];
   };
   fetch(code);
-  for (int k = 0; k < m; ++k) {
+  for (int k = sub; k < m; k += P) {
     const uint32_t c0 = code;
     const bool live = (c0 & mask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
     const bool mir = c0 >> 31;
     unsigned long long D[3], u[NF];
-    fx_offsets<PER, SH>(K, sh, me, P.xy.x, P.xy.y, P.zf.x, P.xf(), P.yf(), mir, D);
+    fx_offsets<PER, SH>(K, sh, me, X.xy.x, X.xy.y, X.zf.x, X.xf(), X.yf(), mir, D);
     {
       const long long mj[3] = {f01.x, f01.y, f23.x};
       const int ej[3] = {(int)(short)f23.y, (int)f23.y >> 16, (int)(short)(f23.y >> 32)};
@@ -455,10 +479,10 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       for (int f = 0; f < NF; ++f)
         u[f] = (unsigned long long)(mj[f] >> min(max(et[f] - ej[f], 0), 63));
     }
-    if (k + 1 < m) {
+    if (k + P < m) {
       code = nxt;
       fetch(code);
-      if (k + 2 < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2) * n + s];
+      if (k + 2 * P < m) nxt = (uint32_t)A.nbr[(int64_t)(k + 2 * P) * n + s];
     }
     if (!live) continue;
     if (mir) {
@@ -488,6 +512,11 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       for (int q = 3; q < kNB; ++q) fx_acc(H[f][q], bq, a[q]);
     }
   }
+  return fits;
+}
+template <int NF, bool SH>
+__device__ __forceinline__ void fx_rhs_values(const StepConsts& K, const long long (*H)[kNB],
+                                              const int* kb, int sh, double (*R9)[kNB]) {
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const double ub = pow2_of(32 - kb[f]);
@@ -501,7 +530,58 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
       R9[f][q] = (double)H[f][q] * (q < 3 ? ul : (q < 6 ? 0.5 * uq : uq));
     }
   }
+}
+template <int NF, bool PER, bool GH, bool SH = false>
+__device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const int* sgn,
+                                       const double* bG, double (*R9)[kNB], int sh = 0) {
+  long long H[NF][kNB];
+  int kb[NF];
+  if (!fx_rhs_rows<NF, PER, GH, SH, 1>(A, s, m, 0, sgn, bG, H, kb, sh)) return false;
+  fx_rhs_values<NF, SH>(A.K, H, kb, sh, R9);
   return true;
+}
+
+// Runs with few particles: kFxLanes lanes to a particle for the rows; the
+// block's first warp then takes a particle a lane for what follows them.
+constexpr int kFxLanes = 4;
+constexpr int kFxSlots = 32;  // particles of a block of kFxLanes * 32 threads
+template <int NV>
+struct FxShared {
+  long long H[NV][kFxSlots];
+  int kb[3][kFxSlots];
+  int fits[kFxSlots];
+};
+// the lanes' sums added (whole numbers), to column slot of the shared ones
+template <int NV>
+__device__ __forceinline__ void fx_lanes_store(FxShared<NV>& S, int slot, int sub, long long* H,
+                                               bool fits) {
+  int ok = fits;
+#pragma unroll
+  for (int o = 1; o < kFxLanes; o <<= 1) ok &= __shfl_xor_sync(0xffffffffu, ok, o);
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    long long v = H[q];
+#pragma unroll
+    for (int o = 1; o < kFxLanes; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (q % kFxLanes == sub) S.H[q][slot] = v;
+  }
+  if (sub == 0) S.fits[slot] = ok;
+}
+
+// right-hand sides from a column of the shared sums
+template <int NV>
+__device__ __forceinline__ void fx_shared_values(const StepConsts& K, const FxShared<NV>& S,
+                                                 int col, double (*R9)[kNB]) {
+  constexpr int NF = NV / kNB;
+  long long H[NF][kNB];
+  int kb[NF];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    kb[f] = S.kb[f][col];
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) H[f][q] = S.H[f * kNB + q][col];
+  }
+  fx_rhs_values<NF, false>(K, H, kb, 0, R9);
 }
 
 }  // namespace lp
