@@ -223,9 +223,9 @@ def pass1_work(prec: str, rows: float, n: int):
     """Instructions one pass-1 phase issues in its own pipe, and that pipe's
     peak (a utilisation figure; the method's own flops are pass1_method_flops).
 
-    FP64 (flops, FMA = 2): per stencil row 6 (offsets) + 6 (quadratic terms) +
-    62 (31 moments) + 3 (differences) + 54 (3 right-hand sides x 9) = 131; per
-    particle about 1000 (9x9 Cholesky, three solves, derived quantities).
+    FP64 (flops, FMA = 2): the stencil rows run in 64-bit fixed point on the
+    integer and FP32 pipes; per particle about 1000 (9x9 Cholesky, three
+    solves, derived quantities).
     MIXED (FP64 flops only; the FP32 moments run on the FP32 pipe): per row 6 +
     9 + 3 + 54 (residual) + 54 (A^T r) = 126; per particle about 550.
     MIXED_FF (FP32 lane operations: every FP32 add, multiply or FMA is one op,
@@ -237,12 +237,12 @@ def pass1_work(prec: str, rows: float, n: int):
     if prec == "mixed_ff":
         return (792.0 * rows + 5331.0 * n, "T FP32 lane-ops/s", FP32_PEAK_TOPS,
                 "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz")
-    flops = 131.0 * rows + 1000.0 * n if prec == "fp64" else 126.0 * rows + 550.0 * n
+    flops = 1000.0 * n if prec == "fp64" else 126.0 * rows + 550.0 * n
     return (flops, "TFLOP/s (FP64)", FP64_PEAK_TFLOPS,
             "nominal FP64 rate (no measured FP64 peak in MEASURED_PEAKS.json)")
 
 
-PASS1_KERNELS = {"mixed_ff": "k_gram_ff + k_pass1_ff_rows + k_pass1_ff_solve", "mixed": "k_pass1", "fp64": "k_pass1"}
+PASS1_KERNELS = {"mixed_ff": "k_gram_ff + k_pass1_ff_rows + k_pass1_ff_solve", "mixed": "k_pass1", "fp64": "k_gram_fx + k_pass1_fx"}
 
 
 def our_arm(args):

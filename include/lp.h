@@ -52,7 +52,10 @@ typedef int32_t lp_status;
 #define LP_ERR_UNIMPLEMENTED 7
 
 /* arithmetic of the least-squares fits */
-#define LP_FP64 0  /* FP64 moments, Cholesky and solve (QR fallback in FP64)   */
+#define LP_FP64 0  /* FP64 results: moments and right-hand sides summed in 64- */
+                   /* bit fixed point (terms err by 2^-54 of the largest; FP64 */
+                   /* rows where the range does not hold), Cholesky, solve and */
+                   /* QR fallback in FP64                                      */
 #define LP_MIXED 1 /* FP32 moments and Cholesky + one FP64 refinement step     */
 #define LP_MIXED_FF 2 /* FP32 only on the stencil rows: offsets, moments and   */
                       /* right-hand sides accumulated as float-float (FP32     */
