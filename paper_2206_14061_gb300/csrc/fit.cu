@@ -128,13 +128,16 @@ __global__ void __launch_bounds__(kFxBlock, WIDE ? 4 : 3) k_pass2_fx(const StepA
   const int s = fit_particle(A);
   pass2_body<kFixedRows, PER, GH>(A, s, s < A.n);
 }
-// Few particles: four lanes to a particle (k_*_fx_lanes). 8,000 particles, one
-// thread each, are 250 warps, fewer than the chip has schedulers, and each row
-// waits for its gathers; four lanes take a quarter of the rows each. Four
-// LP_FP64 steps with a thread and with four lanes each: 512 particles 869 and
-// 715 us, 2,744 908 and 746, 8,000 939 and 786, 17,000 956 and 1039, 26,000
-// 1074 and 1102. The line: what one wave of the lanes' blocks takes, 3 per SM.
-constexpr int kFxSplit = 3 * 152 * kFxSlots;
+// Few particles: four or two lanes to a particle (k_*_fx_lanes). 8,000
+// particles, one thread each, are 250 warps, fewer than the chip has
+// schedulers, and each row waits for its gathers; the lanes take a quarter or
+// half of the rows each. Four LP_FP64 steps with a thread, two and four lanes
+// each (us): 512 particles 869, -, 715; 8,000 939, -, 786; 14,000 -, 831, 822;
+// 17,000 959, 890, 1039; 22,000 1059, 992, -; 26,000 1084, 1036, 1102; 31,000
+// 1138, 1246, -. The lines: what one wave of the lanes' blocks takes at 12
+// warps per SM.
+constexpr int kFxSplit4 = 3 * 152 * kFxSlots;
+constexpr int kFxSplit2 = 6 * 152 * kFxSlots;
 // (particle of rank t, or -1)
 struct FxParticles {
   const StepArgs& A;
@@ -142,36 +145,42 @@ struct FxParticles {
     return t < A.n ? (A.perm ? A.perm[t] : t) : -1;
   }
 };
-template <bool PER, bool GH>
-__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_gram_fx_lanes(const StepArgs A) {
-  gram_fx_lanes<PER, GH>(A, FxParticles{A});
+template <bool PER, bool GH, int P>
+__global__ void __launch_bounds__(P * kFxSlots, 12 / P) k_gram_fx_lanes(const StepArgs A) {
+  gram_fx_lanes<PER, GH, P>(A, FxParticles{A});
 }
-template <bool PER>
-__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_pass1_fx_lanes(const StepArgs A) {
-  pass1_fx_lanes<PER>(A, FxParticles{A});
+template <bool PER, int P>
+__global__ void __launch_bounds__(P * kFxSlots, 12 / P) k_pass1_fx_lanes(const StepArgs A) {
+  pass1_fx_lanes<PER, P>(A, FxParticles{A});
 }
-template <bool PER, bool GH>
-__global__ void __launch_bounds__(kFxLanes * kFxSlots, 3) k_pass2_fx_lanes(const StepArgs A) {
-  pass2_fx_lanes<PER, GH>(A, FxParticles{A});
+template <bool PER, bool GH, int P>
+__global__ void __launch_bounds__(P * kFxSlots, 12 / P) k_pass2_fx_lanes(const StepArgs A) {
+  pass2_fx_lanes<PER, GH, P>(A, FxParticles{A});
 }
 int fx_lane_blocks(int n) { return (n + kFxSlots - 1) / kFxSlots; }
 template <bool PER, bool GH>
 void launch_gram_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
-  if (A.n <= kFxSplit)
-    k_gram_fx_lanes<PER, GH><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  if (A.n <= kFxSplit4)
+    k_gram_fx_lanes<PER, GH, 4><<<fx_lane_blocks(A.n), 4 * kFxSlots, 0, st>>>(A);
+  else if (A.n <= kFxSplit2)
+    k_gram_fx_lanes<PER, GH, 2><<<fx_lane_blocks(A.n), 2 * kFxSlots, 0, st>>>(A);
   else if (A.n > kFxWide) k_gram_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
   else k_gram_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
 }
 template <bool PER>
 void launch_pass1_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
-  if (A.n <= kFxSplit)
-    k_pass1_fx_lanes<PER><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  if (A.n <= kFxSplit4)
+    k_pass1_fx_lanes<PER, 4><<<fx_lane_blocks(A.n), 4 * kFxSlots, 0, st>>>(A);
+  else if (A.n <= kFxSplit2)
+    k_pass1_fx_lanes<PER, 2><<<fx_lane_blocks(A.n), 2 * kFxSlots, 0, st>>>(A);
   else k_pass1_fx<PER><<<nf, b, 0, st>>>(A);
 }
 template <bool PER, bool GH>
 void launch_pass2_fx(const StepArgs& A, int nf, int b, cudaStream_t st) {
-  if (A.n <= kFxSplit)
-    k_pass2_fx_lanes<PER, GH><<<fx_lane_blocks(A.n), kFxLanes * kFxSlots, 0, st>>>(A);
+  if (A.n <= kFxSplit4)
+    k_pass2_fx_lanes<PER, GH, 4><<<fx_lane_blocks(A.n), 4 * kFxSlots, 0, st>>>(A);
+  else if (A.n <= kFxSplit2)
+    k_pass2_fx_lanes<PER, GH, 2><<<fx_lane_blocks(A.n), 2 * kFxSlots, 0, st>>>(A);
   else if (A.n > kFxWide) k_pass2_fx<PER, GH, true><<<nf, b, 0, st>>>(A);
   else k_pass2_fx<PER, GH, false><<<nf, b, 0, st>>>(A);
 }

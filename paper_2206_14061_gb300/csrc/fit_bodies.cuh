@@ -276,19 +276,19 @@ __device__ __forceinline__ void gram_fx_body(const StepArgs& A, int s) {
   const bool fits = fx_moments<PER, GH>(A, s, m, mo, &rows);
   gram_fx_finish(A, s, m, fits, mo);
 }
-// the same with the rows taken by kFxLanes lanes (a block of kFxLanes * 32
+// the same with the rows taken by P lanes (a block of P * 32
 // threads calls it; particle_of(t): the particle of rank t, or -1)
-template <bool PER, bool GH, class F>
+template <bool PER, bool GH, int P, class F>
 __device__ __forceinline__ void gram_fx_lanes(const StepArgs& A, F particle_of) {
   __shared__ FxShared<31> S;
   {
-    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int slot = threadIdx.x / P, sub = threadIdx.x % P;
     const int s = particle_of(blockIdx.x * kFxSlots + slot);
     long long H[31];
     int rows;
-    const bool fits = fx_moment_rows<PER, GH, false, kFxLanes>(
+    const bool fits = fx_moment_rows<PER, GH, false, P>(
         A, max(s, 0), s >= 0 ? min(A.cnt[s], A.cap) : 0, sub, H, &rows, 0);
-    fx_lanes_store(S, slot, sub, H, fits);
+    fx_lanes_store<P>(S, slot, sub, H, fits);
   }
   __syncthreads();
   if (threadIdx.x >= kFxSlots) return;
@@ -338,22 +338,22 @@ __device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
   }
   pass1_fx_finish(A, s, R);
 }
-template <bool PER, class F>
+template <bool PER, int P, class F>
 __device__ __forceinline__ void pass1_fx_lanes(const StepArgs& A, F particle_of) {
   __shared__ FxShared<3 * kNB> S;
   auto has_rows = [&](int s) { return s >= 0 && !A.kx[s] && A.fbslot[s] == -1; };
   {
-    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int slot = threadIdx.x / P, sub = threadIdx.x % P;
     const int s = particle_of(blockIdx.x * kFxSlots + slot);
     int sgn[3], kb[3];
     pass1_signs(A, sgn);
     long long H[3][kNB];
-    const bool fits = fx_rhs_rows<3, PER, false, false, kFxLanes>(
+    const bool fits = fx_rhs_rows<3, PER, false, false, P>(
         A, max(s, 0), has_rows(s) ? min(A.cnt[s], A.cap) : 0, sub, sgn, nullptr, H, kb, 0);
-    fx_lanes_store(S, slot, sub, &H[0][0], fits);
+    fx_lanes_store<P>(S, slot, sub, &H[0][0], fits);
 #pragma unroll
     for (int f = 0; f < 3; ++f)
-      if (sub == f) S.kb[f][slot] = kb[f];
+      if (sub == f % P) S.kb[f][slot] = kb[f];
   }
   __syncthreads();
   if (threadIdx.x >= kFxSlots) return;
@@ -1419,8 +1419,8 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live,
   if (live && nonfin) atomicOr(&A.dg->flags, (unsigned)LP_FLAG_NONFINITE);
   if (live && below) atomicOr(&A.dg->flags, (unsigned)LP_FLAG_BELOW_FLOOR);
 }
-// LP_FP64 with the rows taken by kFxLanes lanes (as gram_fx_lanes)
-template <bool PER, bool GH, class F>
+// LP_FP64 with the rows taken by P lanes (as gram_fx_lanes)
+template <bool PER, bool GH, int P, class F>
 __device__ __forceinline__ void pass2_fx_lanes(const StepArgs& A, F particle_of) {
   __shared__ FxShared<2 * kNB> S;
   __shared__ double ghost_b[2][kFxSlots];
@@ -1438,7 +1438,7 @@ __device__ __forceinline__ void pass2_fx_lanes(const StepArgs& A, F particle_of)
     __syncthreads();
   }
   {
-    const int slot = threadIdx.x / kFxLanes, sub = threadIdx.x % kFxLanes;
+    const int slot = threadIdx.x / P, sub = threadIdx.x % P;
     const int s = particle_of(first + slot);
     const bool rows = s >= 0 && !A.kx[s] && A.fbslot[s] == -1;
     double bG[2] = {0.0, 0.0};
@@ -1446,9 +1446,9 @@ __device__ __forceinline__ void pass2_fx_lanes(const StepArgs& A, F particle_of)
     const int sgn[2] = {0, 1};
     int kb[2];
     long long H[2][kNB];
-    const bool fits = fx_rhs_rows<2, PER, GH, false, kFxLanes>(
+    const bool fits = fx_rhs_rows<2, PER, GH, false, P>(
         A, max(s, 0), rows ? min(A.cnt[s], A.cap) : 0, sub, sgn, bG, H, kb, 0);
-    fx_lanes_store(S, slot, sub, &H[0][0], fits);
+    fx_lanes_store<P>(S, slot, sub, &H[0][0], fits);
 #pragma unroll
     for (int f = 0; f < 2; ++f)
       if (sub == f) S.kb[f][slot] = kb[f];

@@ -541,10 +541,9 @@ __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const in
   return true;
 }
 
-// Runs with few particles: kFxLanes lanes to a particle for the rows; the
-// block's first warp then takes a particle a lane for what follows them.
-constexpr int kFxLanes = 4;
-constexpr int kFxSlots = 32;  // particles of a block of kFxLanes * 32 threads
+// Runs with few particles: P lanes to a particle for the rows; the block's
+// first warp then takes a particle a lane for what follows them.
+constexpr int kFxSlots = 32;  // particles of a block of P * 32 threads
 template <int NV>
 struct FxShared {
   long long H[NV][kFxSlots];
@@ -552,18 +551,18 @@ struct FxShared {
   int fits[kFxSlots];
 };
 // the lanes' sums added (whole numbers), to column slot of the shared ones
-template <int NV>
+template <int P, int NV>
 __device__ __forceinline__ void fx_lanes_store(FxShared<NV>& S, int slot, int sub, long long* H,
                                                bool fits) {
   int ok = fits;
 #pragma unroll
-  for (int o = 1; o < kFxLanes; o <<= 1) ok &= __shfl_xor_sync(0xffffffffu, ok, o);
+  for (int o = 1; o < P; o <<= 1) ok &= __shfl_xor_sync(0xffffffffu, ok, o);
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
     long long v = H[q];
 #pragma unroll
-    for (int o = 1; o < kFxLanes; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (q % kFxLanes == sub) S.H[q][slot] = v;
+    for (int o = 1; o < P; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (q % P == sub) S.H[q][slot] = v;
   }
   if (sub == 0) S.fits[slot] = ok;
 }

@@ -1,8 +1,8 @@
 """The fixed-point rows of LP_FP64, the ghost lanes and the truncated stencils
 at the edges of their launch shapes.
 
-Whole-number sums do not depend on who adds them: the per-phase kernels (four
-lanes, three or four blocks per SM by particle count) give the bits of the
+Whole-number sums do not depend on who adds them: the per-phase kernels (four or
+two lanes, three or four blocks per SM by particle count) give the bits of the
 persistent launch, which takes one thread per particle throughout.
 """
 import numpy as np
@@ -31,7 +31,7 @@ def T(a):
 
 
 @pytest.mark.parametrize("ghosts", [0, 1])
-@pytest.mark.parametrize("n", [1, 31, 33, 129, 14592, 14593, 58368, 58369])
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 14592, 14593, 29184, 29185, 58368, 58369])
 def test_step_bits_do_not_depend_on_the_row_split(capi, n, ghosts):
     wl = W.cube(next(s for s in (6, 25, 39) if s ** 3 >= n))
     pd = W.param_dict(wl)
