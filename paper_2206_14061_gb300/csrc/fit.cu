@@ -93,9 +93,10 @@ __device__ __forceinline__ int fit_particle(const StepArgs& A) {
 }
 
 // FP64 with fixed-point rows (fixed_rows.cuh). 786,000 particles, per step:
-// moments and factor 0.71 ms, right-hand sides and solves 0.97 ms, pass 2
-// 0.85 ms; with the rows in FP64, on whose pipe they were bound (91 % busy),
-// pass 1 took 5.58 and pass 2 2.66 ms. 3 blocks of 128 threads at 168
+// moments and factor 0.58 ms, right-hand sides and solves 0.77 ms, pass 2
+// 0.64 ms; with the rows in FP64, on whose pipe they were bound (91 % busy),
+// pass 1 took 5.58 and pass 2 2.66 ms. Now the FP64 pipe (factor, solves,
+// closure) is 57 % busy and the warps issue in 0.40 to 0.44 of the cycles. 3 blocks of 128 threads at 168
 // registers, or WIDE: 4 blocks at 128 registers, whose few spilled values (8
 // to 156 bytes a thread) cost less than the fourth block gives once there are
 // more particles than 3 blocks per SM take at a time. LP_FP64 steps with 3 and
