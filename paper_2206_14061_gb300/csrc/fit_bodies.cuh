@@ -299,7 +299,7 @@ __device__ __forceinline__ void gram_fx_lanes(const StepArgs& A, F particle_of) 
   for (int q = 0; q < 31; ++q) H[q] = S.H[q][threadIdx.x];
   double mo[31];
   fx_moment_values<false>(A.K, H, 0, mo);
-  gram_fx_finish(A, s, min(A.cnt[s], A.cap), S.fits[threadIdx.x], mo);
+  gram_fx_finish(A, s, min(A.cnt[s], A.cap), S.fits[threadIdx.x] && fx_resolved(H), mo);
 }
 
 __device__ __forceinline__ void pass1_fx_finish(const StepArgs& A, int s, double (*R)[kNB]) {

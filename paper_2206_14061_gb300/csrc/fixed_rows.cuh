@@ -28,7 +28,8 @@
 // copies.
 //
 // What does not fit (offsets beyond about the radius, which only stencils held
-// fixed over several steps can have; fields whose differences are not finite
+// fixed over several steps can have; stencils thin along an axis or small
+// against the radius, see fx_resolved; fields whose differences are not finite
 // or are below 2^-90; non-finite positions) is queued for a kernel that runs
 // the plain FP64 rows.
 #pragma once
@@ -330,6 +331,24 @@ __device__ __forceinline__ bool fx_moment_rows(const StepArgs& A, int s, int m, 
   *rows = in_range;
   return !(bad || big > (unsigned)K.fx_lim);
 }
+// The error of a sum is a few units per row whatever its value (a term errs by
+// up to 2^5 units, 2^2 typically), so a stencil thin along an axis, or small
+// against the radius, has sums with few good bits: with one axis compressed to
+// 0.1 the derivatives err by 5e-12 of the largest instead of 3e-15, at 0.01 by
+// 5e-8, and no relative pivot shows it, as those do not depend on the columns'
+// scale. False if the squared length of a quadratic column is below 2^50 units;
+// the particle then takes the plain rows. At the line errors are two to three
+// times those of FP64 rows (1.2e-15 and 4e-16 rms of the largest derivative on
+// a lattice compressed to 0.35; 2e-14 and 9e-15 in a corner of one). The least
+// such length of a jittered lattice at the usual radius of 2.2 spacings: 2^53
+// in the bulk, 2^50.4 in corners, where the radius is least favourable to its
+// power of two. (The linear columns are at least as well resolved.)
+constexpr int kFxLeastBits = 50;
+__device__ __forceinline__ bool fx_resolved(const long long* H) {
+  long long least = min(min(H[16], H[17]), H[18]);
+  least = min(least, min(min(H[25], H[26]), H[27]));
+  return least >= 1ll << kFxLeastBits;
+}
 template <bool SH>
 __device__ __forceinline__ void fx_moment_values(const StepConsts& K, const long long* H, int sh,
                                                  double* mo) {
@@ -349,7 +368,7 @@ template <bool PER, bool GH, bool SH = false>
 __device__ __forceinline__ bool fx_moments(const StepArgs& A, int s, int m, double* mo,
                                            int* rows, int sh = 0) {
   long long H[31];
-  if (!fx_moment_rows<PER, GH, SH, 1>(A, s, m, 0, H, rows, sh)) return false;
+  if (!fx_moment_rows<PER, GH, SH, 1>(A, s, m, 0, H, rows, sh) || !fx_resolved(H)) return false;
   fx_moment_values<SH>(A.K, H, sh, mo);
   return true;
 }
