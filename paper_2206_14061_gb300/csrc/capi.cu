@@ -691,8 +691,9 @@ void fixed_consts(StepConsts& K, bool shifted = false) {
   K.fx_F2 = fx_of(2.0 * K.floor_z, K.fx_k);
   K.fx_Lx = fx_of(K.Lx, K.fx_k);
   K.fx_Ly = fx_of(K.Ly, K.fx_k);
-  K.fx_hLx = K.Lx > 0.0 ? (float)(0.5 * K.Lx) : INFINITY;
-  K.fx_hLy = K.Ly > 0.0 ? (float)(0.5 * K.Ly) : INFINITY;
+  K.fx_turn = std::ldexp(1.0, K.fx_k - 64);
+  K.fx_hLx = K.Lx > 0.0 ? (float)(0.5 * K.Lx * K.fx_turn) : INFINITY;
+  K.fx_hLy = K.Ly > 0.0 ? (float)(0.5 * K.Ly * K.fx_turn) : INFINITY;
 }
 
 }  // namespace
@@ -1059,6 +1060,7 @@ lp_status lp_fit_derivatives(lp_ctx* c, const lp_particles* p, const lp_neighbor
     A.n = F.n; A.cap = F.cap; A.nbr = F.nbr; A.cnt = F.cnt;
     A.XU = c->XU; A.fs = c->fs; A.slow = c->slow; A.slow_count = c->fb_count + 1; A.kx = c->kx;
     A.fac = c->fac; A.dg = c->dg;
+    A.x = F.x; A.y = F.y; A.z = F.z;
     A.K.inv_h = F.inv_h;
     A.K.floor_z = floor_z;
     A.K.radius = nb->nbr == c->nbr_o && c->nbr_rmax > 0.0 ? c->nbr_rmax : 4.0 * h;

@@ -390,7 +390,7 @@ __global__ void k_fit_fx_split(const FitArgs F, const StepArgs A) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= F.n) return;
   FxRec* R = reinterpret_cast<FxRec*>(A.XU);
-  fx_position(F.x[s], F.y[s], F.z[s], A.K.fx_k, R[s]);
+  fx_position(A, F.x[s], F.y[s], F.z[s], R[s]);
 }
 __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, const StepArgs A) {
   const int s = fit_thread(F);
@@ -432,14 +432,14 @@ __global__ void k_fit_fx_fields(const FitArgs F, const StepArgs A, int f0) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= F.n) return;
   FxRec& r = reinterpret_cast<FxRec*>(A.XU)[s];
-  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  float v[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const double w = F.fields[f0 + f][s];
     fx_field(w, &r.m[f], &r.e[f]);
     v[f] = fx_float(w);
   }
-  A.fs[s] = make_float4(v[0], v[1], v[2], v[3]);
+  A.fs[s] = make_float4(v[0], v[1], v[2], fx_coarse(F.z[s], fx_ref(A).z, A.K.fx_turn));
 }
 template <int NF>
 __global__ void __launch_bounds__(kFxBlock, 3) k_fit_rhs_fx(const FitArgs F, const StepArgs A,
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_rhs_fx(const FitArgs F, con
 #pragma unroll
   for (int f = 0; f < NF; ++f) sgn[f] = (int)F.msign[f0 + f];
   double R[NF][kNB];
-  if (!fx_rhs<NF, false, false, true>(A, s, m, sgn, nullptr, R, sh)) {
+  if (!fx_rhs<NF, false, false, true, true>(A, s, m, sgn, nullptr, R, sh)) {
     A.kx[s] = kFxSlow;  // (all of its fields)
     fx_push(A, s, 0);
     return;

@@ -332,7 +332,8 @@ __device__ __forceinline__ void pass1_fx_body(const StepArgs& A, int s) {
   int sgn[3];
   pass1_signs(A, sgn);
   double R[3][kNB];
-  if (!fx_rhs<3, PER, false>(A, s, min(A.cnt[s], A.cap), sgn, nullptr, R)) {
+  if (!fx_rhs<3, PER, false, true>(A, s, min(A.cnt[s], A.cap), sgn, nullptr, R)) {
+    A.kx[s] = 1;  // (in pass 2 as well)
     fx_push(A, s, 0);
     return;
   }
@@ -348,7 +349,7 @@ __device__ __forceinline__ void pass1_fx_lanes(const StepArgs& A, F particle_of)
     int sgn[3], kb[3];
     pass1_signs(A, sgn);
     long long H[3][kNB];
-    const bool fits = fx_rhs_rows<3, PER, false, false, P>(
+    const bool fits = fx_rhs_rows<3, PER, false, false, true, P>(
         A, max(s, 0), has_rows(s) ? min(A.cnt[s], A.cap) : 0, sub, sgn, nullptr, H, kb, 0);
     fx_lanes_store<P>(S, slot, sub, &H[0][0], fits);
 #pragma unroll
@@ -360,6 +361,7 @@ __device__ __forceinline__ void pass1_fx_lanes(const StepArgs& A, F particle_of)
   const int s = particle_of(blockIdx.x * kFxSlots + threadIdx.x);
   if (!has_rows(s)) return;
   if (!S.fits[threadIdx.x]) {
+    A.kx[s] = 1;  // (in pass 2 as well)
     fx_push(A, s, 0);
     return;
   }
@@ -1176,7 +1178,7 @@ __device__ __forceinline__ void pass2_body(const StepArgs& A, int s, bool live,
         } else {
           if (GH && A.K.free_surface) ghost_rhs2(A, gni, Vi, &bG[0], &bG[1]);
           const int sgn[2] = {0, 1};
-          fits = fx_rhs<2, PER, GH>(A, s, m, sgn, bG, R);
+          fits = fx_rhs<2, PER, GH, false>(A, s, m, sgn, bG, R);
         }
         if (!fits) {  // plain FP64 rows
           fx_push(A, s, 1);
@@ -1446,7 +1448,7 @@ __device__ __forceinline__ void pass2_fx_lanes(const StepArgs& A, F particle_of)
     const int sgn[2] = {0, 1};
     int kb[2];
     long long H[2][kNB];
-    const bool fits = fx_rhs_rows<2, PER, GH, false, P>(
+    const bool fits = fx_rhs_rows<2, PER, GH, false, false, P>(
         A, max(s, 0), rows ? min(A.cnt[s], A.cap) : 0, sub, sgn, bG, H, kb, 0);
     fx_lanes_store<P>(S, slot, sub, &H[0][0], fits);
 #pragma unroll

@@ -22,13 +22,15 @@
 // Positions are integers X = x 2^k modulo 2^64, with r 2^k in (2^59, 2^60]
 // for the stencil radius r: the conversion is exact for all but the last bits
 // of tiny coordinates, and differences of neighbours are exact whatever the
-// distance from the origin (the modular wrap cancels). Field values (u, v, w;
+// distance from the origin (the modular wrap cancels). As entries of a stencil
+// may be anywhere (held stencils, a caller's own lists), the offsets are also
+// taken in FP32 in units of the wrap, to see one that only looks near. Field values (u, v, w;
 // |gdot|, V) are aligned per stencil to its largest value, and their differences
 // shifted up to fill the range; the scales come from a first walk over FP32
 // copies.
 //
 // What does not fit (offsets beyond about the radius, which only stencils held
-// fixed over several steps can have; stencils thin along an axis or small
+// fixed over several steps or a caller's own can have; stencils thin along an axis or small
 // against the radius, see fx_resolved; fields whose differences are not finite
 // or are below 2^-90; non-finite positions) is queued for a kernel that runs
 // the plain FP64 rows.
@@ -56,8 +58,9 @@ __host__ __device__ __forceinline__ unsigned long long fx_of(double v, int k) {
   return (b >> 63) ? 0ull - r : r;
 }
 
-// One particle of the rows: fixed-point position (with the FP32 coordinates
-// that choose the nearest image; xf is NaN for a non-finite position) and the
+// One particle of the rows: fixed-point position (with the coarse coordinates,
+// see fx_coarse, that choose the nearest image and tell far entries; xf is NaN
+// if one of the three is) and the
 // field values of the pass as signed significands (53 bits, the top one at bit
 // 58) with their exponents, so that a row aligns a value to its stencil's scale
 // with one shift. A value is m 2^(e - 58).
@@ -110,29 +113,48 @@ __device__ __forceinline__ void fx_acc(long long& H, const FxV& a, const FxV& b)
   const int c = __float2int_rn(__fmaf_rn(a.l, b.hf, __fmul_rn(a.hf, b.l)));
   H = fx_mad(a.h, b.h, H) + (long long)c;
 }
+// A coordinate in units of the wrap 2^(64 - k), from that of the first
+// particle; NaN from 2^20 on. Its errors (the rounding of both coordinates of
+// a difference, and of the mirror plane) are below 0.16, so a difference below
+// kFxNear is one of less than half a wrap, and every offset that the range
+// takes (1/14 of a wrap) is below it.
+constexpr float kFxNear = 0.25f;
+__device__ __forceinline__ float fx_coarse(double v, double ref, double turn) {
+  const float c = __double2float_rn(__dmul_rn(__dsub_rn(v, ref), turn));
+  return fabsf(c) < 0x1p20f ? c : __int_as_float(0x7fffffff);
+}
 __device__ __forceinline__ double pow2_of(int e) {  // 2^e, a normal double
   return __longlong_as_double((long long)(1023 + e) << 52);
 }
 
 // offsets of entry j of a particle at `me` (PER: nearest images)
-// (SH: shifted up by sh)
+// (SH: shifted up by sh). True if the entry is near along x and y: the offsets
+// are below half a wrap, so the fixed-point ones are the true ones. (Along z:
+// fx_rhs_rows, from the copy that its first walk reads anyway.)
 template <bool PER, bool SH>
-__device__ __forceinline__ void fx_offsets(const StepConsts& K, int sh, const FxRec& me,
+__device__ __forceinline__ bool fx_offsets(const StepConsts& K, int sh, const FxRec& me,
                                            unsigned long long Xj, unsigned long long Yj,
                                            unsigned long long Zj, float xf, float yf, bool mir,
                                            unsigned long long* D) {
   D[0] = Xj - me.X;
   D[1] = Yj - me.Y;
   D[2] = (mir ? K.fx_F2 - Zj : Zj) - me.Z;
+  float dx = xf - me.xf, dy = yf - me.yf;
   if (PER) {
-    const float dx = xf - me.xf, dy = yf - me.yf;
-    if (fabsf(dx) > K.fx_hLx) D[0] -= dx > 0.f ? K.fx_Lx : 0ull - K.fx_Lx;
-    if (fabsf(dy) > K.fx_hLy) D[1] -= dy > 0.f ? K.fx_Ly : 0ull - K.fx_Ly;
+    if (fabsf(dx) > K.fx_hLx) {
+      D[0] -= dx > 0.f ? K.fx_Lx : 0ull - K.fx_Lx;
+      dx -= copysignf(2.f * K.fx_hLx, dx);
+    }
+    if (fabsf(dy) > K.fx_hLy) {
+      D[1] -= dy > 0.f ? K.fx_Ly : 0ull - K.fx_Ly;
+      dy -= copysignf(2.f * K.fx_hLy, dy);
+    }
   }
   if (SH) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) D[a] <<= sh;
   }
+  return fabsf(dx) < kFxNear && fabsf(dy) < kFxNear;  // (false for NaN)
 }
 
 // row loop state: the neighbour's position one row ahead, its code two rows ahead
@@ -170,25 +192,40 @@ __device__ __forceinline__ float fx_float(double v) {
   return (fabsf(f) < 0x1p-100f && (b << 1)) ? copysignf(0x1p-100f, (b >> 63) ? -1.f : 1.f) : f;
 }
 
-// the position half of a record
-__device__ __forceinline__ void fx_position(double x, double y, double z, int k, FxRec& r) {
+// the first particle's coordinates (0 for one that is not finite)
+struct FxRef {
+  double x, y, z;
+};
+__device__ __forceinline__ FxRef fx_ref(const StepArgs& A) {
+  FxRef o{A.x[0], A.y[0], A.z[0]};
+  if (!isfinite(o.x)) o.x = 0.0;
+  if (!isfinite(o.y)) o.y = 0.0;
+  if (!isfinite(o.z)) o.z = 0.0;
+  return o;
+}
+// the position half of a record; the z's coarse coordinate is returned
+__device__ __forceinline__ float fx_position(const StepArgs& A, double x, double y, double z,
+                                             FxRec& r) {
+  const int k = A.K.fx_k;
   r.X = fx_of(x, k); r.Y = fx_of(y, k); r.Z = fx_of(z, k);
-  const bool fin = isfinite(x) && isfinite(y) && isfinite(z);
-  r.xf = fin ? __double2float_rn(x) : __int_as_float(0x7fffffff);
-  r.yf = __double2float_rn(y);
+  const FxRef o = fx_ref(A);
+  const float xf = fx_coarse(x, o.x, A.K.fx_turn), zf = fx_coarse(z, o.z, A.K.fx_turn);
+  r.yf = fx_coarse(y, o.y, A.K.fx_turn);
+  r.xf = r.yf == r.yf && zf == zf ? xf : r.yf + zf;
+  return zf;
 }
 // records of pass 1: positions, u, v, w
 __device__ __forceinline__ void fx_split_state_body(const StepArgs& A, int s) {
   FxRec* R = reinterpret_cast<FxRec*>(A.XU);
   FxRec r;
-  fx_position(A.x[s], A.y[s], A.z[s], A.K.fx_k, r);
+  const float zf = fx_position(A, A.x[s], A.y[s], A.z[s], r);
   const double u = A.u[s], v = A.v[s], w = A.w[s];
   fx_field(u, &r.m[0], &r.e[0]);
   fx_field(v, &r.m[1], &r.e[1]);
   fx_field(w, &r.m[2], &r.e[2]);
   r.e[3] = 0;
   R[s] = r;
-  A.fs[s] = make_float4(fx_float(u), fx_float(v), fx_float(w), 0.f);
+  A.fs[s] = make_float4(fx_float(u), fx_float(v), fx_float(w), zf);
 }
 // fields of pass 2: |gdot|^n and the V of its fit
 __device__ __forceinline__ void fx_split_p1_body(const StepArgs& A, int s) {
@@ -276,8 +313,9 @@ __device__ __forceinline__ bool fx_moment_rows(const StepArgs& A, int s, int m, 
     const uint32_t c0 = code;
     const bool live = (c0 & mask) < (uint32_t)n;  // (else: stale or corrupt stencil entry)
     unsigned long long D[3];
-    fx_offsets<PER, SH>(K, sh, me, X.xy.x, X.xy.y, X.zf.x, X.xf(), X.yf(), c0 >> 31, D);
-    bad = bad || (live && !(X.xf() == X.xf()));
+    const bool near =
+        fx_offsets<PER, SH>(K, sh, me, X.xy.x, X.xy.y, X.zf.x, X.xf(), X.yf(), c0 >> 31, D);
+    bad = bad || (live && !near);
     if (k + P < m) {  // (the position is taken: its registers hold the next one)
       code = nxt;
       X.fetch(R, code & mask, n, s);
@@ -389,8 +427,9 @@ __device__ __forceinline__ void gram_of_moments(const double* mo, double* L) {
 // the right-hand side of a flagged entry's ghost row. False: a field does not
 // fit (the caller queues the particle).
 // kb: the fields' scales. P, sub: as in fx_moment_rows; with P > 1 every lane
-// of the warp must call it.
-template <int NF, bool PER, bool GH, bool SH, int P>
+// of the warp must call it. ZC: the copies of the fields hold the coarse z;
+// entries that are far along it do not fit either.
+template <int NF, bool PER, bool GH, bool SH, bool ZC, int P>
 __device__ __forceinline__ bool fx_rhs_rows(const StepArgs& A, int s, int m, int sub,
                                             const int* sgn, const double* bG, long long (*H)[kNB],
                                             int* kb, int sh) {
@@ -400,9 +439,14 @@ __device__ __forceinline__ bool fx_rhs_rows(const StepArgs& A, int s, int m, int
   const uint32_t mask = K.fx_mask;
   // the scale of each field: its largest difference in this stencil, in FP32
   unsigned mx[NF];
-  float mf[NF];
+  float mf[NF], zi = 0.f, f2 = 0.f;
+  bool near = true;
   {
     const float4 v = A.fs[s];
+    if (ZC) {  // (f2: the mirror of z is f2 - z)
+      zi = v.w;
+      f2 = fx_coarse(2.0 * K.floor_z, 2.0 * fx_ref(A).z, K.fx_turn);
+    }
     const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -428,6 +472,7 @@ __device__ __forceinline__ bool fx_rhs_rows(const StepArgs& A, int s, int m, int
       if ((cd[t] & mask) >= (uint32_t)n) continue;
       const float vv[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
       const bool mir = cd[t] >> 31;
+      if (ZC) near = near && fabsf((mir ? f2 - v[t].w : v[t].w) - zi) < kFxNear;
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
         const float d = (mir ? (float)sgn[f] * vv[f] : vv[f]) - mf[f];
@@ -531,7 +576,7 @@ __device__ __forceinline__ bool fx_rhs_rows(const StepArgs& A, int s, int m, int
       for (int q = 3; q < kNB; ++q) fx_acc(H[f][q], bq, a[q]);
     }
   }
-  return fits;
+  return fits && near;
 }
 template <int NF, bool SH>
 __device__ __forceinline__ void fx_rhs_values(const StepConsts& K, const long long (*H)[kNB],
@@ -550,12 +595,12 @@ __device__ __forceinline__ void fx_rhs_values(const StepConsts& K, const long lo
     }
   }
 }
-template <int NF, bool PER, bool GH, bool SH = false>
+template <int NF, bool PER, bool GH, bool ZC, bool SH = false>
 __device__ __forceinline__ bool fx_rhs(const StepArgs& A, int s, int m, const int* sgn,
                                        const double* bG, double (*R9)[kNB], int sh = 0) {
   long long H[NF][kNB];
   int kb[NF];
-  if (!fx_rhs_rows<NF, PER, GH, SH, 1>(A, s, m, 0, sgn, bG, H, kb, sh)) return false;
+  if (!fx_rhs_rows<NF, PER, GH, SH, ZC, 1>(A, s, m, 0, sgn, bG, H, kb, sh)) return false;
   fx_rhs_values<NF, SH>(A.K, H, kb, sh, R9);
   return true;
 }

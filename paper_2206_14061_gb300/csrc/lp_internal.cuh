@@ -92,11 +92,12 @@ struct StepConsts {
   // offsets are cut by 2^fx_sq (fx_qs = 2^-fx_sq), fx_lim bounds the integer
   // part of an offset; factors from integer sums of degree 2, 3, 4 (moments)
   // and 1, 2 (right-hand sides) to units of h; the mirror plane and the
-  // periods in fixed point; half periods (infinite without)
+  // periods in fixed point; 1 / the length after which fixed-point positions
+  // repeat, and half periods times it (infinite without)
   int fx_k, fx_sq, fx_lim;
   uint32_t fx_mask;  // index bits of a stencil code (the ghost flag is not one in a step)
   float fx_qs, fx_hLx, fx_hLy;
-  double fx_g2, fx_g3, fx_g4, fx_lin, fx_quad;
+  double fx_g2, fx_g3, fx_g4, fx_lin, fx_quad, fx_turn;
   unsigned long long fx_F2, fx_Lx, fx_Ly;
   long long ghost_PX, ghost_PY;
   double ghost_grid, ghost_hk, ghost_V, ghost_num;

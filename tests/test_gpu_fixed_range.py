@@ -213,3 +213,94 @@ def test_step_of_small_clusters(capi, orc, size):
     err = np.abs(du - dr).max() - floor
     print(f"size {size:g}: {err / np.abs(dr).max():.2e}")
     assert err <= TOL * np.abs(dr).max()
+
+
+def _turn(r, bits):
+    """Length after which fixed-point positions repeat, laid out for radius r."""
+    return bits * 2.0 ** np.frexp(r)[1]
+
+
+@pytest.mark.parametrize("lists", ["own", "built", "mirrors"])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("turns", [0.3, 1, 3, 1000, 3e6])
+def test_fit_of_entries_far_along_an_axis(capi, turns, axis, lists):
+    """A lattice whose layers are whole turns of the fixed-point positions apart
+    along one axis: the entries look near. Caller's stencils, those the context
+    built before the layers moved, and caller's with every entry of a higher
+    layer given as the floor mirror of a particle below the floor."""
+    h, X = 1e-3, _lattice(7, 0.05)
+    base = np.round(X)
+    ctx = capi.Context(2 * X.shape[1], cap=64)
+    P = X * h
+    nbr, cnt = _lists(X, 1.9)
+    nb = None
+    if lists == "built":
+        nb = capi.lp_build_neighbors(ctx, *[T(c) for c in P], r_const=1.9 * h, mirror_mode=0)
+        nbr, cnt = nb.export()
+    apart = turns * _turn(1.9 * h if lists == "built" else 4 * h, 64.0)
+    P[axis] = base[axis] * apart + (X - base)[axis] * h
+    F, floor, sign = _fields(X), 0.0, [1.0, 1.0]
+    if lists == "mirrors":
+        n = X.shape[1]
+        up = (np.arange(64) < cnt[:, None]) & (base[2][nbr] > base[2][:, None])
+        floor = -4.0 * (apart if axis == 2 else h)
+        P = np.concatenate([P, np.stack([P[0], P[1], 2.0 * floor - P[2]])], 1)
+        at = P.copy()
+        at[2, n:] = 2.0 * floor - P[2, n:]  # as the stored positions have them
+        ref_nbr = np.concatenate([np.where(up, nbr + n, nbr), np.zeros_like(nbr)])
+        nbr = np.concatenate([np.where(up, (nbr + n) | np.int32(-2 ** 31), nbr),
+                              np.zeros_like(nbr)])
+        cnt = np.concatenate([cnt, np.zeros_like(cnt)])
+        F = np.concatenate([F, -F], 1)  # (odd fields: the mirrors have F again)
+        sign = [-1.0, -1.0]
+        ref_F = np.concatenate([F[:, :n], F[:, :n]], 1)
+    else:
+        at, ref_nbr, ref_F = P, nbr, F
+    if nb is None:
+        nb = _own(capi, ctx, nbr, cnt)
+    got = capi.lp_fit_derivatives(ctx, *[T(c) for c in P], nb, [T(f) for f in F], sign, h,
+                                  floor_z=floor).cpu().numpy()
+    assert ctx.sync()["flags"] == 0
+    fit = cnt >= 26
+    assert fit.sum() >= 100
+    ref = np.zeros_like(got)
+    ref[fit] = _reference(at, ref_nbr, cnt, ref_F, np.nonzero(fit)[0])
+    s = np.full(3, h)
+    s[axis] = apart
+    err = _error(got, ref, s, fit)
+    print(f"turns {turns:g} axis {axis} {lists}: {err:.2e}")
+    assert err <= TOL
+    ctx.close()
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("side", [7, 26, 31])
+@pytest.mark.parametrize("axis", [0, 2])
+def test_step_on_held_stencils_that_spread(capi, orc, axis, side, mode):
+    """A dilute gas (no stress) whose layers move a turn of the fixed-point
+    positions apart in the first step; the second takes the same stencils."""
+    h, dt, radius = 1e-3, 1e-3, 1.9e-3
+    X = _lattice(side, 0.05)
+    base = np.round(X - X.min(1)[:, None])
+    vel = np.zeros_like(X)
+    vel[axis] = base[axis] * _turn(radius, 16.0) / dt
+    wl = W.cube(6)
+    pd = dict(W.param_dict(wl), h=h, radius=radius, mirror_mode=0, dt=dt, gz=0.0)
+    n = X.shape[1]
+    st = dict(zip(capi.FIELDS, [*(X * h), *vel, np.full(n, 1.0 / 0.2)]))
+    ref, _ = orc.step(st, orc.params(**pd), 2, rebuild_every=2, brute=n < 4000)
+    ctx = capi.Context(n, cap=64)
+    dev = {k: T(v) for k, v in st.items()}
+    mui = {k: pd[k] for k in ("mu_s", "mu_2", "I0", "d", "rho_s")}
+    eos = {k: pd[k] for k in ("phi_c", "phi_min", "phi_max", "alpha", "beta")}
+    capi.lp_step(ctx, dev, mui, eos, _params(pd, launch_mode=mode, rebuild_every=2), dt, 2)
+    assert ctx.sync()["flags"] == 0
+    ctx.close()
+    # (two layers from the surface: V of the outermost is an extrapolation, may
+    # leave the gas regime, and then changes velocities that the next one sees)
+    inner = ((base > 1.5) & (base < side - 2.5)).all(0)
+    err = np.abs(dev["V"].cpu().numpy() - ref["V"])[inner].max() / ref["V"][inner].max()
+    print(f"n {n} mode {mode}: {err:.2e}")
+    assert err <= TOL
+    for k in "xyzuvw":
+        assert np.allclose(dev[k].cpu().numpy()[inner], ref[k][inner], rtol=1e-12, atol=0), k
