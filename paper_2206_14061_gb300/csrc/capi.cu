@@ -142,6 +142,7 @@ struct lp_ctx {
   // left to the plain FP64 rows, 1 where offsets are outside the range
   float4* fs = nullptr;
   int32_t* slow = nullptr;
+  int32_t* ill = nullptr;     // lp_fit_derivatives: poorly conditioned stencils (in P1s too)
   uint8_t* kx = nullptr;
   float *Tg = nullptr, *T2 = nullptr;  // twin sums (allocated on first free-surface step)
   double* Y0[7] = {};                  // Heun: state at the start of the step (on first use)
@@ -766,7 +767,8 @@ lp_status lp_ctx_create(const lp_ctx_desc* desc, lp_ctx** out) {
   if (s == LP_OK) {  // FP64 passes use the float-float passes' block (72 B per particle)
     c->fs = (float4*)c->P1s;
     c->slow = (int32_t*)(c->fs + n);
-    c->kx = (uint8_t*)(c->slow + n);
+    c->ill = c->slow + n;
+    c->kx = (uint8_t*)(c->ill + n);
   }
   if (s == LP_OK) s = dalloc(c, &c->R1, n * 27);
   if (s == LP_OK) s = dalloc(c, &c->Lff, n * kTri);
@@ -1041,6 +1043,10 @@ lp_status lp_fit_derivatives(lp_ctx* c, const lp_particles* p, const lp_neighbor
   F.inv_h = 1.0 / h; F.f2 = 2.0 * floor_z;
   F.coeffs = coeffs;
   F.fb_list = c->fb_list; F.fb_count = c->fb_count; F.fb_cap = c->fb_cap;
+  F.ill = c->ill; F.ill_count = c->fb_count + 2;  // (pass 2's slow count: none here)
+  // QR fits of poorly conditioned stencils may cost a sixth of the plain FP64
+  // rows or a tenth of the float-float ones; 64 are less than a warp per SM
+  F.ill_room = std::max(F.n / (precision == LP_FP64 ? 256 : 1024), 64);
   F.dg = c->dg;
   if (precision == LP_MIXED_FF) {  // the step's split and factor buffers serve as scratch
     if (!c->fit_fs) LP_TRY(dalloc(c, &c->fit_fs, (size_t)kMaxFields * c->cap_n));

@@ -381,6 +381,27 @@ __device__ __forceinline__ int fit_thread(const FitArgs& F) {
   return (F.perm && t < F.n) ? F.perm[t] : t;
 }
 
+// Poorly conditioned stencils (a relative pivot below 2^-7 in FP64, 2^-10 in
+// float-float) that the normal equations still take. Rounding is amplified by
+// up to 1 / pivot^2 there (2.5e-11 of the largest derivative for a stencil of
+// nine entries), so they take the QR fit where they are few: 0.15 % (2^-7) and
+// one in 100,000 (2^-10) of the sweep lattice. Surfaces of lattices with little
+// jitter, and all of a sheet of two layers, are such stencils, and a QR fit
+// costs 120 ns (normal equations: 3 ns in FP64, 1.2 in float-float). With all
+// of them by QR 1.0 M particles in a lattice of 10 to 18 entries a stencil,
+// three fields, took 7.6 to 10 ms in FP64 and 7.3 to 8.4 in float-float; plain
+// FP64 rows for every particle took 3.1 to 4.7, float-float sums 1.1 to 1.4.
+// So above ill_room (lp_fit_derivatives sets it) none does: they take the plain
+// FP64 rows, or keep the float-float fit. The line is on their number, so that
+// which stencils take which path does not depend on the order of the threads.
+__device__ __forceinline__ int ill_by_qr(const FitArgs& F) {
+  const int c = F.ill ? *F.ill_count : 0;
+  return c <= F.ill_room ? c : 0;
+}
+__device__ __forceinline__ void push_ill(const FitArgs& F, int s) {
+  F.ill[atomicAdd(F.ill_count, 1)] = s;  // (each particle once: n entries at most)
+}
+
 // ---- lp_fit_derivatives in FP64 with the rows in fixed point (as the step's
 // pass 1, fixed_rows.cuh): records of the positions, moments and factor, then
 // the fields in groups of up to three. 170,000 particles, three fields: 1.61 ms
@@ -391,6 +412,18 @@ __global__ void k_fit_fx_split(const FitArgs F, const StepArgs A) {
   if (s >= F.n) return;
   FxRec* R = reinterpret_cast<FxRec*>(A.XU);
   fx_position(A, F.x[s], F.y[s], F.z[s], R[s]);
+}
+// an entry that may only look near along z (the sums over the fields check all
+// stencils; this one is for those refused before them)
+__device__ __forceinline__ bool fit_far_in_z(const FitArgs& F, const StepArgs& A, int s, int m) {
+  for (int k = 0; k < m; ++k) {
+    const uint32_t code = (uint32_t)F.nbr[(int64_t)k * F.n + s];
+    const int j = code & ~kMirrorBit;
+    if ((unsigned)j >= (unsigned)F.n) continue;  // stale or corrupt stencil entry
+    const double d = ((code >> 31) ? F.f2 - F.z[j] : F.z[j]) - F.z[s];
+    if (!(fabs(d) * A.K.fx_turn < kFxNear)) return true;
+  }
+  return false;
 }
 __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, const StepArgs A) {
   const int s = fit_thread(F);
@@ -409,18 +442,18 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, co
   bool ill = false;
   const bool ok = fits && fx_chol9(L, 1e-9, &ill) && rows >= kNB;
   A.kx[s] = ok && !ill ? sh : kFxSlow;
-  if (!fits) {
+  if (!fits || (!ok && fit_far_in_z(F, A, s, m))) {
     fx_push(A, s, 0);
     return;
   }
-  if (!ok || ill) {
-    // poorly conditioned stencils take the QR fit: rounding of the normal
-    // equations is amplified by 1 / pivot^2 there (2.5e-11 of the largest
-    // derivative for a stencil of nine entries), and the sweep lattice has 0.15 %
-    // of them. Those the normal equations refuse in every mode count as fallbacks.
+  if (!ok) {
     const int slot = atomicAdd(F.fb_count, 1);
-    if (slot < F.fb_cap) F.fb_list[slot] = ok ? s | (int)kMirrorBit : s;
+    if (slot < F.fb_cap) F.fb_list[slot] = s;
     else atomicOr(&F.dg->flags, (unsigned)LP_FLAG_OVERFLOW);
+    return;
+  }
+  if (ill) {
+    push_ill(F, s);
     return;
   }
 #pragma unroll
@@ -471,8 +504,9 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_rhs_fx(const FitArgs F, con
 }
 __global__ void __launch_bounds__(64) k_fit_slow(const FitArgs F, const StepArgs A) {
   const int cnt = min(A.slow_count[0], F.n);
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x)
-    fit_body<LP_FP64>(F, A.slow[t]);
+  const int all = cnt + (ill_by_qr(F) ? 0 : *F.ill_count);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < all; t += gridDim.x * blockDim.x)
+    fit_body<LP_FP64>(F, t < cnt ? A.slow[t] : F.ill[t - cnt]);
 }
 
 // ---- lp_fit_derivatives in float-float (LP_MIXED_FF): positions relative
@@ -535,12 +569,11 @@ __global__ void __launch_bounds__(128, 4) k_fit_gram_ff(const FitArgs F) {
   for (int k = 0; k < kTri; ++k) G[k] = ff_norm(G[k]);
   bool ill = false;
   const bool ok = ff_chol9(G, 1e-4f, &ill) && rows >= kNB;
-  // poorly conditioned stencils take the QR fit, as in FP64, but at 2^-10 (about
-  // one in 100,000 of the sweep lattice; at 2^-7 the QR fits of 2.0 M particles
-  // cost 0.5 ms)
-  if (!ok || ill) {
+  // (at 2^-7, as in FP64, the QR fits of 2.0 M particles of the sweep cost 0.5 ms)
+  if (ok && ill) push_ill(F, s);  // the QR fit overwrites the float-float one
+  if (!ok) {
     const int slot = atomicAdd(F.fb_count, 1);
-    if (slot < F.fb_cap) F.fb_list[slot] = ok ? s | (int)kMirrorBit : s;
+    if (slot < F.fb_cap) F.fb_list[slot] = s;
     else atomicOr(&F.dg->flags, (unsigned)LP_FLAG_OVERFLOW);
     F.lf[s] = make_float2(-1.f, 0.f);  // 1/L_00 > 0 for a factored stencil
     return;
@@ -687,10 +720,11 @@ __device__ __forceinline__ bool qr_column(double (*a)[kNB], double (*b)[4], int*
 }
 __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
   const int cnt = min(*F.fb_count, F.fb_cap);
+  const int all = cnt + ill_by_qr(F);
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < cnt; t += nw) {
-    const int e = F.fb_list[t], s = e & ~kMirrorBit;
+  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < all; t += nw) {
+    const int s = t < cnt ? F.fb_list[t] : F.ill[t - cnt];
     const int n = F.n;
     const int m = min(F.cnt[s], F.cap);
     const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
@@ -775,7 +809,7 @@ __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
               mine * (lane < 3 ? F.inv_h : F.inv_h * F.inv_h);
       }
     }
-    if (lane == 0 && e >= 0) atomicAdd(&F.dg->n_fallback, 1ull);
+    if (lane == 0 && t < cnt) atomicAdd(&F.dg->n_fallback, 1ull);  // (refused ones)
     __syncwarp();  // (pk is reused)
   }
 }

@@ -345,6 +345,12 @@ struct FitArgs {
   int fb_cap;
   DevDiag* dg;
   const int32_t* perm;  // particle of each thread (rows sorted within groups of 128), or NULL
+  // particles whose stencil factors but is poorly conditioned (n at most), their
+  // number, and how many may take the QR fit (LP_MIXED_FF, and LP_FP64 with
+  // fixed-point rows; else NULL)
+  int32_t* ill;
+  int32_t* ill_count;
+  int ill_room;
   // LP_FP64 with fixed-point rows (a context's workspace): the rows' arguments;
   // NULL: plain FP64 rows
   const StepArgs* rows;
