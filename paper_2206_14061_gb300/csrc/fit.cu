@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
       bool run = true;
 #pragma unroll
       for (int q = 0; q < kNB; ++q) {
-        run = run && !(fabs(rd[q]) <= 1e-8 * fabs(rd[0]));  // (NaN: full rank, NaN results)
+        run = run && fabs(rd[q]) > 1e-8 * fabs(rd[0]);  // (NaN: the columns before it count)
         rank += run;
       }
 #pragma unroll
@@ -799,8 +799,10 @@ __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
         for (int k = kNB - 1; k >= 0; --k) {
           double v = __shfl_sync(0xffffffffu, b[0][f], k);
 #pragma unroll
-          for (int j = k + 1; j < kNB; ++j)
-            v -= __shfl_sync(0xffffffffu, a[0][j], k) * y[j];
+          for (int j = k + 1; j < kNB; ++j) {
+            const double t = __shfl_sync(0xffffffffu, a[0][j], k);
+            if (j < rank) v -= t * y[j];  // (past the rank it may be NaN)
+          }
           y[k] = k < rank ? v / rd[k] : 0.0;
           if (perm[k] == lane) mine = y[k];
         }
