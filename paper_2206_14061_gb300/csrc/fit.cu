@@ -387,8 +387,8 @@ __device__ __forceinline__ int fit_thread(const FitArgs& F) {
 // nine entries), so they take the QR fit where they are few: 0.15 % (2^-7) and
 // one in 100,000 (2^-10) of the sweep lattice. Surfaces of lattices with little
 // jitter, and all of a sheet of two layers, are such stencils, and a QR fit
-// costs 120 ns (normal equations: 3 ns in FP64, 1.2 in float-float). With all
-// of them by QR 1.0 M particles in a lattice of 10 to 18 entries a stencil,
+// costs many times the normal equations (3 ns in FP64, 1.2 in float-float). With all
+// of them by QR (120 ns a fit then) 1.0 M particles of 10 to 18 entries a stencil,
 // three fields, took 7.6 to 10 ms in FP64 and 7.3 to 8.4 in float-float; plain
 // FP64 rows for every particle took 3.1 to 4.7, float-float sums 1.1 to 1.4.
 // So above ill_room (lp_fit_derivatives sets it) none does: they take the plain
@@ -664,29 +664,68 @@ __global__ void __launch_bounds__(128, 3) k_fit_rhs_ff(const FitArgs F, int f0) 
   }
 }
 
-// Pivoted-QR fits of the queued particles, a warp for each: a lane holds rows
-// lane and lane + 32 of [A | B] in registers, and every column norm and
-// reflection is a warp sum. The same algorithm as qr_pivoted_solve (pivot: the
-// largest remaining norm, ties to the lower column; rank by 1e-8; basic
-// solution). One thread per particle with its matrix in local memory took 205 us
-// for the few hundred of the 2.0 M-particle sweep, a chain of dependent loads.
-__device__ __forceinline__ double warp_sum(double v) {
+// Pivoted-QR fits of the queued particles, the same algorithm as
+// qr_pivoted_solve (pivot: the largest remaining norm, ties to the lower
+// column; rank by 1e-8; basic solution).
+//
+// Few: a warp for each, a lane holding rows lane and lane + 32 of [A | B] in
+// registers, and every column norm and reflection a sum over the warp. What
+// bounds it is one warp's chain on the FP64 pipe, 75 cycles an instruction, so
+// the sums of a column's norms, or of its reflections, are taken together: each
+// step halves the number of values a lane holds (9 additions for 8 sums instead
+// of 40), rows past the 32nd and absent fields are skipped, and a lane takes the
+// back substitution of one field. A call with one QR fit of 12 to 48 rows takes
+// 45 us longer than one without; with a sum at a time 75 to 90.
+// Many: a thread for each, its matrix in local memory (fit_qr_item). Particles
+// with six entries, all refused, LP_FP64, three fields: 8,000 take 147 us
+// (1046 with a warp each, summed one at a time), 1.0 M 5.8 ms (120). The line:
+// a wave of thread fits takes about as long as 4,096 warp fits.
+template <int N>
+__device__ __forceinline__ void warp_sums(double* v, int lane) {
+  constexpr int P = N > 8 ? 8 : (N > 4 ? 8 : (N > 2 ? 4 : N));
+  double w[P];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+  for (int i = 0; i < P; ++i) w[i] = i < N ? v[i] : 0.0;
+  int bit = 16;
+#pragma unroll
+  for (int h = P / 2; h >= 1; h >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int i = 0; i < h; ++i)
+      w[i] = (up ? w[i + h] : w[i]) + __shfl_xor_sync(0xffffffffu, up ? w[i] : w[i + h], bit);
+    bit >>= 1;
+  }
+#pragma unroll
+  for (; bit; bit >>= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], bit);
+#pragma unroll
+  for (int i = 0; i < P; ++i) {  // (value i lies in the lanes with these bits)
+    int src = 0;
+#pragma unroll
+    for (int h = P / 2, b = 16; h >= 1; h >>= 1, b >>= 1) src |= (i & h) ? b : 0;
+    if (i < N) v[i] = __shfl_sync(0xffffffffu, w[0], src);
+  }
+  if constexpr (N > P) warp_sums<N - P>(v + P, lane);
 }
+// (two: there are rows past the 32nd)
 template <int K>
-__device__ __forceinline__ bool qr_column(double (*a)[kNB], double (*b)[4], int* perm,
-                                          double* rdiag, int lane) {
+__device__ __forceinline__ bool qr_column(double (*a)[kNB], double (*b)[4], int nf, bool two,
+                                          int* perm, double* rdiag, int lane) {
   // row index of a[h]: lane + 32 h; rows above K are done
   const bool in = lane >= K;
+  constexpr int J = kNB - K;  // columns left
+  double s[J + 3];            // (J norms, or J - 1 columns and 4 fields)
+#pragma unroll
+  for (int j = 0; j < J; ++j) s[j] = in ? a[0][K + j] * a[0][K + j] : 0.0;
+  if (two) {
+#pragma unroll
+    for (int j = 0; j < J; ++j) s[j] += a[1][K + j] * a[1][K + j];
+  }
+  warp_sums<J>(s, lane);
   int best = K;
   double bestn = -1.0;
 #pragma unroll
-  for (int j = K; j < kNB; ++j) {
-    const double s = warp_sum((in ? a[0][j] * a[0][j] : 0.0) + a[1][j] * a[1][j]);
-    if (s > bestn) { bestn = s; best = j; }
-  }
+  for (int j = 0; j < J; ++j)
+    if (s[j] > bestn) { bestn = s[j]; best = K + j; }
   const double alpha = sqrt(bestn);
   if (alpha == 0.0 || !(bestn >= 0.0)) {  // (a NaN norm never wins: all columns are NaN)
     rdiag[K] = bestn >= 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
@@ -704,116 +743,172 @@ __device__ __forceinline__ bool qr_column(double (*a)[kNB], double (*b)[4], int*
   const double v0 = lane == K ? akk + sgn * alpha : (in ? a[0][K] : 0.0), v1 = a[1][K];
   const double f = 1.0 / (bestn + fabs(akk) * alpha);  // 2 / v.v
 #pragma unroll
-  for (int j = K + 1; j < kNB; ++j) {
-    const double t = f * warp_sum(v0 * a[0][j] + v1 * a[1][j]);
-    a[0][j] -= t * v0;
-    a[1][j] -= t * v1;
+  for (int j = 1; j < J; ++j) s[j - 1] = v0 * a[0][K + j];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) s[J - 1 + q] = q < nf ? v0 * b[0][q] : 0.0;
+  if (two) {
+#pragma unroll
+    for (int j = 1; j < J; ++j) s[j - 1] += v1 * a[1][K + j];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < nf) s[J - 1 + q] += v1 * b[1][q];
+  }
+  warp_sums<J + 3>(s, lane);
+#pragma unroll
+  for (int j = 1; j < J; ++j) {
+    s[j - 1] *= f;
+    a[0][K + j] -= s[j - 1] * v0;
+    if (two) a[1][K + j] -= s[j - 1] * v1;
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const double t = f * warp_sum(v0 * b[0][q] + v1 * b[1][q]);
-    b[0][q] -= t * v0;
-    b[1][q] -= t * v1;
-  }
+  for (int q = 0; q < 4; ++q)
+    if (q < nf) {
+      s[J - 1 + q] *= f;
+      b[0][q] -= s[J - 1 + q] * v0;
+      if (two) b[1][q] -= s[J - 1 + q] * v1;
+    }
   rdiag[K] = -sgn * alpha;
   return true;
 }
+// one fit by a warp (pk: its shared codes)
+__device__ __forceinline__ void fit_qr_warp(const FitArgs& F, int s, uint32_t* pk, int lane) {
+  const int n = F.n;
+  const int m = min(F.cnt[s], F.cap);
+  const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
+  // rows are packed: an entry whose index is out of range is dropped and the
+  // rows after it move up; lanes past the last row hold zeros
+  pk[lane] = pk[lane + 32] = ~kMirrorBit;
+  __syncwarp();
+  int rows = 0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = lane + 32 * h;
+    const uint32_t c = k < m ? (uint32_t)F.nbr[(int64_t)k * n + s] : ~kMirrorBit;
+    const bool in = (c & ~kMirrorBit) < (uint32_t)n;
+    const unsigned all = __ballot_sync(0xffffffffu, in);
+    if (in) pk[rows + __popc(all & ((1u << lane) - 1u))] = c;
+    rows += __popc(all);
+  }
+  __syncwarp();
+  const bool two = rows > 32;
+  uint32_t code[2];
+  double row[2][kNB];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    code[h] = pk[lane + 32 * h];
+    const int j = code[h] & ~kMirrorBit;
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) row[h][q] = 0.0;
+    if ((unsigned)j < (unsigned)n) {
+      const double zj = (code[h] >> 31) ? F.f2 - F.z[j] : F.z[j];
+      taylor_row((F.x[j] - xi) * F.inv_h, (F.y[j] - yi) * F.inv_h, (zj - zi) * F.inv_h, row[h]);
+    }
+  }
+  for (int f0 = 0; f0 < F.nf; f0 += 4) {
+    const int nf = min(4, F.nf - f0);
+    double a[2][kNB], b[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = code[h] & ~kMirrorBit;
+#pragma unroll
+      for (int q = 0; q < kNB; ++q) a[h][q] = row[h][q];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        b[h][f] = 0.0;
+        if (f < nf && (unsigned)j < (unsigned)n) {
+          double vj = F.fields[f0 + f][j];
+          if (code[h] >> 31) vj *= F.msign[f0 + f];
+          b[h][f] = vj - F.fields[f0 + f][s];
+        }
+      }
+    }
+    int perm[kNB];
+    double rd[kNB];
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) { perm[q] = q; rd[q] = 0.0; }
+    qr_column<0>(a, b, nf, two, perm, rd, lane) && qr_column<1>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<2>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<3>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<4>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<5>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<6>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<7>(a, b, nf, two, perm, rd, lane) &&
+        qr_column<8>(a, b, nf, two, perm, rd, lane);
+    int rank = 0;
+    bool run = true;
+#pragma unroll
+    for (int q = 0; q < kNB; ++q) {
+      run = run && fabs(rd[q]) > 1e-8 * fabs(rd[0]);  // (NaN: the columns before it count)
+      rank += run;
+    }
+    double y[kNB];  // of field f0 + lane
+#pragma unroll
+    for (int k = kNB - 1; k >= 0; --k) {
+      double v = 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double t = __shfl_sync(0xffffffffu, b[0][q], k);
+        if (q == lane) v = t;
+      }
+#pragma unroll
+      for (int j = k + 1; j < kNB; ++j) {
+        const double t = __shfl_sync(0xffffffffu, a[0][j], k);
+        if (j < rank) v -= t * y[j];  // (past the rank it may be NaN)
+      }
+      y[k] = k < rank ? v / rd[k] : 0.0;
+    }
+    if (lane < nf) {
+      double* o = F.coeffs + ((int64_t)s * F.nf + f0 + lane) * kNB;
+#pragma unroll
+      for (int k = 0; k < kNB; ++k)
+        o[perm[k]] = y[k] * (perm[k] < 3 ? F.inv_h : F.inv_h * F.inv_h);
+    }
+  }
+  __syncwarp();  // (pk is reused)
+}
+// one fit by a thread
+__device__ __noinline__ void fit_qr_item(const FitArgs& F, int s) {
+  double Am[LP_MAX_CAP * kNB], Bm[LP_MAX_CAP * 4], C[4 * kNB];
+  const int n = F.n;
+  const int m = min(F.cnt[s], F.cap);
+  const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
+  for (int f0 = 0; f0 < F.nf; f0 += 4) {
+    const int nf = min(4, F.nf - f0);
+    int rows = 0;  // (packed, as above)
+    for (int k = 0; k < m; ++k) {
+      const uint32_t code = (uint32_t)F.nbr[(int64_t)k * n + s];
+      const int j = code & ~kMirrorBit;
+      if ((unsigned)j >= (unsigned)n) continue;  // stale or corrupt stencil entry
+      const bool mir = code >> 31;
+      const double zj = mir ? F.f2 - F.z[j] : F.z[j];
+      taylor_row((F.x[j] - xi) * F.inv_h, (F.y[j] - yi) * F.inv_h, (zj - zi) * F.inv_h,
+                 &Am[rows * kNB]);
+      for (int f = 0; f < nf; ++f) {
+        double vj = F.fields[f0 + f][j];
+        if (mir) vj *= F.msign[f0 + f];
+        Bm[rows * nf + f] = vj - F.fields[f0 + f][s];
+      }
+      ++rows;
+    }
+    qr_pivoted_solve(rows, Am, nf, Bm, C);
+    for (int f = 0; f < nf; ++f) write_coeffs(F, s, f0 + f, C + f * kNB);
+  }
+}
+constexpr int kQrWarpFits = 4096;
 __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
   const int cnt = min(*F.fb_count, F.fb_cap);
   const int all = cnt + ill_by_qr(F);
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < all; t += nw) {
-    const int s = t < cnt ? F.fb_list[t] : F.ill[t - cnt];
-    const int n = F.n;
-    const int m = min(F.cnt[s], F.cap);
-    const double xi = F.x[s], yi = F.y[s], zi = F.z[s];
-    // rows are packed: an entry whose index is out of range is dropped and the
-    // rows after it move up; lanes past the last row hold zeros
-    __shared__ uint32_t packed[2][LP_MAX_CAP];
-    uint32_t* pk = packed[threadIdx.x >> 5];
-    pk[lane] = pk[lane + 32] = ~kMirrorBit;
-    __syncwarp();
-    int rows = 0;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = lane + 32 * h;
-      const uint32_t c = k < m ? (uint32_t)F.nbr[(int64_t)k * n + s] : ~kMirrorBit;
-      const bool in = (c & ~kMirrorBit) < (uint32_t)n;
-      const unsigned all = __ballot_sync(0xffffffffu, in);
-      if (in) pk[rows + __popc(all & ((1u << lane) - 1u))] = c;
-      rows += __popc(all);
-    }
-    __syncwarp();
-    uint32_t code[2];
-    double row[2][kNB];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      code[h] = pk[lane + 32 * h];
-      const int j = code[h] & ~kMirrorBit;
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) row[h][q] = 0.0;
-      if ((unsigned)j < (unsigned)n) {
-        const double zj = (code[h] >> 31) ? F.f2 - F.z[j] : F.z[j];
-        taylor_row((F.x[j] - xi) * F.inv_h, (F.y[j] - yi) * F.inv_h, (zj - zi) * F.inv_h, row[h]);
-      }
-    }
-    for (int f0 = 0; f0 < F.nf; f0 += 4) {
-      const int nf = min(4, F.nf - f0);
-      double a[2][kNB], b[2][4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = code[h] & ~kMirrorBit;
-#pragma unroll
-        for (int q = 0; q < kNB; ++q) a[h][q] = row[h][q];
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          b[h][f] = 0.0;
-          if (f < nf && (unsigned)j < (unsigned)n) {
-            double vj = F.fields[f0 + f][j];
-            if (code[h] >> 31) vj *= F.msign[f0 + f];
-            b[h][f] = vj - F.fields[f0 + f][s];
-          }
-        }
-      }
-      int perm[kNB];
-      double rd[kNB];
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) { perm[q] = q; rd[q] = 0.0; }
-      qr_column<0>(a, b, perm, rd, lane) && qr_column<1>(a, b, perm, rd, lane) &&
-          qr_column<2>(a, b, perm, rd, lane) && qr_column<3>(a, b, perm, rd, lane) &&
-          qr_column<4>(a, b, perm, rd, lane) && qr_column<5>(a, b, perm, rd, lane) &&
-          qr_column<6>(a, b, perm, rd, lane) && qr_column<7>(a, b, perm, rd, lane) &&
-          qr_column<8>(a, b, perm, rd, lane);
-      int rank = 0;
-      bool run = true;
-#pragma unroll
-      for (int q = 0; q < kNB; ++q) {
-        run = run && fabs(rd[q]) > 1e-8 * fabs(rd[0]);  // (NaN: the columns before it count)
-        rank += run;
-      }
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        double y[kNB], mine = 0.0;
-#pragma unroll
-        for (int k = kNB - 1; k >= 0; --k) {
-          double v = __shfl_sync(0xffffffffu, b[0][f], k);
-#pragma unroll
-          for (int j = k + 1; j < kNB; ++j) {
-            const double t = __shfl_sync(0xffffffffu, a[0][j], k);
-            if (j < rank) v -= t * y[j];  // (past the rank it may be NaN)
-          }
-          y[k] = k < rank ? v / rd[k] : 0.0;
-          if (perm[k] == lane) mine = y[k];
-        }
-        if (f < nf && lane < kNB)
-          F.coeffs[((int64_t)s * F.nf + f0 + f) * kNB + lane] =
-              mine * (lane < 3 ? F.inv_h : F.inv_h * F.inv_h);
-      }
-    }
-    if (lane == 0 && t < cnt) atomicAdd(&F.dg->n_fallback, 1ull);  // (refused ones)
-    __syncwarp();  // (pk is reused)
+  __shared__ uint32_t packed[2][LP_MAX_CAP];
+  if (all <= kQrWarpFits) {
+    for (int t = tid >> 5; t < all; t += nth >> 5)
+      fit_qr_warp(F, t < cnt ? F.fb_list[t] : F.ill[t - cnt], packed[threadIdx.x >> 5], lane);
+  } else {
+    for (int t = tid; t < all; t += nth) fit_qr_item(F, t < cnt ? F.fb_list[t] : F.ill[t - cnt]);
   }
+  // (those of the normal equations' choice count: the refused ones)
+  if (tid == 0 && cnt > 0) atomicAdd(&F.dg->n_fallback, (unsigned long long)cnt);
 }
 
 // ---------------------------------------------------------- lp_mui_stress
