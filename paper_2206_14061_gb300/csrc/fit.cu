@@ -1034,7 +1034,7 @@ void launch_pass2(int prec, const StepArgs& A, cudaStream_t st, int bs) {
 void launch_fit(int prec, const FitArgs& F, cudaStream_t st) {
   const int bs = spread_block(F.n, kBlock);
   const int nb = (F.n + bs - 1) / bs;
-  if (F.perm && (prec == LP_MIXED_FF || F.rows))
+  if (F.perm)
     k_row_order<<<(F.n + kRowGroup - 1) / kRowGroup, kRowGroup, 0, st>>>(
         F.n, F.cnt, const_cast<int32_t*>(F.perm));
   if (prec == LP_FP64 && F.rows) {
