@@ -1044,9 +1044,14 @@ lp_status lp_fit_derivatives(lp_ctx* c, const lp_particles* p, const lp_neighbor
   F.coeffs = coeffs;
   F.fb_list = c->fb_list; F.fb_count = c->fb_count; F.fb_cap = c->fb_cap;
   F.ill = c->ill; F.ill_count = c->fb_count + 2;  // (pass 2's slow count: none here)
-  // QR fits of poorly conditioned stencils may cost a sixth of the plain FP64
-  // rows or a tenth of the float-float ones; 64 are less than a warp per SM
-  F.ill_room = std::max(F.n / (precision == LP_FP64 ? 256 : 1024), 64);
+  // How many poorly conditioned stencils take the QR fit. LP_FP64: the plain
+  // rows, the other way, take 75 to 200 us for a wave of 39,000 (a thread's
+  // chain of FP64 operations), the QR fits 45 us for each 608; in calls of over
+  // 150,000 particles more of them do not show. LP_MIXED_FF: the other way costs
+  // nothing (their float-float fit is done anyway), so few. (59,000 particles,
+  // 24 nearest, three fields, LP_FP64, some 300 such stencils: 282 us by the
+  // plain rows, 225 by QR; 1,700 with 700 of them 137 and 229.)
+  F.ill_room = precision == LP_FP64 ? std::max(F.n / 256, 608) : std::max(F.n / 1024, 64);
   F.dg = c->dg;
   if (precision == LP_MIXED_FF) {  // the step's split and factor buffers serve as scratch
     if (!c->fit_fs) LP_TRY(dalloc(c, &c->fit_fs, (size_t)kMaxFields * c->cap_n));
