@@ -394,6 +394,11 @@ __device__ __forceinline__ int fit_thread(const FitArgs& F) {
 // So above ill_room (lp_fit_derivatives sets it) none does: they take the plain
 // FP64 rows, or keep the float-float fit. The line is on their number, so that
 // which stencils take which path does not depend on the order of the threads.
+// The QR fit's rank is relative to the largest column (1e-8), the pivots here to
+// their own, so that a stencil whose columns' lengths differ by 2^8 or more
+// (spacings far from h, or unequal) is not one of them: the QR fit might leave
+// columns out.
+constexpr int kQrSpreadBits = 16;  // of the squared lengths
 __device__ __forceinline__ int ill_by_qr(const FitArgs& F) {
   const int c = F.ill ? *F.ill_count : 0;
   return c <= F.ill_room ? c : 0;
@@ -439,10 +444,20 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, co
     fits = fx_moments<false, false, true>(A, s, m, mo, &rows, sh);
     if (fits) gram_of_moments(mo, L);
   }
+  bool even = false;  // the columns' lengths
+  if (fits) {
+    int lo = __double2hiint(L[0]), hi = lo;
+#pragma unroll
+    for (int j = 1; j < kNB; ++j) {
+      lo = min(lo, __double2hiint(L[tri(j, j)]));
+      hi = max(hi, __double2hiint(L[tri(j, j)]));
+    }
+    even = hi - lo < kQrSpreadBits << 20;
+  }
   bool ill = false;
   const bool ok = fits && fx_chol9(L, 1e-9, &ill) && rows >= kNB;
   A.kx[s] = ok && !ill ? sh : kFxSlow;
-  if (!fits || (!ok && fit_far_in_z(F, A, s, m))) {
+  if (!fits || (ok && ill && !even) || (!ok && fit_far_in_z(F, A, s, m))) {
     fx_push(A, s, 0);
     return;
   }
@@ -570,7 +585,18 @@ __global__ void __launch_bounds__(128, 4) k_fit_gram_ff(const FitArgs F) {
   bool ill = false;
   const bool ok = ff_chol9(G, 1e-4f, &ill) && rows >= kNB;
   // (at 2^-7, as in FP64, the QR fits of 2.0 M particles of the sweep cost 0.5 ms)
-  if (ok && ill) push_ill(F, s);  // the QR fit overwrites the float-float one
+  if (ok && ill) {  // the QR fit overwrites the float-float one
+    float shortest = INFINITY, longest = 0.f;  // the columns' squared lengths, from the factor
+#pragma unroll
+    for (int j = 0; j < kNB; ++j) {
+      float d = 1.f / (G[tri(j, j)].h * G[tri(j, j)].h);
+#pragma unroll
+      for (int k = 0; k < j; ++k) d += G[tri(j, k)].h * G[tri(j, k)].h;
+      shortest = fminf(shortest, d);
+      longest = fmaxf(longest, d);
+    }
+    if (shortest * (float)(1 << kQrSpreadBits) > longest) push_ill(F, s);
+  }
   if (!ok) {
     const int slot = atomicAdd(F.fb_count, 1);
     if (slot < F.fb_cap) F.fb_list[slot] = s;

@@ -96,3 +96,35 @@ def test_more_poorly_conditioned_stencils_than_the_queue_holds(capi, prec):
     err = (out[:, 0, 0] * h - (Xg[1] / k - 1.0)).abs()
     assert float(err.max()) < 1e-3
     assert float((err < (1e-10 if prec == 0 else 1e-6)).double().mean()) > 0.99
+
+
+@pytest.mark.parametrize("prec,unit,aspect", [(0, 3e-10, 1.0), (0, 1e-3, 1.0), (0, 1.0, 1e-5),
+                                              (2, 1e-3, 1.0), (2, 1.0, 1e-4)])
+def test_poorly_conditioned_stencils_whose_columns_differ_in_size(capi, prec, unit, aspect):
+    """The spacing `unit` h, compressed along z to `aspect`: pivots relative to
+    the columns are those of the lattice, but the QR fit's rank, relative to
+    the largest column, would leave out the smallest."""
+    h, X = 1.0, _lattice(5, 0.06, seed=11)
+    P = X * unit
+    ctx = capi.Context(X.shape[1], cap=64)
+    nb = capi.lp_build_neighbors(ctx, *[T(c) for c in P], r_const=2.2 * unit, mirror_mode=0,
+                                 cap=12, keep_nearest=1)
+    nbr, cnt = nb.export()
+    P[2] *= aspect
+    F = np.stack([np.sin(0.4 * X[0] + 0.3 * X[1] - 0.2 * X[2]), np.cos(0.3 * X[0] - 0.5 * X[2])])
+    got = capi.lp_fit_derivatives(ctx, *[T(c) for c in P], nb, [T(f) for f in F], [1.0, 1.0], h,
+                                  precision=prec).cpu().numpy()
+    assert ctx.sync()["flags"] == 0
+    ctx.close()
+    pick = np.arange(X.shape[1])
+    p = _pivots(X, nbr, cnt, pick)
+    pick, p = pick[p > 2e-4], p[p > 2e-4]
+    ill = (p < (2.0 ** -7 if prec == 0 else 2.0 ** -10)).sum()
+    ref = _reference(P, nbr, cnt, F, pick)
+    u, v = unit, unit * aspect
+    err = np.abs((got[pick] - ref) * np.array([u, u, v, u * u, u * u, v * v, u * u, u * v, u * v]))
+    err = err.max((1, 2))
+    eps = 2.0 ** -53 if prec == 0 else 2.0 ** -44
+    print(f"prec {prec} unit {unit:g} aspect {aspect:g}: {ill} ill, largest error "
+          f"{err.max():.1e}, in bounds {(err * p * p).max() / eps:.2f}")
+    assert 0 < ill and (err * p * p <= 2 ** 10 * eps).all()
