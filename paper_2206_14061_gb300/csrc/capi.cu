@@ -689,6 +689,9 @@ void fixed_consts(StepConsts& K, bool shifted = false) {
   const double q = l * l * std::ldexp(1.0, K.fx_sq);  // of a product as a factor
   K.fx_g2 = l * l; K.fx_g3 = l * q; K.fx_g4 = q * q;
   K.fx_lin = l; K.fx_quad = q;
+  // (a spacing h of over 1e69 radii: the factor, or a shifted one, is not normal;
+  // all particles take the plain rows)
+  if (!(K.fx_g4 >= 0x1p-970)) K.fx_lim = 0;
   K.fx_F2 = fx_of(2.0 * K.floor_z, K.fx_k);
   K.fx_Lx = fx_of(K.Lx, K.fx_k);
   K.fx_Ly = fx_of(K.Ly, K.fx_k);

@@ -304,3 +304,24 @@ def test_step_on_held_stencils_that_spread(capi, orc, axis, side, mode):
     assert err <= TOL
     for k in "xyzuvw":
         assert np.allclose(dev[k].cpu().numpy()[inner], ref[k][inner], rtol=1e-12, atol=0), k
+
+
+@pytest.mark.parametrize("h", [1e60, 1e69, 1e70, 1e72, 1e75, 1e77])
+def test_fit_with_h_far_above_the_spacing(capi, h):
+    """h is only the unit of the offsets: fourth powers of 1 / h near the
+    smallest normal number."""
+    X = _lattice(7, 0.1)
+    nbr, cnt = _lists(X, 1.9)
+    F = _fields(X)
+    for built in (False, True):
+        ctx = capi.Context(X.shape[1], cap=64)
+        nb = (capi.lp_build_neighbors(ctx, *[T(c) for c in X], r_const=1.9, mirror_mode=0)
+              if built else _own(capi, ctx, nbr, cnt))
+        got = capi.lp_fit_derivatives(ctx, *[T(c) for c in X], nb, [T(f) for f in F], [1.0, 1.0],
+                                      h).cpu().numpy()
+        assert ctx.sync()["flags"] == 0
+        fit = cnt >= 17
+        err = _error(got, _reference(X, nbr, cnt, F), np.ones(3), fit)
+        print(f"h {h:g} built {built}: {err:.2e}")
+        assert err <= TOL
+        ctx.close()
