@@ -509,9 +509,11 @@ __device__ __forceinline__ void chol9_solve(const T* L, TB* b) {
 // same bits), one call per column (as a loop over the columns the factor is not
 // unrolled and lives in local memory), and 1/sqrt in 5 operations.
 //
-// 1 / sqrt(v) for a positive normal v: the hardware's approximation (about 20
-// bits) and one step of Halley's third-order iteration y (1 + e/2 + 3 e^2/8),
-// e = 1 - v y^2, which leaves the rounding of the step itself (about 1 ulp).
+// 1 / sqrt(v) for a positive normal v (no pivot that is used is subnormal, see
+// fixed_consts): the hardware's approximation and one step of Halley's
+// third-order iteration y (1 + e/2 + 3 e^2/8), e = 1 - v y^2. Off by at most
+// 1.75 x 2^-53 of the result (measured over all exponents 1.25; rsqrt() 1.01,
+// with which LP_FP64 steps of 786,000 particles are 1.3 % slower).
 __device__ __forceinline__ double inv_sqrt(double v) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
