@@ -675,7 +675,7 @@ bool valid_params(const lp_params* q, const lp_eos* e, double dt) {
 // f 2^28, and products are cut to at most 2^28 as well. fx_lim leaves a tenth
 // of the radius for stencils that are held while the particles move.
 // shifted: the rows shift a particle's offsets to its own largest one (up to
-// 2^12), and leave room for offsets beyond r.
+// 2^6), and leave room for offsets beyond r.
 void fixed_consts(StepConsts& K, bool shifted = false) {
   int e;
   const double f = std::frexp(K.radius, &e);  // radius = f 2^e, f in [1/2, 1)
@@ -1069,7 +1069,7 @@ lp_status lp_fit_derivatives(lp_ctx* c, const lp_particles* p, const lp_neighbor
   // FP64: rows in fixed point, the range laid out for the largest radius of the
   // stencils where the context built them, else for four lattice spacings, and
   // shifted to each particle's offsets. Offsets beyond three times that, or
-  // below a thousandth of it, take the plain rows, and so do mirror factors other
+  // below a fiftieth of it, take the plain rows, and so do mirror factors other
   // than -1, 0 and 1.
   StepArgs A{};
   bool unit_signs = true;

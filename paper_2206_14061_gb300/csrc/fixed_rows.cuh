@@ -242,6 +242,12 @@ __device__ __forceinline__ void fx_split_p1_body(const StepArgs& A, int s) {
   A.fs[s] = make_float4(fx_float(g), fx_float(v), 0.f, 0.f);
 }
 
+// A position is rounded to a unit, 2^-58 of the largest radius or less; near the
+// origin that loses bits of the coordinate, which a shift brings up: after 6 bits
+// to 2^-53 of the stencil's largest offset, as much as FP64 loses. (Up to 12 were
+// taken: stencils of a thousandth of the largest radius around the origin erred
+// by 1.3e-14 of the largest coefficient, where FP64 rows give 1.5e-15.)
+constexpr int kFxMostShift = 6;
 // Stencils whose radius is not known (lp_fit_derivatives): the shift that
 // brings a particle's largest offset into (fx_lim / 2, fx_lim], from a walk over
 // the positions; -1 if the offsets are too large, or so small that the shift
@@ -279,7 +285,7 @@ __device__ __forceinline__ int fx_shift(const StepArgs& A, int s, int m) {
   if (big + 1u > lim) return -1;
   int sh = max(__clz((int)(big + 1u)) - __clz((int)lim), 0);
   if (((big + 1u) << sh) > lim) --sh;
-  return sh <= 12 ? sh : -1;
+  return sh <= kFxMostShift ? sh : -1;
 }
 
 // The 31 moments of a stencil (order of ff_moments_add) in units of the

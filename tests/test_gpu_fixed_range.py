@@ -325,3 +325,29 @@ def test_fit_with_h_far_above_the_spacing(capi, h):
         print(f"h {h:g} built {built}: {err:.2e}")
         assert err <= TOL
         ctx.close()
+
+
+@pytest.mark.parametrize("ratio", [1, 20, 60, 500, 1000, 2000, 4000, 10000])
+def test_fit_of_small_stencils_near_the_origin(capi, ratio):
+    """Radii 1 : ratio in one call, the small ones where coordinates have more
+    bits than the layout for the largest keeps: 64 roundings of FP64."""
+    big = 2.2e-3
+    X = _lattice(7, 0.1)
+    d = big / ratio / 1.9
+    P = np.concatenate([X * d, np.full((3, 1), 1.0)], 1)
+    rad = np.append(np.full(X.shape[1], 1.9 * d), big)
+    ctx = capi.Context(P.shape[1], cap=64)
+    nb = capi.lp_build_neighbors(ctx, *[T(c) for c in P], radius=T(rad), mirror_mode=0)
+    nbr, cnt = nb.export()
+    F = np.concatenate([_fields(X), np.zeros((2, 1))], 1)
+    got = capi.lp_fit_derivatives(ctx, *[T(c) for c in P], nb, [T(f) for f in F], [1.0, 1.0],
+                                  d).cpu().numpy()
+    assert ctx.sync()["flags"] == 0
+    ctx.close()
+    fit = cnt >= 26
+    assert fit.sum() >= 100
+    ref = np.zeros_like(got)
+    ref[fit] = _reference(P, nbr, cnt, F, np.nonzero(fit)[0])
+    err = _error(got, ref, np.full(3, d), fit)
+    print(f"ratio {ratio}: {err:.2e}")
+    assert err <= 64 * 2.0 ** -53
