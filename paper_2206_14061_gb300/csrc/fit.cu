@@ -438,11 +438,14 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, co
   double L[kTri];
   int rows = 0;
   const int sh = fx_shift(A, s, m);
-  bool fits = sh >= 0;
+  bool fits = sh >= 0, resolved = false;
   if (fits) {
+    long long H[31];
     double mo[31];
-    fits = fx_moments<false, false, true>(A, s, m, mo, &rows, sh);
-    if (fits) gram_of_moments(mo, L);
+    fits = fx_moment_rows<false, false, true, 1>(A, s, m, 0, H, &rows, sh);
+    resolved = fx_resolved(H);
+    fx_moment_values<true>(A.K, H, sh, mo);
+    gram_of_moments(mo, L);
   }
   bool even = false;  // the columns' lengths
   if (fits) {
@@ -456,15 +459,16 @@ __global__ void __launch_bounds__(kFxBlock, 3) k_fit_gram_fx(const FitArgs F, co
   }
   bool ill = false;
   const bool ok = fits && fx_chol9(L, 1e-9, &ill) && rows >= kNB;
+  ill = ill || !resolved;  // (QR needs no moments: it does for these as well)
   A.kx[s] = ok && !ill ? sh : kFxSlow;
-  if (!fits || (ok && ill && !even) || (!ok && fit_far_in_z(F, A, s, m))) {
-    fx_push(A, s, 0);
-    return;
-  }
-  if (!ok) {
+  if (!ok && fits && (resolved || rows < kNB) && !fit_far_in_z(F, A, s, m)) {
     const int slot = atomicAdd(F.fb_count, 1);
     if (slot < F.fb_cap) F.fb_list[slot] = s;
     else atomicOr(&F.dg->flags, (unsigned)LP_FLAG_OVERFLOW);
+    return;
+  }
+  if (!ok || (ill && !even)) {
+    fx_push(A, s, 0);
     return;
   }
   if (ill) {
