@@ -708,8 +708,10 @@ __global__ void __launch_bounds__(128, 3) k_fit_rhs_ff(const FitArgs F, int f0) 
 // 45 us longer than one without; with a sum at a time 75 to 90.
 // Many: a thread for each, its matrix in local memory (fit_qr_item). Particles
 // with six entries, all refused, LP_FP64, three fields: 8,000 take 147 us
-// (1046 with a warp each, summed one at a time), 1.0 M 5.8 ms (120). The line:
-// a wave of thread fits takes about as long as 4,096 warp fits.
+// (1046 with a warp each, summed one at a time), 1.0 M 5.8 ms (120). The line,
+// two waves of warps: 1,728 fits of six entries take 131 us with a thread each
+// and 166 with a warp (LP_MIXED_FF 119 and 154); with 48 entries a wave of
+// thread fits takes 200 us, one of 608 warp fits 45.
 template <int N>
 __device__ __forceinline__ void warp_sums(double* v, int lane) {
   constexpr int P = N > 8 ? 8 : (N > 4 ? 8 : (N > 2 ? 4 : N));
@@ -924,7 +926,7 @@ __device__ __noinline__ void fit_qr_item(const FitArgs& F, int s) {
     for (int f = 0; f < nf; ++f) write_coeffs(F, s, f0 + f, C + f * kNB);
   }
 }
-constexpr int kQrWarpFits = 4096;
+constexpr int kQrWarpFits = 1216;
 __global__ void __launch_bounds__(64) k_fit_fallback(const FitArgs F) {
   const int cnt = min(*F.fb_count, F.fb_cap);
   const int all = cnt + ill_by_qr(F);

@@ -51,9 +51,9 @@ def test_stencils_with_an_entry_that_is_not_finite(capi, orc, axes, value, prec)
 
 @pytest.mark.parametrize("prec", [0, 2])
 @pytest.mark.parametrize("nf", [1, 4, 6])
-@pytest.mark.parametrize("side,r", [(5, 1.2), (12, 1.2), (16, 1.2), (17, 1.2)])
+@pytest.mark.parametrize("side,r", [(5, 1.2), (10, 1.2), (11, 1.2), (17, 1.2)])
 def test_refused_stencils_few_and_many(capi, orc, side, r, nf, prec):
-    """Six entries at most, so every particle takes the QR fit: up to 4096 of
+    """Six entries at most, so every particle takes the QR fit: up to 1216 of
     them a warp each, above that a thread each."""
     h, X = 1e-3, _lattice(side, 0.05)
     P = X * h
