@@ -53,9 +53,10 @@ typedef int32_t lp_status;
 
 /* arithmetic of the least-squares fits */
 #define LP_FP64 0  /* FP64 results: moments and right-hand sides summed in 64- */
-                   /* bit fixed point (terms err by 2^-54 of the largest; FP64 */
-                   /* rows where the range does not hold), Cholesky, solve and */
-                   /* QR fallback in FP64                                      */
+                   /* bit fixed point where a stencil's terms fit and resolve  */
+                   /* in it (they err by 2^-54 of the largest possible one rms */
+                   /* and 2^-51 at most), in FP64 for all other stencils;      */
+                   /* Cholesky, solve and QR fallback in FP64                  */
 #define LP_MIXED 1 /* FP32 moments and Cholesky + one FP64 refinement step     */
 #define LP_MIXED_FF 2 /* FP32 only on the stencil rows: offsets, moments and   */
                       /* right-hand sides accumulated as float-float (FP32     */
@@ -217,7 +218,9 @@ typedef struct {
   int32_t min_stencil, max_stencil;
   int32_t pad;
   int64_t n_overflow;    /* particle-steps whose stencil exceeded cap            */
-  int64_t n_fallback;    /* fits that used the pivoted-QR path                   */
+  int64_t n_fallback;    /* stencils that the normal equations refused (pivoted  */
+                         /* QR instead; lp_fit_derivatives may also take QR for  */
+                         /* poorly conditioned ones, which do not count)         */
   int64_t n_gas, n_quasistatic, n_over_c; /* particle-steps per regime (phi > phi_c) */
   int64_t n_nonfinite, n_below_floor;
   int64_t n_stencil_rows;  /* sum of stencil sizes over all stencils built     */
@@ -386,8 +389,10 @@ lp_status lp_step(lp_ctx* ctx, lp_particles* p, const lp_mui* mui, const lp_eos*
 
 /* Launch configuration of lp_step (not in the paper). Block sizes are threads
  * per block of the neighbour search and of the two fit passes (64, 128 or
- * 256); launch_mode is the faster of LP_LAUNCH_GRAPH and LP_LAUNCH_PERSISTENT
- * for the tuned workload, for the caller to pass in lp_params. */
+ * 256), upper bounds: runs of few particles take smaller blocks, LP_FP64 fits
+ * at most 128 and, up to 29,184 particles, a shape of their own; launch_mode is
+ * the faster of LP_LAUNCH_GRAPH and LP_LAUNCH_PERSISTENT for the tuned workload,
+ * for the caller to pass in lp_params. */
 typedef struct {
   int32_t block_neighbors, block_pass1, block_pass2;
   int32_t launch_mode;

@@ -10,11 +10,12 @@
 // kernel, the same algorithm the paper names (QR least squares).
 //
 // FP64 mode: the sums over the rows in 64-bit fixed point (fixed_rows.cuh;
-// plain FP64 rows for the particles that do not fit it, and in
-// lp_fit_derivatives), the factor, the solves and the rest in FP64. MIXED mode: moments, right-hand sides and the
-// Cholesky factor in FP32 on the scaled, centred offsets, followed by one FP64
-// refinement sweep (residual r = b - A c and A^T r in FP64, correction solved
-// with the FP32 factor).
+// plain FP64 rows for the particles that do not fit it, for
+// lp_fit_derivatives with mirror factors other than -1, 0 and 1, and for
+// lp_fit_derivatives_noalloc), the factor, the solves and the rest in FP64.
+// MIXED mode: moments, right-hand sides and the Cholesky factor in FP32 on the
+// scaled, centred offsets, followed by one FP64 refinement sweep (residual
+// r = b - A c and A^T r in FP64, correction solved with the FP32 factor).
 //
 // Time levels of one step: pass 1 fits u, v, w at time n and sets
 // V^{n+1} = V^n + dt V^n div u^n; pass 2 fits |gdot|^n and V^{n+1} and forms

@@ -12,28 +12,33 @@
 // units of h, |l| <= 1/2, as a float. A product a b enters its sum as
 //   a.h b.h                       exact, one 32 x 32 + 64-bit multiply-add
 //   round(a.h b.l + a.l b.h)      FP32, to an integer (a.l b.l is below 1/4)
-// so a term errs by about 2^-54 of the largest possible one, less than an FP64
-// sum, which rounds at 2^-53 of the running sum in every row. The sums are
+// so a term errs by 2^-54 of the largest possible one (rms; the FP32 operations,
+// on 28-bit values, put the most at 2^-51), where an FP64 sum rounds at 2^-53 of
+// the running sum in every row. The sums are
 // exact, so their order does not matter, and 64 rows of 2^56 cannot overflow
 // them. (Keeping the second part as a float sum, moved into the integer one
 // every fourth row, is as fast and errs by 2^-50.) About 8 cycles per
 // accumulation and scheduler; an FP64 multiply-add takes about 75.
 //
 // Positions are integers X = x 2^k modulo 2^64, with r 2^k in (2^59, 2^60]
-// for the stencil radius r: the conversion is exact for all but the last bits
+// for the stencil radius r (a quarter of it in lp_fit_derivatives, see
+// kFxMostShift): the conversion is exact for all but the last bits
 // of tiny coordinates, and differences of neighbours are exact whatever the
 // distance from the origin (the modular wrap cancels). As entries of a stencil
 // may be anywhere (held stencils, a caller's own lists), the offsets are also
-// taken in FP32 in units of the wrap, to see one that only looks near. Field values (u, v, w;
-// |gdot|, V) are aligned per stencil to its largest value, and their differences
-// shifted up to fill the range; the scales come from a first walk over FP32
-// copies.
+// taken in FP32 in units of the wrap, to see one that only looks near. Field
+// values (u, v, w; |gdot|, V) are aligned per stencil to its largest value, and
+// their differences shifted up to fill the range; the scales come from a first
+// walk over FP32 copies.
 //
 // What does not fit (offsets beyond about the radius, which only stencils held
-// fixed over several steps or a caller's own can have; stencils thin along an axis or small
-// against the radius, see fx_resolved; fields whose differences are not finite
-// or are below 2^-90; non-finite positions) is queued for a kernel that runs
-// the plain FP64 rows.
+// fixed over several steps or a caller's own can have; stencils thin along an
+// axis or small against the radius, see fx_resolved; fields whose differences
+// are not finite or are below 2^-90; non-finite positions) is queued for a
+// kernel that runs the plain FP64 rows. Where all particles are, a step takes 3
+// to 9 % longer than with those rows alone (640,000 particles in a sheet
+// compressed to 0.1: 6.89 and 6.35 ms; 2.07 in fixed point, wrong in the twelfth
+// digit).
 #pragma once
 
 #include "lp_internal.cuh"
